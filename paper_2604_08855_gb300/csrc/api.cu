@@ -583,7 +583,7 @@ int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   pl->nparts = 2 * c->nsm;
   if (c->precision == CTB_PREC_FP32) {
     // one wave of the FP32 contraction's resident blocks
-    const int cb = contract_fp32_blocks_per_sm(c->nbins, c->lmax, c->lay.row, c->sphere);
+    const int cb = contract_fp32_blocks_per_sm(c->nbins, c->lay.row);
     if (cb < 1) return fail(c, CTB_ERR_CUDA, "the contraction kernel cannot be resident");
     pl->ncon = cb * c->nsm;
   } else {
@@ -880,9 +880,9 @@ int compute_impl(ctb_ctx* c, const uint32_t* dprim, int64_t np, double* zeta_out
   const int evs = 2 + 8;
   CK(c, cudaEventRecord(c->ev[evs], c->st));
   if (tc)
-    CK(c, launch_finalize_tc(P<double>(c->partial_tc), c->lmax, pl.ncon, c->nbins, P<double>(c->zeta), c->st));
+    CK(c, launch_finalize_tc(P<double>(c->partial_tc), c->lmax, pl.ncon, c->nbins, P<double>(c->zeta), 1, c->st));
   else
-    CK(c, launch_finalize(P<double>(c->partial), pl.ncon, c->lmax, c->nbins, P<double>(c->zeta), c->sphere != 0,
+    CK(c, launch_finalize(P<double>(c->partial), pl.ncon, c->lmax, c->nbins, P<double>(c->zeta), c->sphere != 0, 1,
                           c->st));
   CK(c, cudaEventRecord(c->ev[evs + 1], c->st));
   const bool dev_out = is_device_ptr(zeta_out);
@@ -1027,13 +1027,15 @@ int batch_impl(ctb_ctx* c, const double* const* xyz, const double* const* w, con
   c->batch_keys = nullptr;
   if (r) return r;
   CK(c, cudaEventRecord(c->ev[10], c->st));
-  for (int i = 0; i < k; ++i) {
+  // every catalogue in one launch (blockIdx.y, 65535 at most)
+  for (int i = 0; i < k; i += 65535) {
     const double* pi = P<double>(part) + (size_t)i * pl.ncon * zsz;
     double* zi = P<double>(c->zeta) + (size_t)i * zsz;
+    const int kc = std::min(k - i, 65535);
     if (tc)
-      CK(c, launch_finalize_tc(pi, c->lmax, pl.ncon, c->nbins, zi, c->st));
+      CK(c, launch_finalize_tc(pi, c->lmax, pl.ncon, c->nbins, zi, kc, c->st));
     else
-      CK(c, launch_finalize(pi, pl.ncon, c->lmax, c->nbins, zi, c->sphere != 0, c->st));
+      CK(c, launch_finalize(pi, pl.ncon, c->lmax, c->nbins, zi, false, kc, c->st));
   }
   CK(c, cudaEventRecord(c->ev[11], c->st));
   const bool dev_out = is_device_ptr(zeta_out);

@@ -9,408 +9,482 @@
 
 namespace ctb {
 
-// Register-tiled form.  For one l, zeta~_l restricted to bins [4B1, 4B1+4) x
-// [4B2, 4B2+4) is a 4x4 tile: per primary and per m, one 16-byte shared load
-// of each side (four bins contiguous) and eight paired FMAs.  Work split of a
-// block: every (multipole pair (l, L - l), tile B1 <= B2) is a task, and G
-// consecutive threads share a task, splitting its m-steps (m = g, g + G,
-// ...) and adding their partial tiles in thread order at the end.  A pair
-// does 2L + 2 m-steps per primary whatever its l (one l when l = L - l), so
-// the threads of a warp stay in step.  All pairs of a primary fit one block
-// (up to 512 threads), so each row is read from HBM once; larger shapes
-// split the pairs over blockIdx.y.
+// Outer-product form.  A thread owns one coefficient slot c of the rows and a
+// T x T tile of bin pairs (B1 <= B2), and walks the primaries of the block's
+// slice: per primary it reads its slot of the tile's bins (2 T scalar shared
+// loads, T on the diagonal) and adds w x y^T in T^2 / 2 paired FMAs.  A
+// warp's lanes are 32 consecutive slots of one tile, so the loads are
+// conflict-free on the rows as they lie in memory: nothing is transposed, any
+// row length will do, and the staging is one asynchronous copy per element.
+// The sum over m within a multipole is left to the end, where the slots of
+// each l are added in a fixed order.
 //
-// Staging: the block walks its slice of the launch's primaries in stages of
-// Q primaries, double-buffered in shared memory.  While the FMAs run on one
-// buffer, the next stage's rows are in flight in registers: a warp loads 4
-// bins x 8 float4 (one 128-byte line per bin), and each thread scatters its
-// float4 to the staged layout [slot][bin], slot s at row s * nbp + 4 (s / 8):
-// the 4 (s / 8) shift puts the 32 scalar stores of a warp (8 consecutive
-// slots x 4 bins) in 32 distinct banks when nbp = 4 mod 32.  Bins are padded
-// to a multiple of 4 with zeros.  Shapes whose tasks fit 256 threads (short
-// rows: the sphere's, l_max 10) run two such blocks per SM with half-size
-// stages; the stage size of short rows is raised with extra loader warps so
-// that a stage still fits the registers.  When two buffers do not fit (64 bins at
-// l_max 20), one buffer is staged between two barriers, the next stage's
-// loads still in flight during the FMAs.  FP32 over the block's slice, then one FP64
-// add per (l, b1 <= b2) entry, whose owner is a single thread: the partial
-// sums are deterministic.
-constexpr int kConTile = 4;
-constexpr int kConMaxThreads = 512;
-constexpr int kConStageFloats = 20480;  // one staged buffer at most (80 KB; two are used)
-constexpr int kConPF = 8;              // float4 loads a thread keeps in flight per stage
-constexpr size_t kConSmemCap = 220 * 1024;
+// What bounds it: the paired FMAs (2.65 issue cycles each, measured) at 20 to
+// 64 bins, HBM for fewer.  A 10 x 10 tile does 50 of them on 20 loads; tiles
+// of 4 x 4 with 16-byte loads of transposed rows, the form before this one,
+// spent most of their time on shared-memory loads and on the transposition.
+//
+// Block: CH slots x tiles x PG primary groups (group g takes the stage's
+// primaries q = g mod PG).  Rows of more than CH slots are taken in chunks of
+// CH, the block walking its slice once per chunk: each element is still read
+// from HBM once.  Where the tiles do not fit a block they are split over
+// blockIdx.y.  FP32 over at most kConFlush primaries of a group, then one
+// FP64 add per (l, b1 <= b2) entry by one owner thread: the partial sums are
+// deterministic.
+//
+// Copies (16 bytes each where the rows allow it): rows that fit one chunk are
+// copied as they lie, one contiguous run per stage, and read at the row's own
+// stride (kConLinear: 121-float rows then cost no more than padded ones);
+// chunks of longer rows are copied row by row (kConRows16, kConRows4).
+constexpr int kConFlush = 1024;         // primaries of a group between two flushes
 constexpr int kConMaxQ = 64;            // primaries per stage at most
-// shapes whose tasks fit this many threads run two blocks per SM (half the
-// threads, half the staged rows each: 2 x 256 threads x 128 registers)
-constexpr int kConSmallThreads = 256;
+constexpr int kConStageFloats = 11264;  // one staged buffer at most, when more than PG primaries fit it
+constexpr int kConStages = 3;
+constexpr int kConMaxTiles = 24;        // tiles per block at most (768 threads / 32)
+enum { kConRows4 = 0, kConRows16 = 1, kConLinear = 2 };
+constexpr size_t kConSmemCap = 220 * 1024;
 
 struct ConShape {
-  int nbb;           // bin quads
-  int nbp;           // floats per staged slot row
-  int tiles;         // 4x4 tiles B1 <= B2
-  int pairs;         // multipole pairs (l, L - l)
-  int G;             // threads per task
-  int ppb, ny;       // pairs per block, blocks in y
+  int T;        // tile side
+  int nbt;      // tiles across the bins
+  int tiles;    // tiles B1 <= B2 per block
+  int ntiles;   // all of them (split over blockIdx.y)
+  int ch;       // slots per chunk
+  int nchunk;
+  int pg;       // primary groups
   int threads;
-  int nch;           // load chunks of 8 float4 along a row
-  int srow;          // floats per staged primary
-  int Q;             // primaries per stage
-  int nbuf;          // staged buffers: 2, or 1 when two do not fit
-  int tab_ints;      // coefficient -> slot table
-  int stage_floats;  // all buffers
-  int red_floats;    // the end-of-kernel combine buffer (aliases the stages)
-  int smem_floats;
+  int stride;   // staged floats between bins: the row, or CH when the row is chunked
+  int Q;        // primaries per stage
+  int stages;
+  int stage_floats;  // one staged buffer
+  int smem_bytes;
 };
 
-__host__ __device__ inline ConShape con_shape(int nbins, int lmax, int row, int sphere) {
+// threads of a block by tile side: T^2 accumulators and 2 T operands a thread
+// (T 6: 80 registers, T 8: 128, T 10: 168)
+__host__ __device__ constexpr int con_max_threads(int T) { return T == 6 ? 768 : (T == 8 ? 512 : 384); }
+
+// Work of one slot and primary in issue cycles of an SM sub-partition: paired
+// FMAs at 2.65, or four shared loads' time per load where that is more (an SM
+// serves one load of a warp per cycle, for four sub-partitions).
+static double con_cost(int T, int nb) {
+  const int nbt = (nb + T - 1) / T, off = nbt * (nbt - 1) / 2;
+  const double fma = 2.65 * (nbt * (T / 2) * (T / 2 + 1) + off * T * T / 2);
+  const double lds = 4.0 * (nbt * T + off * 2 * T);
+  return fma > lds ? fma + 0.3 * lds : lds + 0.3 * fma;
+}
+
+static ConShape con_shape(int nbins, int row) {
   ConShape c{};
-  c.nbb = (nbins + kConTile - 1) / kConTile;
-  c.nbp = kConTile * c.nbb;
-  if (c.nbp % 32 == 0) c.nbp += 4;
-  c.tiles = c.nbb * (c.nbb + 1) / 2;
-  c.pairs = lmax / 2 + 1;
-  const int nc = sphere ? 2 * lmax + 1 : (lmax + 1) * (lmax + 1);
-  const int msteps = sphere ? 4 : 2 * lmax + 2;  // m-steps of the longest pair
-  const bool small = c.pairs * c.tiles <= kConSmallThreads;
-  const int tmax = small ? kConSmallThreads : kConMaxThreads;
-  if (c.pairs * c.tiles <= kConMaxThreads) {
-    c.ppb = c.pairs;
-    c.G = tmax / (c.pairs * c.tiles);
-    if (c.G > msteps) c.G = msteps;
-    if (c.G > 32) c.G = 32;
-  } else {
-    c.G = 1;
-    c.ppb = kConMaxThreads / c.tiles;
-  }
-  c.ny = (c.pairs + c.ppb - 1) / c.ppb;
-  c.threads = (c.ppb * c.tiles * c.G + 31) / 32 * 32;
-  c.nch = ((row + 3) / 4 + 7) / 8;
-  {
-    // enough warps that one primary's rows are in flight in registers
-    const int wl = (c.nbb * c.nch + kConPF - 1) / kConPF;
-    if (c.threads < 32 * wl) c.threads = 32 * wl < tmax ? 32 * wl : tmax;
-  }
-  c.srow = (row * c.nbp + 4 * ((row + 7) / 8) + 3) & ~3;
-  const int units1 = c.nbb * c.nch;  // load units of one primary
-  int q = (small ? kConStageFloats / 2 : kConStageFloats) / c.srow;
-  if (q > kConMaxQ) q = kConMaxQ;
-  if (q < 1) q = 1;
-  {
-    // short rows: more warps (idle in the FMAs) so that a stage of q
-    // primaries is still loaded from registers
-    const int wq = (q * units1 + kConPF - 1) / kConPF;
-    if (c.threads < 32 * wq) c.threads = 32 * wq < tmax ? 32 * wq : tmax;
-  }
-  const int warps = c.threads / 32;
+  // the tile side with the least work: 10 for 10 and 20 bins, 8 for 16 and
+  // 32, 6 for 36 (the side that pads the bins least wins over a larger one)
+  c.T = 6;
+  for (int T = 8; T <= 10; T += 2)
+    if (con_cost(T, nbins) < con_cost(c.T, nbins)) c.T = T;
+  const int cap = con_max_threads(c.T);
+  c.nbt = (nbins + c.T - 1) / c.T;
+  c.ntiles = c.nbt * (c.nbt + 1) / 2;
+  c.tiles = c.ntiles * 32 <= cap ? c.ntiles : cap / 32;
+  const int rows32 = (row + 31) / 32 * 32;
+  c.ch = 32;
+  while (c.ch < 128 && 2 * c.ch * c.tiles <= cap && c.ch < rows32) c.ch *= 2;
+  c.nchunk = (row + c.ch - 1) / c.ch;
+  c.pg = cap / (c.ch * c.tiles);
+  if (c.pg > 8) c.pg = 8;
+  c.threads = c.ch * c.tiles * c.pg;
+  c.stride = c.nchunk == 1 ? row : c.ch;
+  // primaries per stage: a multiple of the groups, and of four so that every
+  // contiguous run starts on 16 bytes when the base does
+  const int unit = c.pg % 4 == 0 ? c.pg : (c.pg % 2 == 0 ? 2 * c.pg : 4 * c.pg);
+  int q = kConStageFloats / (nbins * c.stride) / unit * unit;
+  if (q > kConMaxQ) q = kConMaxQ / unit * unit;
+  if (q < unit) q = unit;
   c.Q = q;
-  if (c.Q * units1 > kConPF * warps) c.Q = kConPF * warps / units1;  // keep a stage's loads in registers
-  if (c.Q < 1) c.Q = 1;
-  // coefficient -> staged row offset, then the staged primaries' weights
-  c.tab_ints = ((nc + 3) & ~3) + 2 * kConMaxQ;
-  c.nbuf = (size_t)(c.tab_ints + 2 * c.Q * c.srow) * 4 <= kConSmemCap ? 2 : 1;
-  c.stage_floats = c.nbuf * c.Q * c.srow;
-  c.red_floats = c.threads * 17;
-  c.smem_floats = c.tab_ints + (c.stage_floats > c.red_floats ? c.stage_floats : c.red_floats);
-  (void)nc;
+  // a tile wider than the bins and a chunk wider than the row read on past
+  // their end: slots and bins that nothing owns
+  c.stage_floats = c.Q * nbins * c.stride + (nbins < c.T ? (c.T - nbins) * c.stride : 0) + c.ch;
+  c.stage_floats = (c.stage_floats + 3) & ~3;
+  const int red = c.threads * c.T;  // the flush buffer aliases the stages
+  c.stages = kConStages;
+  while (c.stages > 1 && (size_t)(c.stages * (c.stage_floats + kConMaxQ)) * 4 + 4096 > kConSmemCap) --c.stages;
+  const int body = c.stages * c.stage_floats > red ? c.stages * c.stage_floats : red;
+  c.smem_bytes = (body + c.stages * kConMaxQ + kConMaxTiles) * 4;
   return c;
 }
 
-__device__ __forceinline__ int group_start(int l, int sphere) { return sphere ? (l == 0 ? 0 : 2 * l - 1) : l * l; }
-__device__ __forceinline__ int group_size(int l, int sphere) { return sphere ? (l == 0 ? 1 : 2) : 2 * l + 1; }
-
-// offset of slot s of staged primary q
-__device__ __forceinline__ int con_off(const ConShape& sh, int q, int s) { return q * sh.srow + s * sh.nbp + 4 * (s >> 3); }
-
-// 4x4 tile of one group (a multipole l: components l^2 .. l^2 + 2l; on the
-// sphere, m: component 0, or 2m-1 and 2m): acc += w x y^T summed over the
-// group's components, the task's threads taking every G-th component.
-// acc[2 i + j] holds entries (i, 2j) and (i, 2j + 1).
-__device__ __forceinline__ void con_tile(const float* __restrict__ S, int G, const int* s_offc, int c0, int nc, int g,
-                                         int B1, int B2, float w, float2 (&acc)[8]) {
-  const float* Sx = S + 4 * B1;
-  const float* Sy = S + 4 * B2;
-#pragma unroll 2
-  for (int m = g; m < nc; m += G) {
-    const int off = s_offc[c0 + m];
-    const float4 x = *reinterpret_cast<const float4*>(Sx + off);
-    const float4 y = *reinterpret_cast<const float4*>(Sy + off);
-    const float2 y01 = make_float2(y.x, y.y), y23 = make_float2(y.z, y.w);
-    const float2 x01 = __fmul2_rn(make_float2(w, w), make_float2(x.x, x.y));
-    const float2 x23 = __fmul2_rn(make_float2(w, w), make_float2(x.z, x.w));
-    acc[0] = __ffma2_rn(make_float2(x01.x, x01.x), y01, acc[0]);
-    acc[1] = __ffma2_rn(make_float2(x01.x, x01.x), y23, acc[1]);
-    acc[2] = __ffma2_rn(make_float2(x01.y, x01.y), y01, acc[2]);
-    acc[3] = __ffma2_rn(make_float2(x01.y, x01.y), y23, acc[3]);
-    acc[4] = __ffma2_rn(make_float2(x23.x, x23.x), y01, acc[4]);
-    acc[5] = __ffma2_rn(make_float2(x23.x, x23.x), y23, acc[5]);
-    acc[6] = __ffma2_rn(make_float2(x23.y, x23.y), y01, acc[6]);
-    acc[7] = __ffma2_rn(make_float2(x23.y, x23.y), y23, acc[7]);
-  }
+__device__ __forceinline__ void con_cp4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void con_cp16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
 
-// The G threads of a task add their tiles in thread order (through shared
-// memory), and the first adds the result to the block's FP64 partial.
-__device__ __forceinline__ void con_flush(const ConShape& sh, const float2 (&acc)[8], bool own, int l, int g,
-                                          int B1, int B2, int nb, double* __restrict__ out, float* s_red) {
-  float* mine = s_red + threadIdx.x * 17;
+// one primary: S1, S2 the first bin of the tile's sides, st floats between bins
+template <int T, bool DIAG>
+__device__ __forceinline__ void con_step(float2 (&acc)[T][T / 2], const float* S1, const float* S2, int st, float w) {
+  float x[T], y[T];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    mine[2 * k] = acc[k].x;
-    mine[2 * k + 1] = acc[k].y;
-  }
-  __syncthreads();
-  if (own && g == 0) {
+  for (int i = 0; i < T; ++i) x[i] = S1[i * st];
+  if constexpr (!DIAG) {
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      float v = mine[k];
-      for (int h = 1; h < sh.G; ++h) v += s_red[(threadIdx.x + h) * 17 + k];
-      // k = 2 (2 i + j') + e: entry (i, 2 j' + e)
-      const int i = k >> 2, j = k & 3;
-      const int b1 = 4 * B1 + i, b2 = 4 * B2 + j;
-      if (b1 < nb && b2 < nb && b1 <= b2) out[((size_t)l * nb + b1) * nb + b2] += (double)v;
-    }
+    for (int i = 0; i < T; ++i) y[i] = S2[i * st];
   }
-  __syncthreads();
-}
-
-// Load units: 4 bins x 8 float4 of a row (lane l: bin 4 bq + l / 8, float4
-// 8 ch + l % 8) of staged primary q, u = (q nbb + bq) nch + ch.  Warp w owns
-// units [w upw, (w + 1) upw) of a stage, walked by incrementing (q, bq, ch).
-struct ConUnit {
-  int q, bq, ch;
-};
-__device__ __forceinline__ void con_next(const ConShape& sh, ConUnit& t) {
-  if (++t.ch == sh.nch) {
-    t.ch = 0;
-    if (++t.bq == sh.nbb) {
-      t.bq = 0;
-      ++t.q;
+#pragma unroll
+  for (int i = 0; i < T; ++i) {
+    const float xi = w * x[i];
+#pragma unroll
+    for (int j = DIAG ? i / 2 : 0; j < T / 2; ++j) {
+      const float2 v = DIAG ? make_float2(x[2 * j], x[2 * j + 1]) : make_float2(y[2 * j], y[2 * j + 1]);
+      acc[i][j] = __ffma2_rn(make_float2(xi, xi), v, acc[i][j]);
     }
   }
 }
 
-__device__ __forceinline__ void con_store4(float* buf, const ConShape& sh, int q, int b, int c4, float4 v) {
-  const int s = 4 * c4;
-  float* d = buf + con_off(sh, q, s) + b;
-  // slots s .. s + 3 share s / 8
-  d[0] = v.x;
-  d[sh.nbp] = v.y;
-  d[2 * sh.nbp] = v.z;
-  d[3 * sh.nbp] = v.w;
-}
-
-__global__ void __launch_bounds__(kConMaxThreads, 1) k_contract_fp32(ContractArgs a) {
+template <int T, int CH, int MODE>
+__global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(ContractArgs a, ConShape sh) {
   extern __shared__ __align__(16) float s_dyn[];
+  __shared__ int s_slotl[CH];  // multipole of each slot of the chunk (-1: none)
+  __shared__ int s_ord[CH];    // the chunk's slots by multipole
+  __shared__ int s_l[kLmaxCap + 1], s_l0[kLmaxCap + 2], s_nl;  // its multipoles and where their slots start
   const int nb = a.nbins, L = a.lmax;
   const int nc = a.sphere ? 2 * L + 1 : (L + 1) * (L + 1);  // coefficients per (primary, bin)
-  const ConShape sh = con_shape(nb, L, a.row, a.sphere);
-  // [coefficient -> staged row offset | weights of the staged primaries, per
-  //  buffer | staged buffers (the combine buffer at the end)]
-  int* s_offc = reinterpret_cast<int*>(s_dyn);
-  float* s_w = s_dyn + (sh.tab_ints - 2 * kConMaxQ);
-  float* s_stage = s_dyn + sh.tab_ints;
-  for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-    const int sl = a.slot[c];
-    s_offc[c] = sl * sh.nbp + 4 * (sl >> 3);
-  }
-  for (int k = threadIdx.x; k < sh.stage_floats; k += blockDim.x) s_stage[k] = 0.f;  // bin padding stays zero
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  const int task = tid / sh.G, g = tid - task * sh.G;
-  const int pair = blockIdx.y * sh.ppb + task / sh.tiles;
-  const int tile = task % sh.tiles;
-  const bool active = task < sh.ppb * sh.tiles && pair < sh.pairs;
-  int B1 = 0, B2 = 0;
-  {
-    int r = active ? tile : 0;
-    while (r >= sh.nbb - B1) {
-      r -= sh.nbb - B1;
-      ++B1;
-    }
-    B2 = B1 + r;
-  }
-  const int la = pair, lb = L - pair;
-  float2 acc_a[8], acc_b[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) acc_a[k] = acc_b[k] = make_float2(0.f, 0.f);
-  const int64_t slice = (a.np + gridDim.x - 1) / gridDim.x;
+  int* s_tile = reinterpret_cast<int*>(s_dyn);              // [kConMaxTiles] B1 | B2 << 8 (-1: none)
+  float* s_w = s_dyn + kConMaxTiles;                        // [stages][kConMaxQ]
+  float* s_stage = s_w + sh.stages * kConMaxQ;              // [stages][Q][nb][stride]
+  const int tid = threadIdx.x;
+  const int c = tid % CH;
+  const int tl = (tid / CH) % sh.tiles, pg = tid / (CH * sh.tiles);
+  const int64_t slice = ((a.np + gridDim.x - 1) / gridDim.x + 3) & ~(int64_t)3;
   const int64_t p0 = (int64_t)blockIdx.x * slice;
   const int64_t p1 = min(a.np, p0 + slice);
-  const int64_t rowsz = (int64_t)nb * a.row;
-  const bool vec4 = (a.row & 3) == 0 && (reinterpret_cast<uintptr_t>(a.M) & 15) == 0;
-  const int row4 = a.row >> 2;
-  const int units = sh.Q * sh.nbb * sh.nch;  // load units of a full stage
-  const int upw = (units + nwarps - 1) / nwarps;   // units per warp
-  ConUnit t0;  // this warp's first unit
-  {
-    const int u0 = warp * upw, per = sh.nbb * sh.nch;
-    t0.q = u0 / per;
-    t0.bq = (u0 - t0.q * per) / sh.nch;
-    t0.ch = u0 - t0.q * per - t0.bq * sh.nch;
-  }
-  const int lb8 = lane >> 3, lc8 = lane & 7;
-  __syncthreads();
-
-  // rows of the stage at pb (cnt primaries) into buffer buf: the warp's
-  // first kConPF units from registers (loaded by issue), the rest here
-  float4 pf[kConPF];
-  float wpf = 0.f;  // thread q < Q: the weight of staged primary q
-  auto issue = [&](int64_t pb, int cnt) {
-    if (tid < cnt) wpf = __ldg(a.wprim + pb + tid);
-    const float4* src = reinterpret_cast<const float4*>(a.M + pb * rowsz);
-    ConUnit t = t0;
-#pragma unroll
-    for (int i = 0; i < kConPF; ++i) {
-      const int b = 4 * t.bq + lb8, c4 = 8 * t.ch + lc8;
-      if (i < upw && t.q < cnt && b < nb && c4 < row4) pf[i] = __ldcs(src + ((int64_t)t.q * nb + b) * row4 + c4);
-      con_next(sh, t);
+  if (p0 >= p1) return;  // uniform for the block
+  // tile -> (B1 <= B2); the last tile of a side is moved back so that it ends
+  // at the last bin (its bins before B T are computed twice, written once)
+  for (int t = tid; t < sh.tiles; t += blockDim.x) {
+    int r = blockIdx.y * sh.tiles + t, v = -1;
+    if (r < sh.ntiles) {
+      int B = 0;
+      while (r >= sh.nbt - B) {
+        r -= sh.nbt - B;
+        ++B;
+      }
+      v = B | (B + r) << 8;
     }
-  };
-  auto land = [&](float* buf, int64_t pb, int cnt) {
-    if (tid < cnt) s_w[(buf == s_stage ? 0 : kConMaxQ) + tid] = wpf;
-    ConUnit t = t0;
-#pragma unroll
-    for (int i = 0; i < kConPF; ++i) {
-      const int b = 4 * t.bq + lb8, c4 = 8 * t.ch + lc8;
-      if (i < upw && t.q < cnt && b < nb && c4 < row4) con_store4(buf, sh, t.q, b, c4, pf[i]);
-      con_next(sh, t);
-    }
-    const float4* src = reinterpret_cast<const float4*>(a.M + pb * rowsz);
-    for (int i = kConPF; i < upw; ++i) {
-      const int b = 4 * t.bq + lb8, c4 = 8 * t.ch + lc8;
-      if (t.q < cnt && b < nb && c4 < row4)
-        con_store4(buf, sh, t.q, b, c4, __ldcs(src + ((int64_t)t.q * nb + b) * row4 + c4));
-      con_next(sh, t);
-    }
-  };
-  // scalar rows (a row length that is not a multiple of 4, or an unaligned base)
-  auto land1 = [&](float* buf, int64_t pb, int cnt) {
-    if (tid < cnt) s_w[(buf == s_stage ? 0 : kConMaxQ) + tid] = __ldg(a.wprim + pb + tid);
-    const float* src = a.M + pb * rowsz;
-    for (int64_t k = tid; k < (int64_t)cnt * rowsz; k += blockDim.x) {
-      const int64_t pr = k / a.row;
-      const int s = (int)(k - pr * a.row);
-      const int q = (int)(pr / nb), b = (int)(pr - (int64_t)q * nb);
-      buf[con_off(sh, q, s) + b] = __ldcs(src + k);
-    }
-  };
-
-  int cur = 0;
-  if (p0 < p1) {
-    const int cnt = (int)min((int64_t)sh.Q, p1 - p0);
-    if (vec4) {
-      issue(p0, cnt);
-      land(s_stage, p0, cnt);
-    } else {
-      land1(s_stage, p0, cnt);
-    }
+    s_tile[t] = v;
   }
   __syncthreads();
-  for (int64_t pb = p0; pb < p1; pb += sh.Q) {
-    const int cnt = (int)min((int64_t)sh.Q, p1 - pb);
-    const int64_t pn = pb + sh.Q;
-    const int cntn = pn < p1 ? (int)min((int64_t)sh.Q, p1 - pn) : 0;
-    float* bufc = s_stage + cur * sh.Q * sh.srow;
-    float* bufn = s_stage + (sh.nbuf == 2 ? cur ^ 1 : 0) * sh.Q * sh.srow;
-    if (vec4 && cntn > 0) issue(pn, cntn);  // in flight during the FMAs
-    if (active) {
-      const float* wq = s_w + (bufc == s_stage ? 0 : kConMaxQ);
-      for (int q = 0; q < cnt; ++q) {
-        const float w = wq[q];
-        const float* S = bufc + q * sh.srow;
-        con_tile(S, sh.G, s_offc, group_start(la, a.sphere), group_size(la, a.sphere), g, B1, B2, w, acc_a);
-        if (lb != la) con_tile(S, sh.G, s_offc, group_start(lb, a.sphere), group_size(lb, a.sphere), g, B1, B2, w, acc_b);
+  const int tv = s_tile[tl];
+  const bool active = tv >= 0;
+  const int B1 = active ? tv & 255 : 0, B2 = active ? tv >> 8 : 0;
+  auto start = [&](int B) { return max(min(B * T, nb - T), 0); };
+  const int stride = MODE == kConLinear ? sh.stride : CH;
+  const int off1 = start(B1) * stride + c, off2 = start(B2) * stride + c;
+  const int qstride = nb * stride;
+  double* out = a.partial + (size_t)(a.part0 + blockIdx.x) * (L + 1) * nb * nb;
+  float2 acc[T][T / 2];
+#pragma unroll
+  for (int i = 0; i < T; ++i)
+#pragma unroll
+    for (int j = 0; j < T / 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
+
+  for (int ck = 0; ck < sh.nchunk; ++ck) {
+    const int c0 = ck * CH;
+    // the multipole of each slot of the chunk, its slots sorted by multipole,
+    // and the multipoles that have any
+    __syncthreads();
+    if (tid < CH) s_slotl[tid] = -1;
+    __syncthreads();
+    for (int k = tid; k < nc; k += blockDim.x) {
+      const int s = __ldg(a.slot + k) - c0;
+      if (s >= 0 && s < CH) {
+        int l = a.sphere ? (k + 1) / 2 : (int)sqrtf((float)k);
+        if (!a.sphere) {
+          while ((l + 1) * (l + 1) <= k) ++l;
+          while (l * l > k) --l;
+        }
+        s_slotl[s] = l;
       }
     }
-    if (cntn > 0) {
-      if (sh.nbuf == 1) __syncthreads();  // one buffer: every thread is done reading it
-      if (vec4) land(bufn, pn, cntn);
-      else land1(bufn, pn, cntn);
+    __syncthreads();
+    if (tid < CH) {
+      const int l = s_slotl[tid];
+      int below = 0, distinct = 0, prev = 0;  // prev: an earlier slot has this l
+      unsigned seen = 0;                      // multipoles below l
+      for (int k = 0; k < CH; ++k) {
+        const int lk = s_slotl[k];
+        if (lk < 0) continue;
+        below += lk < l || (lk == l && k < tid);
+        prev |= lk == l && k < tid;
+        if (lk < l) seen |= 1u << lk;
+      }
+      distinct = __popc(seen);
+      if (l >= 0) {
+        s_ord[below] = tid;
+        if (!prev) {
+          s_l[distinct] = l;
+          s_l0[distinct] = below;
+        }
+      }
     }
-    __syncthreads();  // bufc is read no more; bufn is staged
-    if (sh.nbuf == 2) cur ^= 1;
+    if (tid == 0) {
+      unsigned all = 0;
+      int n = 0;
+      for (int k = 0; k < CH; ++k) {
+        const int lk = s_slotl[k];
+        if (lk >= 0) {
+          all |= 1u << lk;
+          ++n;
+        }
+      }
+      s_nl = __popc(all);
+      s_l0[__popc(all)] = n;
+    }
+    __syncthreads();
+
+    // copy of the stage of primaries [pb, pb + cnt)
+    auto issue = [&](int64_t pb, int cnt, int st) {
+      float* buf = s_stage + st * sh.stage_floats;
+      if (tid < cnt) con_cp4(s_w + st * kConMaxQ + tid, a.wprim + pb + tid);
+      const float* src = a.M + pb * nb * (int64_t)a.row;
+      if constexpr (MODE == kConLinear) {
+        const int total = cnt * nb * a.row;
+        int k = tid * 4;
+        if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+#pragma unroll 4
+          for (; k + 4 <= total; k += blockDim.x * 4) con_cp16(buf + k, src + k);
+          for (k = (total & ~3) + tid; k < total; k += blockDim.x) con_cp4(buf + k, src + k);
+        } else {
+#pragma unroll 4
+          for (k = tid; k < total; k += blockDim.x) con_cp4(buf + k, src + k);
+        }
+      } else {
+        // thread tid takes one column (four with 16-byte copies) of every
+        // (threads / columns)-th row
+        constexpr int E = MODE == kConRows16 ? 4 : 1, COLS = CH / E;
+        const int col = (tid % COLS) * E, rs = blockDim.x / COLS, r0 = tid / COLS;
+        if (c0 + col < a.row) {
+          const float* sp = src + c0 + col + (int64_t)r0 * a.row;
+          float* dp = buf + r0 * CH + col;
+          const int64_t sstep = (int64_t)rs * a.row;
+          const int dstep = rs * CH, rows = cnt * nb;
+#pragma unroll 4
+          for (int r = r0; r < rows; r += rs) {
+            if constexpr (E == 4) con_cp16(dp, sp);
+            else con_cp4(dp, sp);
+            sp += sstep;
+            dp += dstep;
+          }
+        }
+      }
+    };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    // the sums over each multipole's slots, row i of every tile at a time
+    auto flush = [&] {
+      float* red = s_stage;  // [pg][tile][T][CH]
+      const int nl = s_nl, total = sh.tiles * T * nl;
+#pragma unroll
+      for (int i = 0; i < T; ++i) {
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < T / 2; ++j) {
+          red[((pg * sh.tiles + tl) * T + 2 * j) * CH + c] = acc[i][j].x;
+          red[((pg * sh.tiles + tl) * T + 2 * j + 1) * CH + c] = acc[i][j].y;
+          acc[i][j] = make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+        for (int o = tid; o < total; o += blockDim.x) {
+          const int tj = o / nl, k = o - tj * nl;
+          const int t = tj / T, j = tj % T;
+          const int v2 = s_tile[t];
+          if (v2 < 0) continue;
+          const int C1 = v2 & 255, C2 = v2 >> 8;
+          const int b1 = start(C1) + i, b2 = start(C2) + j;
+          if (b1 >= nb || b2 >= nb || b1 > b2 || b1 < C1 * T || b2 < C2 * T) continue;
+          const int q0 = s_l0[k], q1 = s_l0[k + 1];
+          float v = 0.f;
+          for (int g = 0; g < sh.pg; ++g) {
+            const float* rg = red + ((g * sh.tiles + t) * T + j) * CH;
+            for (int q = q0; q < q1; ++q) v += rg[s_ord[q]];
+          }
+          out[((size_t)s_l[k] * nb + b1) * nb + b2] += (double)v;
+        }
+      }
+      __syncthreads();
+    };
+
+    for (int64_t f0 = p0; f0 < p1; f0 += (int64_t)kConFlush * sh.pg) {
+      const int64_t f1 = min(p1, f0 + (int64_t)kConFlush * sh.pg);
+      const int nst = (int)((f1 - f0 + sh.Q - 1) / sh.Q);
+      auto count = [&](int k) { return (int)min((int64_t)sh.Q, f1 - f0 - (int64_t)k * sh.Q); };
+      for (int k = 0; k < sh.stages - 1; ++k) {
+        if (k < nst) issue(f0 + (int64_t)k * sh.Q, count(k), k);
+        commit();
+      }
+      int st = 0, nx = sh.stages - 1;
+      for (int k = 0; k < nst; ++k) {
+        if (sh.stages == 1) {  // one buffer: copy, wait, use
+          __syncthreads();
+          issue(f0 + (int64_t)k * sh.Q, count(k), 0);
+          commit();
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          __syncthreads();
+        } else {
+          if (sh.stages == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
+          else asm volatile("cp.async.wait_group 1;" ::: "memory");
+          __syncthreads();  // stage k is in, and every thread is done with stage k - 1
+          if (k + sh.stages - 1 < nst) issue(f0 + (int64_t)(k + sh.stages - 1) * sh.Q, count(k + sh.stages - 1), nx);
+          commit();
+        }
+        const int cnt = count(k);
+        const float* buf = s_stage + st * sh.stage_floats + pg * qstride;
+        const float* wq = s_w + st * kConMaxQ;
+        if (active) {
+          if (B1 == B2) {
+            for (int q = pg; q < cnt; q += sh.pg, buf += sh.pg * qstride)
+              con_step<T, true>(acc, buf + off1, nullptr, stride, wq[q]);
+          } else {
+            for (int q = pg; q < cnt; q += sh.pg, buf += sh.pg * qstride)
+              con_step<T, false>(acc, buf + off1, buf + off2, stride, wq[q]);
+          }
+        }
+        if (sh.stages > 1) {
+          st = st + 1 == sh.stages ? 0 : st + 1;
+          nx = nx + 1 == sh.stages ? 0 : nx + 1;
+        }
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      flush();
+    }
   }
-  if (blockIdx.y * sh.ppb >= sh.pairs) return;  // the whole block has no pair (uniform)
-  double* out = a.partial + (size_t)(a.part0 + blockIdx.x) * (L + 1) * nb * nb;
-  float* s_red = s_stage;  // the stages are done
-  con_flush(sh, acc_a, active && la <= L, la, g, B1, B2, nb, out, s_red);
-  con_flush(sh, acc_b, active && lb != la && lb >= 0, lb, g, B1, B2, nb, out, s_red);
+}
+
+template <int T, int CH>
+static const void* con_fn(int mode) {
+  return mode == kConLinear   ? (const void*)k_contract_fp32<T, CH, kConLinear>
+         : mode == kConRows16 ? (const void*)k_contract_fp32<T, CH, kConRows16>
+                              : (const void*)k_contract_fp32<T, CH, kConRows4>;
+}
+
+static const void* con_kernel(const ConShape& sh, int row, bool aligned) {
+  const int mode = sh.nchunk == 1 ? kConLinear : ((row & 3) == 0 && aligned ? kConRows16 : kConRows4);
+  switch (sh.T * 1000 + sh.ch) {
+    case 6032: return con_fn<6, 32>(mode);
+    case 6064: return con_fn<6, 64>(mode);
+    case 6128: return con_fn<6, 128>(mode);
+    case 8032: return con_fn<8, 32>(mode);
+    case 8064: return con_fn<8, 64>(mode);
+    case 8128: return con_fn<8, 128>(mode);
+    case 10032: return con_fn<10, 32>(mode);
+    case 10064: return con_fn<10, 64>(mode);
+    default: return con_fn<10, 128>(mode);
+  }
 }
 
 // Resident blocks per SM of the contraction for this shape (0 if it cannot run).
-int contract_fp32_blocks_per_sm(int nbins, int lmax, int row, int sphere) {
-  const ConShape sh = con_shape(nbins, lmax, row, sphere);
-  const size_t smem = (size_t)sh.smem_floats * sizeof(float);
-  if (smem > kConSmemCap) return 0;
-  if (cudaFuncSetAttribute(k_contract_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_contract_fp32, sh.threads, smem) != cudaSuccess) return 0;
-  return nb;
+int contract_fp32_blocks_per_sm(int nbins, int row) {
+  const ConShape sh = con_shape(nbins, row);
+  if ((size_t)sh.smem_bytes > kConSmemCap) return 0;
+  int least = 1 << 30;
+  for (int al = 0; al < 2; ++al) {
+    const void* fn = con_kernel(sh, row, al != 0);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem_bytes) != cudaSuccess) return 0;
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, sh.threads, sh.smem_bytes) != cudaSuccess) return 0;
+    if (nb < least) least = nb;
+  }
+  return least;
 }
 
 cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t st) {
   if (a.np == 0) return cudaSuccess;
-  const ConShape sh = con_shape(a.nbins, a.lmax, a.row, a.sphere);
-  const size_t smem = (size_t)sh.smem_floats * sizeof(float);
-  if (smem > kConSmemCap) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_contract_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const ConShape sh = con_shape(a.nbins, a.row);
+  if ((size_t)sh.smem_bytes > kConSmemCap) return cudaErrorInvalidValue;
+  const void* fn = con_kernel(sh, a.row, (reinterpret_cast<uintptr_t>(a.M) & 15) == 0);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem_bytes);
   if (e != cudaSuccess) return e;
-  k_contract_fp32<<<dim3(nparts, sh.ny), sh.threads, smem, st>>>(a);
+  ContractArgs ca = a;
+  ConShape cs = sh;
+  void* args[] = {&ca, &cs};
+  e = cudaLaunchKernel(fn, dim3(nparts, (sh.ntiles + sh.tiles - 1) / sh.tiles), dim3(sh.threads), args,
+                       (size_t)sh.smem_bytes, st);
+  if (e != cudaSuccess) return e;
   ++g_launches;
   return cudaGetLastError();
 }
 
-// zeta_l(b1,b2) = f_l * sum_parts partial[part][l][min b][max b], in part
-// order; f_l = 4 pi/(2l+1) for the 3-D multipoles, 1 on the sphere.
-__global__ void k_finalize(const double* __restrict__ partial, int nparts, int lmax, int nb, int sphere,
-                           double* __restrict__ zeta) {
+// zeta_l(b1,b2) = f_l * sum_parts partial[part][l][min b][max b]; f_l =
+// 4 pi/(2l+1) for the 3-D multipoles, 1 on the sphere.  32 consecutive entries
+// per block, eight threads an entry taking every eighth partial row and added
+// in a fixed order: one thread an entry walked 152 to 304 rows one latency
+// after another (75 us at 4400 entries; 6 us so).  blockIdx.y: the catalogue
+// of a batch.
+constexpr int kFinGroups = 8;
+__global__ void __launch_bounds__(32 * kFinGroups) k_finalize(const double* __restrict__ partial, int nparts, int lmax,
+                                                              int nb, int sphere, double* __restrict__ zeta) {
+  __shared__ double s[kFinGroups][32];
   const int total = (lmax + 1) * nb * nb;
-  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < total; o += gridDim.x * blockDim.x) {
-    const int l = o / (nb * nb), r = o % (nb * nb);
-    int b1 = r / nb, b2 = r % nb;
-    if (b1 > b2) {
-      int t = b1;
-      b1 = b2;
-      b2 = t;
-    }
-    const size_t idx = ((size_t)l * nb + b1) * nb + b2;
-    const size_t stride = (size_t)(lmax + 1) * nb * nb;
-    double s = 0.0;
-    for (int p = 0; p < nparts; ++p) s += partial[(size_t)p * stride + idx];
-    zeta[o] = sphere ? s : s * (4.0 * 3.14159265358979323846 / (2.0 * l + 1.0));
+  const size_t stride = (size_t)total;
+  partial += (size_t)blockIdx.y * nparts * stride;
+  zeta += (size_t)blockIdx.y * stride;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int o = blockIdx.x * 32 + lane;
+  const int l = o / (nb * nb), r = o - l * nb * nb;
+  const int b1 = r / nb, b2 = r - b1 * nb;
+  const bool own = o < total && b1 <= b2;
+  double v = 0.0;
+  if (own) {
+#pragma unroll 4
+    for (int p = g; p < nparts; p += kFinGroups) v += partial[(size_t)p * stride + o];
+  }
+  s[g][lane] = v;
+  __syncthreads();
+  if (own && g == 0) {
+#pragma unroll
+    for (int k = 1; k < kFinGroups; ++k) v += s[k][lane];
+    if (!sphere) v *= 4.0 * 3.14159265358979323846 / (2.0 * l + 1.0);
+    zeta[o] = v;
+    zeta[((size_t)l * nb + b2) * nb + b1] = v;
   }
 }
 
 cudaError_t launch_finalize(const double* partial, int nparts, int lmax, int nbins, double* zeta, bool sphere,
-                            cudaStream_t st) {
+                            int ncat, cudaStream_t st) {
   const int total = (lmax + 1) * nbins * nbins;
-  const int blocks = (total + 255) / 256;
-  k_finalize<<<blocks, 256, 0, st>>>(partial, nparts, lmax, nbins, sphere ? 1 : 0, zeta);
+  k_finalize<<<dim3((total + 31) / 32, ncat), 32 * kFinGroups, 0, st>>>(partial, nparts, lmax, nbins, sphere ? 1 : 0,
+                                                                        zeta);
   ++g_launches;
   return cudaGetLastError();
 }
 
 // Weighted pair sums of the two-point function from the same pass:
 // sum_p w_p sum_{j in b} w_j = sqrt(4 pi) sum_p w_p a_00(p, b), the a_00 column
-// of the M rows (col).  Block bx takes a fixed slice of the primaries, four
-// thread groups interleave over it, and the groups are added in a fixed order
-// to partial[bx][b] (FP64; accumulated over the chunks of one compute).
+// of the M rows (col).  Block bx takes a fixed slice of the primaries; its
+// 256 / nbins groups of nbins threads interleave over the slice (each thread
+// keeps its bin) and are added in a fixed order to partial[bx][b] (FP64;
+// accumulated over the chunks of one compute).
 __global__ void __launch_bounds__(256) k_pair_sums(const float* __restrict__ M, const float* __restrict__ w,
                                                    int64_t np, int nbins, int row, int col,
                                                    double* __restrict__ partial) {
-  __shared__ double s[4][kNbinsCap];
+  __shared__ double s[256];
   const int64_t nparts = gridDim.x, bx = blockIdx.x;
   const int64_t p0 = np * bx / nparts, p1 = np * (bx + 1) / nparts;
-  const int g = threadIdx.x >> 6, b = threadIdx.x & 63;
+  const int ng = 256 / nbins;
+  const int g = threadIdx.x / nbins, b = threadIdx.x - g * nbins;
   double acc = 0.0;
-  if (b < nbins)
-    for (int64_t p = p0 + g; p < p1; p += 4) acc += (double)w[p] * (double)M[(p * nbins + b) * row + col];
-  s[g][b] = acc;
+  if (g < ng) {
+    const float* m = M + ((p0 + g) * nbins + b) * (int64_t)row + col;
+    const int64_t step = (int64_t)ng * nbins * row;
+#pragma unroll 8
+    for (int64_t p = p0 + g; p < p1; p += ng, m += step) acc += (double)(__ldg(w + p)) * (double)__ldg(m);
+  }
+  s[threadIdx.x] = acc;
   __syncthreads();
   if (threadIdx.x < nbins) {
-    const int bb = threadIdx.x;
-    partial[bx * nbins + bb] += (s[0][bb] + s[1][bb]) + (s[2][bb] + s[3][bb]);
+    double v = 0.0;
+    for (int k = 0; k < ng; ++k) v += s[k * nbins + threadIdx.x];
+    partial[bx * nbins + threadIdx.x] += v;
   }
 }
 

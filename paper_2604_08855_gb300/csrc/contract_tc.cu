@@ -624,19 +624,34 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(const float* __restrict__
   }
 }
 
-// zeta_l(b1,b2) = 4 pi/(2l+1) * sum_split (D(b1,b2) + D(b2,b1)) / 2, in split order
-__global__ void k_finalize_tc(const double* __restrict__ partial, int nl, int nsplit, int nb,
-                              double* __restrict__ zeta) {
-  const int total = nl * nb * nb;
-  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < total; o += gridDim.x * blockDim.x) {
-    const int l = o / (nb * nb), r = o % (nb * nb);
-    const int b1 = r / nb, b2 = r % nb;
-    double s = 0.0;
-    for (int c = 0; c < nsplit; ++c) {
-      const double* blk = partial + ((size_t)l * nsplit + c) * nb * nb;
-      s += 0.5 * (blk[b1 * nb + b2] + blk[b2 * nb + b1]);
-    }
-    zeta[o] = s * (4.0 * 3.14159265358979323846 / (2.0 * l + 1.0));
+// zeta_l(b1,b2) = 4 pi/(2l+1) * sum_split (D(b1,b2) + D(b2,b1)) / 2: 32
+// consecutive entries per block, eight threads an entry taking every eighth
+// partial row (of its multipole) and added in a fixed order.  blockIdx.y: the
+// catalogue of a batch.
+constexpr int kFinTcGroups = 8;
+__global__ void __launch_bounds__(32 * kFinTcGroups) k_finalize_tc(const double* __restrict__ partial, int nl,
+                                                                   int nsplit, int nb, double* __restrict__ zeta) {
+  __shared__ double s[kFinTcGroups][32];
+  const int plane = nb * nb, total = nl * plane;
+  partial += (size_t)blockIdx.y * nsplit * total;
+  zeta += (size_t)blockIdx.y * total;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int o = blockIdx.x * 32 + lane;
+  const int l = o / plane, r = o - l * plane;
+  const int b1 = r / nb, b2 = r - b1 * nb;
+  double v = 0.0;
+  if (o < total) {
+    const double* blk = partial + (size_t)l * nsplit * plane;
+#pragma unroll 4
+    for (int c = g; c < nsplit; c += kFinTcGroups)
+      v += 0.5 * (blk[(size_t)c * plane + r] + blk[(size_t)c * plane + b2 * nb + b1]);
+  }
+  s[g][lane] = v;
+  __syncthreads();
+  if (o < total && g == 0) {
+#pragma unroll
+    for (int k = 1; k < kFinTcGroups; ++k) v += s[k][lane];
+    zeta[o] = v * (4.0 * 3.14159265358979323846 / (2.0 * l + 1.0));
   }
 }
 
@@ -767,9 +782,10 @@ cudaError_t launch_contract_tc(bool tf32, int64_t np, int nbins, int lmax, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize_tc(const double* partial, int lmax, int nsplit, int nbins, double* zeta, cudaStream_t st) {
+cudaError_t launch_finalize_tc(const double* partial, int lmax, int nsplit, int nbins, double* zeta, int ncat,
+                               cudaStream_t st) {
   const int total = (lmax + 1) * nbins * nbins;
-  k_finalize_tc<<<(total + 255) / 256, 256, 0, st>>>(partial, lmax + 1, nsplit, nbins, zeta);
+  k_finalize_tc<<<dim3((total + 31) / 32, ncat), 32 * kFinTcGroups, 0, st>>>(partial, lmax + 1, nsplit, nbins, zeta);
   ++g_launches;
   return cudaGetLastError();
 }

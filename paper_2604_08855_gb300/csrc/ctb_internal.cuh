@@ -341,7 +341,7 @@ struct ContractArgs {
   int sphere;              // 0: group l = components l^2 .. l^2+2l; 1: group m = {0} or {2m-1, 2m}
 };
 cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t st);
-int contract_fp32_blocks_per_sm(int nbins, int lmax, int row, int sphere);
+int contract_fp32_blocks_per_sm(int nbins, int row);
 
 // edge.cu
 void make_threej_table(int lmax, std::vector<double>& t);  // (a b c; 0 0 0)^2, [a][b][c], a,b,c <= lmax
@@ -350,8 +350,9 @@ cudaError_t launch_edge_correct(const double* zn, const double* zr, const double
 // partial[part][b] += sum over a fixed slice of the primaries of w_p * M[p][b][col]
 cudaError_t launch_pair_sums(const float* M, const float* w, int64_t np, int nbins, int row, int col,
                              double* partial, int nparts, cudaStream_t st);
+// ncat catalogues one after another: partial rows of nparts each, zeta rows
 cudaError_t launch_finalize(const double* partial, int nparts, int lmax, int nbins, double* zeta, bool sphere,
-                            cudaStream_t st);
+                            int ncat, cudaStream_t st);
 
 // contract_tc.cu -- tcgen05 contraction (BF16 hi/lo split or TF32)
 int tc_npad(int nbins);
@@ -366,7 +367,7 @@ cudaError_t launch_pack(bool tf32, const float* M, const float* wprim, int64_t n
 cudaError_t launch_contract_tc(bool tf32, int64_t np, int nbins, int lmax, const unsigned long long* h_lbase,
                                const unsigned long long* h_kp, void* opA, void* opH, void* opL, double* partial,
                                int nsplit, unsigned int* err, bool inject_stall, cudaStream_t st);
-cudaError_t launch_finalize_tc(const double* partial, int lmax, int nsplit, int nbins, double* zeta,
+cudaError_t launch_finalize_tc(const double* partial, int lmax, int nsplit, int nbins, double* zeta, int ncat,
                                cudaStream_t st);
 
 }  // namespace ctb

@@ -92,7 +92,7 @@ extern "C" int ctb_contract_noalloc(const float* alm, const float* w, int64_t np
   // blocks (as ctb_compute runs it), as far as the fixed array holds them, so
   // that each block's FP32 run over its slice of the primaries stays short.
   const int row = (ell_max + 1) * (ell_max + 1);
-  const int bps = contract_fp32_blocks_per_sm(nbins, ell_max, row, 0);
+  const int bps = contract_fp32_blocks_per_sm(nbins, row);
   if (bps < 1) return CTB_ERR_CUDA;
   const int nparts = (int)std::min<size_t>((size_t)bps * sc.nsm, kNoallocPartialDoubles / per_part);
   // the partial sums are accumulated in place: clear the part this call uses
@@ -113,7 +113,7 @@ extern "C" int ctb_contract_noalloc(const float* alm, const float* w, int64_t np
     e = launch_contract_fp32(ca, nparts, st);
     if (e != cudaSuccess) return CTB_ERR_CUDA;
   }
-  e = launch_finalize(sc.partial, nparts, ell_max, nbins, zeta_out, false, st);
+  e = launch_finalize(sc.partial, nparts, ell_max, nbins, zeta_out, false, 1, st);
   if (e != cudaSuccess) return CTB_ERR_CUDA;
   return CTB_OK;
 }
