@@ -192,17 +192,8 @@ int ensure_tables_sphere(ctb_ctx* c) {
   y.npass = 1;
   y.row = ((nc + 31) / 32) * 32;
   for (int i = 0; i < (kLmaxCap + 1) * (kLmaxCap + 1); ++i) y.slot[i] = i < nc ? (i == 0 ? 2 * c->lmax : i - 1) : -1;
-  // identity flush conversion (one entry per slot; padding slots map to 0)
-  std::vector<int2> tab(y.row);
-  for (int k = 0; k < y.row; ++k) {
-    const float one = k < nc ? 1.f : 0.f;
-    tab[k].x = k;
-    std::memcpy(&tab[k].y, &one, 4);
-  }
   CK(c, ensure(c, c->slot, sizeof(y.slot)));
   CK(c, cudaMemcpyAsync(c->slot.p, y.slot, sizeof(y.slot), cudaMemcpyHostToDevice, c->st));
-  CK(c, ensure(c, c->conv, tab.size() * sizeof(int2)));
-  CK(c, cudaMemcpyAsync(c->conv.p, tab.data(), tab.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
   CK(c, cudaStreamSynchronize(c->st));  // host sources go out of scope
   c->tables_ready = true;
   return CTB_OK;
@@ -225,10 +216,10 @@ int ensure_tables(ctb_ctx* c) {
   std::vector<int> slot_lm(c->lay.row, -1);
   for (int l = 0; l <= c->lmax; ++l)
     for (int m = -l; m <= l; ++m) slot_lm[c->lay.slot[l * l + l + m]] = l * 64 + (m + l);
-  std::vector<int2> tab;
+  std::vector<uint8_t> tab;
   if (!make_conversion(c->lay, tab)) return fail(c, CTB_ERR_CUDA, "internal: flush conversion table overflow");
-  CK(c, ensure(c, c->conv, tab.size() * sizeof(int2)));
-  CK(c, cudaMemcpyAsync(c->conv.p, tab.data(), tab.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
+  CK(c, ensure(c, c->conv, tab.size()));
+  CK(c, cudaMemcpyAsync(c->conv.p, tab.data(), tab.size(), cudaMemcpyHostToDevice, c->st));
   CK(c, ensure(c, c->slot_lm, slot_lm.size() * sizeof(int)));
   CK(c, cudaMemcpyAsync(c->slot_lm.p, slot_lm.data(), slot_lm.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CK(c, cudaStreamSynchronize(c->st));  // host sources go out of scope
@@ -543,7 +534,7 @@ int load_points(ctb_ctx* c, const double* xyz, const double* w, int64_t n) {
 // the next chunk's size follows the observed pairs per primary.
 
 struct PairPlan {
-  int wpb, alm_blocks, stream_blocks, count_blocks;
+  int wpb, stream_blocks, count_blocks;
   int64_t chunk_first;   // primaries in the first chunk (from the mean density)
   int64_t chunk_max;     // primaries per chunk at most
   uint64_t list_cap;     // neighbour-list entries per chunk at most
@@ -573,7 +564,6 @@ int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   int cbps = stream_blocks_per_sm(false, c->nbins, c->sphere != 0);
   if (bps < 1 || sbps < 1 || cbps < 1) return fail(c, CTB_ERR_CUDA, "pair kernels cannot be resident");
   pl->wpb = wpb;
-  pl->alm_blocks = bps * c->nsm;
   pl->stream_blocks = sbps * c->nsm;
   pl->count_blocks = cbps * c->nsm;
   const size_t rowbytes = (size_t)c->nbins * c->lay.row * sizeof(float);
@@ -705,7 +695,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   aa.counts = P<uint32_t>(c->counts);
   aa.offsets = P<uint32_t>(c->offsets);
   aa.M = P<float>(c->M);
-  aa.conv = P<int2>(c->conv);
+  aa.conv = P<uint8_t>(c->conv);
   aa.work = work;
   aa.nbins = nb;
   aa.row = c->lay.row;
@@ -763,10 +753,11 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     CK(c, launch_stream(sa, true, pl.stream_blocks, c->st));
     CK(c, cudaEventRecord(ev[2], c->st));
     CK(c, cudaMemsetAsync(work, 0, 8, c->st));
+    const int lists = lists_per_warp((double)tot / ((double)cnt * nb));
     if (c->sphere)
-      CK(c, launch_am(aa, c->lmax, pl.wpb, pl.alm_blocks, c->st));
+      CK(c, launch_am(aa, c->lmax, lists, pl.wpb, c->nsm, c->st));
     else
-      CK(c, launch_alm(aa, c->Lk, pl.wpb, c->nsm, c->st));
+      CK(c, launch_alm(aa, c->Lk, lists, pl.wpb, c->nsm, c->st));
     CK(c, cudaEventRecord(ev[3], c->st));
     if (contract) {
       // split the chunk at catalogue boundaries (a batch): each piece adds to its catalogue's partials

@@ -182,6 +182,22 @@ __host__ __device__ constexpr int local_slot(int L, int l, int m, int m0, int m1
   return 2 * (pairs_below(l, m0, m1) + (am - ms)) + (m < 0 ? 1 : 0);
 }
 
+// Units of the flush conversion (two slots each, see pair.cuh) are sorted by
+// degree: the entries that the units [32 r, 32 r + 32) of a pass need.
+__host__ __device__ constexpr int conv_round_entries(int L, int m0, int m1, int r) {
+  const int ms = m0 < 1 ? 1 : m0;
+  int most = 0;
+  for (int l = m0; l <= L; ++l) {
+    for (int m = m0; m <= m1 && m <= l; ++m) {
+      const int u = (m == 0 ? 2 * pairs_below(L + 1, m0, m1) + l : 2 * (pairs_below(l, m0, m1) + (m - ms))) / 2;
+      if (u / 32 == r && (l - m) / 2 + 1 > most) most = (l - m) / 2 + 1;
+    }
+  }
+  return most;
+}
+// bytes of a conversion table of `ncp` slots and `e` entries per unit
+__host__ __device__ constexpr int conv_table_bytes(int ncp, int e) { return ((ncp / 2) * e * 9 + 15) / 16 * 16; }
+
 // pair-kernel instantiation that serves a requested ell_max
 __host__ __device__ constexpr int lmax_kernel(int lmax) {
   return lmax <= 10 ? lmax : (lmax + 1) / 2 * 2;
@@ -209,9 +225,10 @@ unsigned long long sq_threshold(double edge, double unit);
 // recurrence constants (pair_dispatch.cu)
 void fill_beta(float* beta);   // beta_lm at [l*(kLmaxCap+1)+m]
 double norm_lm(int l, int m);  // C_lm of the real orthonormal Y_l,m
-// flush conversion table of kernel L: accumulator totals -> normalised a_lm
-// (entries padded per pass to conv_entries(L, m0_p), entry-major; see AlmArgs::conv)
-bool make_conversion(const Layout& lay, std::vector<int2>& tab);
+// flush conversion tables of kernel L, pass after pass: accumulator totals ->
+// normalised a_lm (entries padded per pass to conv_entries(L, m0_p), entry-
+// major: coefficient pairs, then source units; see pair.cuh)
+bool make_conversion(const Layout& lay, std::vector<uint8_t>& tab);
 
 // ---------------------------------------------------------------------------
 // kernels and launchers (all asynchronous on `st`)
@@ -311,8 +328,7 @@ struct AlmArgs {
   const uint32_t* offsets;        // [prim_count][nbins]
   const uint32_t* lists;
   float* M;                       // [prim_count][nbins][row]
-  const int2* conv;               // flush conversion, per pass p (at conv_pass_offset(L, p)): entry e of local
-                                  //   slot s at [e * ncp_p + s] = (source local slot, coefficient bits)
+  const uint8_t* conv;            // flush conversion tables, pass p at conv_pass_offset(L, p)
   unsigned long long* work;
   int nbins;
   int row;
@@ -323,9 +339,12 @@ struct AlmArgs {
 int alm_blocks_per_sm(int lmax_kernel, int warps_per_block);
 // sphere.cu: projected multipoles m = 0..mmax (mmax <= CTB_MMAX_CAP)
 int am_blocks_per_sm(int mmax, int warps_per_block);
-cudaError_t launch_am(const AlmArgs& a, int mmax, int warps_per_block, int nblocks, cudaStream_t st);
-// one launch per m-pass, each sized from its own occupancy on nsm SMs
-cudaError_t launch_alm(const AlmArgs& a, int lmax_kernel, int warps_per_block, int nsm, cudaStream_t st);
+cudaError_t launch_am(const AlmArgs& a, int mmax, int lists, int warps_per_block, int nsm, cudaStream_t st);
+// one launch per m-pass, each sized from its own occupancy on nsm SMs; lists:
+// (primary, bin) lists a warp accumulates side by side
+cudaError_t launch_alm(const AlmArgs& a, int lmax_kernel, int lists, int warps_per_block, int nsm, cudaStream_t st);
+// Lists per warp for lists of this mean length.
+int lists_per_warp(double mean_list);
 
 // contract.cu
 struct ContractArgs {

@@ -205,80 +205,107 @@ __device__ __forceinline__ void accum_pass(const AlmArgs& a, float2* acc, float 
 
 // Cross-lane sum of the accumulators through shared memory, in chunks of
 // at most kFlushChunk slots: every lane writes its chunk (stride W + 4 floats,
-// so 16-byte stores of 8 consecutive lanes cover all 32 banks), then lane l
-// sums the chunk's column block [l * W/32, (l+1) * W/32) over the 32 rows and
-// writes the totals to tot[chunk start + that block].
+// so 16-byte stores of 8 consecutive lanes cover all 32 banks), then the G =
+// 32 / S lanes of list s sum the chunk's columns over that list's G rows and
+// write its totals to tot[s][chunk start + column].  The 32 rows are written
+// and read once whatever S, so S lists share the cost of one flush.
 constexpr int kFlushChunk = 64;
 __host__ __device__ constexpr int flush_buf_floats(int ncp) {
   return 32 * ((ncp < kFlushChunk ? ncp : kFlushChunk) + 4);
 }
 
-template <int NCP, int C0>
+template <int NCP, int S, int C0>
 __device__ __forceinline__ void flush_chunks(const float2* acc, float* buf, float* tot, int lane) {
   if constexpr (C0 < NCP) {
     constexpr int W = NCP - C0 < kFlushChunk ? NCP - C0 : kFlushChunk;
-    constexpr int S = W + 4;
-    constexpr int V = W / 32;
-    float* row = buf + lane * S;
+    constexpr int ST = W + 4;
+    constexpr int G = 32 / S;
+    constexpr int V = W / G;  // columns per lane
+    float* row = buf + lane * ST;
 #pragma unroll
     for (int i = 0; i < W / 2; i += 2)
       *reinterpret_cast<float4*>(row + 2 * i) =
           make_float4(acc[C0 / 2 + i].x, acc[C0 / 2 + i].y, acc[C0 / 2 + i + 1].x, acc[C0 / 2 + i + 1].y);
     __syncwarp();
-    if constexpr (V == 4) {
-      float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+    const int sl = lane & (G - 1), s = lane / G;
+    const float* rows = buf + s * G * ST;
+    float* t = tot + s * NCP + C0;
+    if constexpr (V >= 4) {
+      // columns h 4 G + 4 sl .. + 3: contiguous over the list's lanes
 #pragma unroll
-      for (int r = 0; r < 32; r += 2) {
-        const float4 u = *reinterpret_cast<const float4*>(buf + r * S + 4 * lane);
-        const float4 v = *reinterpret_cast<const float4*>(buf + (r + 1) * S + 4 * lane);
-        s0.x += u.x; s0.y += u.y; s0.z += u.z; s0.w += u.w;
-        s1.x += v.x; s1.y += v.y; s1.z += v.z; s1.w += v.w;
+      for (int h = 0; h < V / 4; ++h) {
+        const int col = (h * G + sl) * 4;
+        float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+#pragma unroll
+        for (int r = 0; r < G; r += 2) {
+          const float4 u = *reinterpret_cast<const float4*>(rows + r * ST + col);
+          const float4 v = *reinterpret_cast<const float4*>(rows + (r + 1) * ST + col);
+          s0.x += u.x; s0.y += u.y; s0.z += u.z; s0.w += u.w;
+          s1.x += v.x; s1.y += v.y; s1.z += v.z; s1.w += v.w;
+        }
+        *reinterpret_cast<float4*>(t + col) = make_float4(s0.x + s1.x, s0.y + s1.y, s0.z + s1.z, s0.w + s1.w);
       }
-      *reinterpret_cast<float4*>(tot + C0 + 4 * lane) =
-          make_float4(s0.x + s1.x, s0.y + s1.y, s0.z + s1.z, s0.w + s1.w);
     } else if constexpr (V == 2) {
       float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
-      for (int r = 0; r < 32; r += 2) {
-        const float2 u = *reinterpret_cast<const float2*>(buf + r * S + 2 * lane);
-        const float2 v = *reinterpret_cast<const float2*>(buf + (r + 1) * S + 2 * lane);
+      for (int r = 0; r < G; r += 2) {
+        const float2 u = *reinterpret_cast<const float2*>(rows + r * ST + 2 * sl);
+        const float2 v = *reinterpret_cast<const float2*>(rows + (r + 1) * ST + 2 * sl);
         s0.x += u.x; s0.y += u.y;
         s1.x += v.x; s1.y += v.y;
       }
-      *reinterpret_cast<float2*>(tot + C0 + 2 * lane) = make_float2(s0.x + s1.x, s0.y + s1.y);
+      *reinterpret_cast<float2*>(t + 2 * sl) = make_float2(s0.x + s1.x, s0.y + s1.y);
     } else {
       float sm[V];
 #pragma unroll
       for (int c = 0; c < V; ++c) sm[c] = 0.f;
 #pragma unroll
-      for (int r = 0; r < 32; ++r)
+      for (int r = 0; r < G; ++r)
 #pragma unroll
-        for (int c = 0; c < V; ++c) sm[c] += buf[r * S + V * lane + c];
+        for (int c = 0; c < V; ++c) sm[c] += rows[r * ST + V * sl + c];
 #pragma unroll
-      for (int c = 0; c < V; ++c) tot[C0 + V * lane + c] = sm[c];
+      for (int c = 0; c < V; ++c) t[V * sl + c] = sm[c];
     }
     __syncwarp();  // the buffer is rewritten by the next chunk
-    flush_chunks<NCP, C0 + W>(acc, buf, tot, lane);
+    flush_chunks<NCP, S, C0 + W>(acc, buf, tot, lane);
   }
 }
 
-// Flush conversion of one pass, padded to E entries per slot and stored
-// entry-major in shared memory: entry e of local slot s at tab[e * NCP + s],
-// as (source local slot, coefficient bits); unused entries have coefficient
-// 0.  Lane l maps slots l, l + 32, ...: out[s] = sum_e coef * tot[src], the
-// loads of every entry independent of each other.
-template <int NCP, int E>
-__device__ __forceinline__ void flush_store(const int2* tab, const float* tot, float* __restrict__ out, int lane) {
+// Flush conversion of one pass, in units of two slots (2u, 2u + 1): the (+m,
+// -m) pair of one (l, m), or the m = 0 slots of l and l + 1.  Entry e of unit
+// u, at [e * NCP / 2 + u]: the coefficients of both slots and the unit whose
+// totals they multiply (zero coefficients pad the units with fewer entries).
+// Lane l maps units l, l + 32, ..: out[u] = sum_e coef * tot[src], one table
+// read for the S lists, the loads of every entry independent of each other.
+// `tab`: the coefficient pairs, then the source units as bytes.
+template <class Step, int S, int I>
+__device__ __forceinline__ void flush_store(const float2* tab, const float* tot, float* __restrict__ out, int64_t row,
+                                            int nlists, int lane) {
+  constexpr int U = Step::NCP / 2;
+  if constexpr (32 * I < U) {
+    const int u = lane + 32 * I;
+    if (32 * I + 32 <= U || u < U) {
+      float2 v[S];
+      if constexpr (Step::kConvE == 0) {  // the totals are the row itself
 #pragma unroll
-  for (int i = 0; i < NCP / 32; ++i) {
-    const int s = lane + 32 * i;
-    float v = 0.f;
+        for (int s = 0; s < S; ++s) v[s] = *reinterpret_cast<const float2*>(tot + s * Step::NCP + 2 * u);
+      } else {
+        constexpr int E = Step::conv_round(I);
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int2 t = tab[e * NCP + s];
-      v = fmaf(__int_as_float(t.y), tot[t.x], v);
+        for (int s = 0; s < S; ++s) v[s] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const float2 c = tab[e * U + u];
+          const float* t = tot + 2 * reinterpret_cast<const uint8_t*>(tab + U * Step::kConvE)[e * U + u];
+#pragma unroll
+          for (int s = 0; s < S; ++s) v[s] = __ffma2_rn(c, *reinterpret_cast<const float2*>(t + s * Step::NCP), v[s]);
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if (S == 1 || s < nlists) __stcs(reinterpret_cast<float2*>(out + s * row) + u, v[s]);
     }
-    __stcs(out + s, v);
+    flush_store<Step, S, I + 1>(tab, tot, out, row, nlists, lane);
   }
 }
 
@@ -331,8 +358,10 @@ struct Step3D {
   // Each launch runs one m-pass, so the full-lane copy of the step and the
   // general one are the only code in the instruction cache.
   static constexpr bool kFullLaneLoop = true;
-  // flush conversion entries per slot: moment degrees of the same parity
+  // flush conversion entries per unit: moment degrees of the same parity, and
+  // how many the units of one round of 32 need (they are sorted by degree)
   static constexpr int kConvE = conv_entries(L, M0);
+  static constexpr int conv_round(int r) { return conv_round_entries(L, M0, M1, r); }
   const AlmArgs& a;
   __device__ __forceinline__ void operator()(float2* acc, float w, float dx, float dy, float dz) const {
     const float ir = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
@@ -347,8 +376,11 @@ struct Step3D {
     const float dx = __int2float_rn((int)(q.x - P.x));
     const float dy = __int2float_rn((int)(q.y - P.y));
     const float dz = __int2float_rn((int)(q.z - P.z));
+    return unit(__uint_as_float(q.w), dx, dy, dz);
+  }
+  __device__ __forceinline__ float4 unit(float w, float dx, float dy, float dz) const {
     const float ir = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-    return make_float4(dx * ir, dy * ir, dz * ir, __uint_as_float(q.w));
+    return make_float4(dx * ir, dy * ir, dz * ir, w);
   }
   __device__ __forceinline__ void accum(float2* acc, float4 s) const { accum_pass<L, M0, M1>(a, acc, s.w, s.x, s.y, s.z); }
   static constexpr bool kPrep = L <= kSinglePassLmax;
@@ -364,6 +396,20 @@ __host__ __device__ constexpr bool use_prep() {
   else return false;
 }
 
+// Totals of the S lists held by the warp, in chunks of at most kFlushChunk
+// slots through the transpose buffer, into tot[list][slot]; then every lane
+// maps its units' totals to normalised a_lm (moments in the pass's basis ->
+// the Legendre values of their column).
+template <class Step, int S>
+__device__ __forceinline__ void flush(const float2* acc, float* __restrict__ out, int64_t row, int nlists,
+                                      const float2* ctab, float* sbuf, int lane) {
+  float* tot = sbuf + flush_buf_floats(Step::NCP);
+  flush_chunks<Step::NCP, S, 0>(acc, sbuf, tot, lane);
+  __syncwarp();
+  flush_store<Step, S, 0>(ctab, tot, out, row, nlists, lane);
+  __syncwarp();
+}
+
 // Accumulate one pass over one run and store it to the row; the loads for
 // the first iterations of `nxt` are issued inside the loop, so the next run
 // starts without a memory bubble.  `step` adds one neighbour (weight and
@@ -371,7 +417,7 @@ __host__ __device__ constexpr bool use_prep() {
 // Step::NCP accumulators.
 template <class Step>
 __device__ __forceinline__ void run_steps(const AlmArgs& a, const Step& step, Run cur, Run nxt, const uint4 P,
-                                          Prefetch& pf, float* __restrict__ out, const int2* ctab, float* sbuf,
+                                          Prefetch& pf, float* __restrict__ out, const float2* ctab, float* sbuf,
                                           int lane, uint32_t pe) {
   constexpr int NCP = Step::NCP;
   const uint32_t* __restrict__ lists = a.lists;
@@ -468,22 +514,145 @@ __device__ __forceinline__ void run_steps(const AlmArgs& a, const Step& step, Ru
     }
     step(acc, w, dx, dy, dz);
   }
-  // Warp totals, in chunks of at most kFlushChunk slots through the
-  // transpose buffer, into tot[slot]; then every lane maps its slots' totals
-  // to normalised a_lm: out[s] = sum_e coef_e * tot[src_e] (moments in the
-  // pass's basis -> the Legendre values of their column).
-  float* tot = sbuf + flush_buf_floats(NCP);
-  flush_chunks<NCP, 0>(acc, sbuf, tot, lane);
-  __syncwarp();
-  flush_store<NCP, Step::kConvE>(ctab, tot, out, lane);
-  __syncwarp();
+  flush<Step, 1>(acc, out, a.row, 1, ctab, sbuf, lane);
 }
 
-template <int L, int M0, int M1>
-__device__ __forceinline__ void run_pass(const AlmArgs& a, Run cur, Run nxt, const uint4 P, Prefetch& pf,
-                                         float* __restrict__ out, const int2* ctab, float* sbuf, int lane,
-                                         uint32_t pe) {
-  run_steps(a, Step3D<L, M0, M1>{a}, cur, nxt, P, pf, out, ctab, sbuf, lane, pe);
+// One primary's lists, one after another (S = 1): long lists.
+template <class Step>
+__device__ __forceinline__ void run_primary1(const AlmArgs& a, const Step& step, const uint32_t* s_off,
+                                             const uint32_t* s_n, const uint4 P, float* __restrict__ rows,
+                                             const float2* ctab, float* sbuf, int lane) {
+  const int nbins = a.nbins;
+  int b = 0;
+  while (b < nbins && s_n[b] == 0) ++b;
+  if (b >= nbins) return;
+  int nb = b + 1;
+  while (nb < nbins && s_n[nb] == 0) ++nb;
+  Run cur{s_off[b], s_n[b]};
+  Run nxt = nb < nbins ? Run{s_off[nb], s_n[nb]} : Run{0, 0};
+  // end of this primary's list range; its first lines go to L2 now
+  const uint32_t pe = s_off[nbins - 1] + s_n[nbins - 1];
+  if (lane < (int)kListPrefetchLines && cur.off + (uint32_t)lane * 32u < pe)
+    prefetch_l2(a.lists + cur.off + (uint32_t)lane * 32u);
+  Prefetch pf = prefetch_start(a.lists, a.pts, cur, nxt, P, lane);
+  while (true) {
+    run_steps(a, step, cur, nxt, P, pf, rows + (int64_t)b * a.row, ctab, sbuf, lane, pe);
+    b = nb;
+    if (b >= nbins) return;
+    cur = nxt;
+    nb = b + 1;
+    while (nb < nbins && s_n[nb] == 0) ++nb;
+    nxt = nb < nbins ? Run{s_off[nb], s_n[nb]} : Run{0, 0};
+  }
+}
+
+// One primary's lists S bins at a time, 32 / S lanes a list: short lists.
+// The flush costs the same for S lists as for one, and the lanes of a list
+// that is not a multiple of 32 are filled by the others'.  A group runs as
+// long as its longest list (neighbouring bins are alike in size), lanes past
+// the end of theirs adding a zero weight.  The loads run three steps ahead
+// of the accumulation on a cursor of their own that walks the primary's
+// groups: the record word, a step later its neighbour, a step later its
+// direction (where the step prepares it).
+template <class Step, int S>
+__device__ __forceinline__ void run_groups(const AlmArgs& a, const Step& step, const uint32_t* s_off,
+                                           const uint32_t* s_n, const uint4 P, float* __restrict__ rows,
+                                           const float2* ctab, float* sbuf, int lane) {
+  constexpr uint32_t G = 32 / S;
+  constexpr int NCP = Step::NCP;
+  const int nbins = a.nbins;
+  const int ls = lane / (int)G;
+  const uint32_t sl = lane & (G - 1);
+  // steps of the group at bin b: those of its longest list
+  auto iters = [&](int b) {
+    uint32_t n = 0;
+#pragma unroll
+    for (int s = 0; s < S; ++s) n = max(n, s_n[b + s]);
+    return (n + G - 1) / G;
+  };
+  auto skip = [&](int b, uint32_t& T) {  // first group with a neighbour at or after b
+    for (T = 0; b < nbins; b += S)
+      if ((T = iters(b)) != 0) break;
+    return b;
+  };
+  // a group's list words to L2, while the group before it is read
+  auto fetch = [&](int b) {
+    if (b >= nbins) return;
+    const uint32_t e = s_off[b + S - 1] + s_n[b + S - 1];
+    for (uint32_t w = s_off[b] + (uint32_t)lane * 32u; w < e; w += 1024u) prefetch_l2(a.lists + w);
+  };
+  uint32_t T;
+  int b = skip(0, T);
+  if (b >= nbins) return;
+  fetch(b);
+  // the load cursor: group lb, step lt of lT, this lane's list
+  int lb = b;
+  uint32_t lT = T, k = sl, n = s_n[b + ls], ln = 0;
+  const uint32_t* lp = a.lists + s_off[b + ls];
+  fetch(b + S);
+  auto word = [&] {
+    const uint32_t j = k < n ? __ldcs(lp + k) : kNone;
+    k += G;
+    if (++ln == lT) {  // the group's last step: on to the next
+      lb = skip(lb + S, lT);
+      ln = 0;
+      k = sl;
+      n = lb < nbins ? s_n[lb + ls] : 0u;
+      lp = a.lists + (lb < nbins ? s_off[lb + ls] : 0u);
+      fetch(lb + S);
+    }
+    return j;
+  };
+  uint32_t j0 = word(), j1 = word(), j2 = word();
+  uint4 q0 = gather(a.pts, j0, P), q1 = gather(a.pts, j1, P);
+  auto sep = [&](uint4 q, bool valid, float& w, float& dx, float& dy, float& dz) {
+    dx = valid ? __int2float_rn((int)(q.x - P.x)) : 1.f;  // an idle lane holds q = P
+    dy = __int2float_rn((int)(q.y - P.y));
+    dz = __int2float_rn((int)(q.z - P.z));
+    w = valid ? __uint_as_float(q.w) : 0.f;
+  };
+  float4 D = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (use_prep<Step>()) {
+    float w, dx, dy, dz;
+    sep(q0, j0 != kNone, w, dx, dy, dz);
+    D = step.unit(w, dx, dy, dz);
+  }
+  while (b < nbins) {
+    float2 acc[NCP / 2];
+#pragma unroll
+    for (int i = 0; i < NCP / 2; ++i) acc[i] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (uint32_t t = 0; t < T; ++t) {
+      float w, dx, dy, dz;
+      if constexpr (use_prep<Step>()) {
+        sep(q1, j1 != kNone, w, dx, dy, dz);
+        const float4 Dn = step.unit(w, dx, dy, dz);
+        q1 = gather(a.pts, j2, P);
+        j1 = j2;
+        j2 = word();
+        step.accum(acc, D);
+        D = Dn;
+      } else {
+        sep(q0, j0 != kNone, w, dx, dy, dz);
+        q0 = q1;
+        j0 = j1;
+        q1 = gather(a.pts, j2, P);
+        j1 = j2;
+        j2 = word();
+        step(acc, w, dx, dy, dz);
+      }
+    }
+    flush<Step, S>(acc, rows + (int64_t)b * a.row, a.row, nbins - b, ctab, sbuf, lane);
+    b = skip(b + S, T);
+  }
+}
+
+template <class Step, int S>
+__device__ __forceinline__ void run_primary(const AlmArgs& a, const Step& step, const uint32_t* s_off,
+                                            const uint32_t* s_n, const uint4 P, float* __restrict__ rows,
+                                            const float2* ctab, float* sbuf, int lane) {
+  if constexpr (S == 1) run_primary1(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+  else run_groups<Step, S>(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
 }
 
 // number of m-passes of kernel L, and the columns and row offset of pass P
@@ -504,14 +673,15 @@ __host__ __device__ constexpr int pass_base(int L, int P) {
   for (int p = 0; p < P; ++p) b += pass_ncp(L, p);
   return b;
 }
-// entries of the padded conversion tables of the passes before P
-__host__ __device__ constexpr int conv_pass_offset(int L, int P) {
-  int b = 0;
-  for (int p = 0; p < P; ++p) b += pass_ncp(L, p) * conv_entries(L, pass_m0(L, p));
-  return b;
+// bytes of one pass's conversion table ([E][U] coefficient pairs, then [E][U]
+// source units), and of the passes before P
+__host__ __device__ constexpr size_t conv_bytes(int L, int P) {
+  return (size_t)conv_table_bytes(pass_ncp(L, P), conv_entries(L, pass_m0(L, P)));
 }
-__host__ __device__ constexpr size_t alm_table_bytes(int L, int P) {
-  return (size_t)pass_ncp(L, P) * conv_entries(L, pass_m0(L, P)) * sizeof(int2);
+__host__ __device__ constexpr size_t conv_pass_offset(int L, int P) {
+  size_t b = 0;
+  for (int p = 0; p < P; ++p) b += conv_bytes(L, p);
+  return b;
 }
 
 // resident blocks of 4 warps the register budget of a pass is sized for
@@ -519,15 +689,34 @@ __host__ __device__ constexpr size_t alm_table_bytes(int L, int P) {
 // warps per scheduler allow 255 registers a thread, 3 allow 168, 4 allow 128)
 __host__ __device__ constexpr int alm_min_blocks(int ncp) { return ncp <= 32 ? 5 : (ncp <= 64 ? 4 : (ncp <= 136 ? 3 : 2)); }
 
-// per warp: the flush's transpose buffer, the slot totals, then the
-// primary's list offsets and counts
-__host__ __device__ constexpr size_t alm_smem_per_warp(int ncp) {
-  return (size_t)(flush_buf_floats(ncp) + ncp) * sizeof(float) + 2 * kNbinsCap * sizeof(uint32_t);
+// per warp: the flush's transpose buffer, the slot totals of S lists, then
+// the primary's list offsets and counts
+__host__ __device__ constexpr size_t alm_smem_per_warp(int ncp, int S) {
+  return (size_t)(flush_buf_floats(ncp) + S * ncp) * sizeof(float) + 2 * kNbinsCap * sizeof(uint32_t);
+}
+
+// Counts and offsets of primary i into shared memory (empty lists at the end
+// of its range past nbins, so that every group of S bins is whole); with
+// `zero`, the rows of its empty bins are cleared (the slots of every pass).
+__device__ __forceinline__ void load_lists(const AlmArgs& a, uint64_t ib, uint32_t* s_off, uint32_t* s_n, bool zero,
+                                           int lane) {
+  for (int b = lane; b < kNbinsCap; b += 32) {
+    const bool in = b < a.nbins;
+    const uint32_t n = in ? __ldg(a.counts + ib + b) : 0u;
+    s_n[b] = n;
+    s_off[b] = in ? __ldg(a.offsets + ib + b) : __ldg(a.offsets + ib + a.nbins - 1) + __ldg(a.counts + ib + a.nbins - 1);
+    if (zero && in && n == 0) {
+      float4* o = reinterpret_cast<float4*>(a.M + (ib + b) * (uint64_t)a.row);
+      for (int k = 0; k < a.row / 4; ++k) o[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  __syncwarp();
 }
 
 // One warp per primary: its (primary, bin) lists are consecutive runs of the
-// lists buffer; each list is accumulated in registers for m-pass P of kernel
-// L and flushed once, with the next list's first loads already in flight.
+// lists buffer; S of them at a time are accumulated in registers for m-pass P
+// of kernel L and flushed once, with the next lists' first loads already in
+// flight.  S: see alm_lists_per_warp.
 //
 // The passes of a kernel with several (l_max > 10) are separate kernels,
 // launched one after another.  With all passes in one launch, warps in
@@ -535,105 +724,84 @@ __host__ __device__ constexpr size_t alm_smem_per_warp(int ncp) {
 // every warp on the GPU runs the same pass body, and each pass gets its own
 // register budget (a pass with fewer accumulators runs more warps per SM).
 // The lists are re-read once per pass; the points stay in L2.
-template <int L, int P>
+template <int L, int P, int S>
 __global__ void __launch_bounds__(128, alm_min_blocks(pass_ncp(L, P))) k_alm(AlmArgs a) {
   constexpr int M0 = pass_m0(L, P), M1 = pass_m1(L, P), NCP = pass_ncp(L, P), BASE = pass_base(L, P);
-  constexpr int NTAB = NCP * conv_entries(L, M0);
-  extern __shared__ float s_alm[];
+  constexpr int TB = (int)conv_bytes(L, P);
+  extern __shared__ __align__(16) char s_alm[];
   // [the pass's conversion table | per warp: flush buffers, list offsets, counts]
-  int2* s_tab = reinterpret_cast<int2*>(s_alm);
-  for (int k = threadIdx.x; k < NTAB; k += blockDim.x) s_tab[k] = __ldg(a.conv + conv_pass_offset(L, P) + k);
+  for (int k = threadIdx.x; k < TB / 4; k += blockDim.x)
+    reinterpret_cast<uint32_t*>(s_alm)[k] = __ldg(reinterpret_cast<const uint32_t*>(a.conv + conv_pass_offset(L, P)) + k);
   __syncthreads();
+  const float2* ctab = reinterpret_cast<const float2*>(s_alm);
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
-  char* wbase = reinterpret_cast<char*>(s_alm) + alm_table_bytes(L, P) + (size_t)warp * alm_smem_per_warp(NCP);
+  char* wbase = s_alm + TB + (size_t)warp * alm_smem_per_warp(NCP, S);
   float* sbuf = reinterpret_cast<float*>(wbase);
-  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)(flush_buf_floats(NCP) + NCP) * sizeof(float));
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)(flush_buf_floats(NCP) + S * NCP) * sizeof(float));
   uint32_t* s_n = s_off + kNbinsCap;
-  const int nbins = a.nbins;
   while (true) {
     unsigned long long i = 0;
     if (lane == 0) i = atomicAdd(a.work, 1ull);
     i = __shfl_sync(0xffffffffu, i, 0);
     if (i >= (unsigned long long)a.prim_count) break;
-    const uint64_t ib = i * (uint64_t)nbins;
-    for (int b = lane; b < nbins; b += 32) {
-      const uint32_t n = __ldg(a.counts + ib + b);
-      s_n[b] = n;
-      s_off[b] = __ldg(a.offsets + ib + b);
-      if (P == 0 && n == 0) {
-        // empty bin: its row is zero (all passes' slots)
-        float4* o = reinterpret_cast<float4*>(a.M + (ib + b) * (uint64_t)a.row);
-        for (int k = 0; k < a.row / 4; ++k) o[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-    __syncwarp();
-    int b = 0;
-    while (b < nbins && s_n[b] == 0) ++b;
-    if (b < nbins) {
-      const int64_t gi = a.prim_begin + (int64_t)i;
-      const uint32_t sp = a.prim ? __ldg(a.prim + gi) : (uint32_t)gi;
-      const uint4 Pt = __ldg(a.pts + sp);
-      int nb = b + 1;
-      while (nb < nbins && s_n[nb] == 0) ++nb;
-      Run cur{s_off[b], s_n[b]};
-      Run nxt = nb < nbins ? Run{s_off[nb], s_n[nb]} : Run{0, 0};
-      // end of this primary's list range; its first lines go to L2 now
-      const uint32_t pe = s_off[nbins - 1] + s_n[nbins - 1];
-      if (lane < (int)kListPrefetchLines && cur.off + (uint32_t)lane * 32u < pe)
-        prefetch_l2(a.lists + cur.off + (uint32_t)lane * 32u);
-      Prefetch pf = prefetch_start(a.lists, a.pts, cur, nxt, Pt, lane);
-      while (true) {
-        run_pass<L, M0, M1>(a, cur, nxt, Pt, pf, a.M + (ib + b) * (uint64_t)a.row + BASE, s_tab, sbuf, lane, pe);
-        b = nb;
-        if (b >= nbins) break;
-        cur = nxt;
-        nb = b + 1;
-        while (nb < nbins && s_n[nb] == 0) ++nb;
-        nxt = nb < nbins ? Run{s_off[nb], s_n[nb]} : Run{0, 0};
-      }
-    }
+    const uint64_t ib = i * (uint64_t)a.nbins;
+    load_lists(a, ib, s_off, s_n, P == 0, lane);
+    const int64_t gi = a.prim_begin + (int64_t)i;
+    const uint32_t sp = a.prim ? __ldg(a.prim + gi) : (uint32_t)gi;
+    const uint4 Pt = __ldg(a.pts + sp);
+    run_primary<Step3D<L, M0, M1>, S>(a, Step3D<L, M0, M1>{a}, s_off, s_n, Pt, a.M + ib * (uint64_t)a.row + BASE, ctab,
+                                      sbuf, lane);
     __syncwarp();  // s_n / s_off are rewritten for the next primary
   }
 }
 
-template <int L, int P>
+template <int L, int P, int S>
+constexpr size_t alm_smem(int wpb) {
+  return conv_bytes(L, P) + (size_t)wpb * alm_smem_per_warp(pass_ncp(L, P), S);
+}
+
+template <int L, int P, int S>
 int alm_occupancy_pass(int wpb) {
-  const size_t smem = alm_table_bytes(L, P) + (size_t)wpb * alm_smem_per_warp(pass_ncp(L, P));
-  if (cudaFuncSetAttribute(k_alm<L, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  const size_t smem = alm_smem<L, P, S>(wpb);
+  if (cudaFuncSetAttribute(k_alm<L, P, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return 0;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_alm<L, P>, wpb * 32, smem) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_alm<L, P, S>, wpb * 32, smem) != cudaSuccess) return 0;
   return nb;
 }
 
 // passes P.. of kernel L: each launch resident-sized from its own occupancy,
 // the work counter zeroed before every pass after the first
-template <int L, int P>
+template <int L, int P, int S>
 cudaError_t launch_passes(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
   if constexpr (P >= pass_count(L)) {
     return cudaSuccess;
   } else {
-    const size_t smem = alm_table_bytes(L, P) + (size_t)wpb * alm_smem_per_warp(pass_ncp(L, P));
-    cudaError_t e = cudaFuncSetAttribute(k_alm<L, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int bps = alm_occupancy_pass<L, P>(wpb);
+    const int bps = alm_occupancy_pass<L, P, S>(wpb);
     if (bps < 1) return cudaErrorInvalidConfiguration;
+    cudaError_t e;
     if (P > 0) {
       e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), st);
       if (e != cudaSuccess) return e;
     }
-    k_alm<L, P><<<bps * nsm, wpb * 32, smem, st>>>(a);
+    k_alm<L, P, S><<<bps * nsm, wpb * 32, alm_smem<L, P, S>(wpb), st>>>(a);
     ++g_launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_passes<L, P + 1>(a, wpb, nsm, st);
+    return launch_passes<L, P + 1, S>(a, wpb, nsm, st);
   }
 }
 
 template <int L>
-cudaError_t launch_alm_L(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
-  return launch_passes<L, 0>(a, wpb, nsm, st);
+cudaError_t launch_alm_L(const AlmArgs& a, int lists, int wpb, int nsm, cudaStream_t st) {
+  switch (lists) {
+    case 2:
+      return launch_passes<L, 0, 2>(a, wpb, nsm, st);
+    case 4:
+      return launch_passes<L, 0, 4>(a, wpb, nsm, st);
+  }
+  return launch_passes<L, 0, 1>(a, wpb, nsm, st);
 }
 
 // the smallest occupancy over the passes (0: some pass cannot be resident)
@@ -642,7 +810,7 @@ int alm_occupancy_from(int wpb) {
   if constexpr (P >= pass_count(L)) {
     return 1 << 30;
   } else {
-    const int o = alm_occupancy_pass<L, P>(wpb);
+    const int o = alm_occupancy_pass<L, P, 1>(wpb);
     const int r = alm_occupancy_from<L, P + 1>(wpb);
     return o < r ? o : r;
   }

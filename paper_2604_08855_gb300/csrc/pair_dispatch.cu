@@ -11,7 +11,7 @@ namespace ctb {
 
 // explicit instantiations live in pair_[a-f].cu
 template <int L>
-cudaError_t launch_alm_L(const AlmArgs&, int, int, cudaStream_t);
+cudaError_t launch_alm_L(const AlmArgs&, int, int, int, cudaStream_t);
 template <int L>
 int alm_occupancy_L(int);
 
@@ -118,49 +118,53 @@ static std::vector<double> monic_in_basis(int l, int m, int m0) {
 // slot (m + k, +-m), q_k its basis: the Chebyshev T_k for the pass that
 // starts at m = 0, else p^{m0}_{m0+k}.  Normalised a_lm = C_lm sum_k D_k S_{m,k},
 // D the coefficients of p^m_l in that basis.
-bool make_conversion(const Layout& lay, std::vector<int2>& tab) {
+bool make_conversion(const Layout& lay, std::vector<uint8_t>& tab) {
   const int L = lay.L;
-  std::vector<std::vector<std::pair<int, float>>> ent(lay.row);
+  struct Ent {
+    int src;  // source slot of the even slot of a unit
+    float c[2];
+  };
+  std::vector<std::vector<Ent>> ent(lay.row / 2);  // by unit
   for (int p = 0; p < lay.npass; ++p) {
     const int m0 = lay.m0[p];
     for (int am = m0; am <= lay.m1[p] && am <= L; ++am) {
       for (int l = am; l <= L; ++l) {
         const std::vector<double> d = m0 == 0 ? monic_in_T(l, am) : monic_in_basis(l, am, m0);
-        double dmax = 0.0;
-        for (double v : d) dmax = std::fmax(dmax, std::fabs(v));
-        for (int sg = (am == 0 ? 1 : -1); sg <= 1; sg += 2) {
-          const int m = sg * am;
-          const int s = lay.slot[l * l + l + m];
-          const double nrm = norm_lm(l, m);
-          for (int k = 0; k <= l - am; ++k) {
-            if (std::fabs(d[k]) <= 1e-13 * dmax) continue;  // the other parity: exactly zero
-            const int sl = am + k;
-            ent[s].push_back({lay.slot[sl * sl + sl + m], (float)(nrm * d[k])});
+        const int s = lay.slot[l * l + l + am];
+        std::vector<Ent>& v = ent[s / 2];
+        // degrees of the polynomial's parity, from the highest (the others
+        // are exactly zero).  Column 0: slots l and l + 1 share a unit, and
+        // their e-th entries lie in one unit too.
+        for (int k = l - am, e = 0; k >= 0; k -= 2, ++e) {
+          const int sl = am + k;
+          const int src = lay.slot[sl * sl + sl + am];
+          const float c = (float)(norm_lm(l, am) * d[k]);
+          if (am > 0) {
+            v.push_back({src, {c, (float)(norm_lm(l, -am) * d[k])}});
+          } else {
+            if ((int)v.size() <= e) v.push_back({src & ~1, {0.f, 0.f}});
+            if (v[e].src != (src & ~1) || (src & 1) != (s & 1)) return false;
+            v[e].c[s & 1] = c;
           }
         }
       }
     }
   }
-  // padded, entry-major per pass; local slot numbers
+  // padded, entry-major per pass; local units
   tab.clear();
   for (int p = 0; p < lay.npass; ++p) {
-    const int E = conv_entries(L, lay.m0[p]), ncp = lay.ncp[p], base = lay.base[p];
+    const int E = conv_entries(L, lay.m0[p]), U = lay.ncp[p] / 2, base = lay.base[p];
     const size_t t0 = tab.size();
-    tab.resize(t0 + (size_t)E * ncp);
-    for (int sl = 0; sl < ncp; ++sl) {
-      const auto& v = ent[base + sl];
-      if ((int)v.size() > E) return false;
+    tab.resize(t0 + (size_t)conv_table_bytes(lay.ncp[p], E), 0);
+    for (int u = 0; u < U; ++u) {
+      const auto& v = ent[base / 2 + u];
+      if ((int)v.size() > conv_round_entries(L, lay.m0[p], lay.m1[p], u / 32)) return false;
       for (int e = 0; e < E; ++e) {
-        int2 t;
-        if (e < (int)v.size()) {
-          t.x = v[e].first - base;
-          float cf = v[e].second;
-          std::memcpy(&t.y, &cf, 4);
-        } else {
-          t.x = sl;
-          t.y = 0;  // +0.0f
-        }
-        tab[t0 + (size_t)e * ncp + sl] = t;
+        const size_t k = (size_t)e * U + u;
+        const bool in = e < (int)v.size();
+        const float c[2] = {in ? v[e].c[0] : 0.f, in ? v[e].c[1] : 0.f};
+        std::memcpy(tab.data() + t0 + k * 8, c, 8);
+        tab[t0 + (size_t)E * U * 8 + k] = (uint8_t)(in ? (v[e].src - base) / 2 : u);
       }
     }
   }
@@ -180,11 +184,25 @@ int alm_blocks_per_sm(int L, int wpb) {
   }
 }
 
-cudaError_t launch_alm(const AlmArgs& a, int L, int wpb, int nsm, cudaStream_t st) {
+// Four lists side by side below a mean of 160 neighbours, two below 800, one
+// above.  A flush costs the same for S lists as for one, but a group of S runs
+// as long as its longest list and its steps carry the validity of each lane
+// (about 5 % more).  Accumulation with 1 / 2 / 4 lists (8: slower than 4
+// except at 8 neighbours a list, where they tie):
+//   mean list 8 (20k uniform points, l_max 10)      0.226 / 0.144 / 0.116 ms
+//   28 (200k points, l_max 20)                      24.0 / 16.7 / 14.7 ms
+//   80 (24 mock catalogues, l_max 10)               52.3 / 39.4 / 39.4 ms
+//   132 (3.1M-pixel sphere, m_max 8)                38.0 / 29.6 / 28.4 ms
+//   522 (cut sky of 800k points, l_max 10)          118.1 / 111.1 / 113.2 ms
+//   525 (250k primaries of 4M, l_max 20)            134.1 / 132.3 / 145.7 ms
+//   1680 (10^6 points, l_max 10)                    221.5 / 243.1 / 274.0 ms
+int lists_per_warp(double mean_list) { return mean_list < 160.0 ? 4 : (mean_list < 800.0 ? 2 : 1); }
+
+cudaError_t launch_alm(const AlmArgs& a, int L, int lists, int wpb, int nsm, cudaStream_t st) {
   switch (L) {
 #define CASE(X) \
   case X:       \
-    return launch_alm_L<X>(a, wpb, nsm, st);
+    return launch_alm_L<X>(a, lists, wpb, nsm, st);
     CASE(0) CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8) CASE(9) CASE(10)
     CASE(12) CASE(14) CASE(16) CASE(18) CASE(20)
 #undef CASE

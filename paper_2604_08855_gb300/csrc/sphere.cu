@@ -26,7 +26,7 @@ template <int K>
 struct StepSphere {
   static constexpr int NCP = round32(2 * K + 1);
   static constexpr bool kFullLaneLoop = true;
-  static constexpr int kConvE = 1;  // the row holds a_m itself: one identity entry per slot
+  static constexpr int kConvE = 0;  // the row holds a_m itself: no conversion
   float ex, ey;      // east unit vector (its z component is zero)
   float nx, ny, nz;  // north unit vector
   __device__ __forceinline__ void operator()(float2* acc, float w, float dx, float dy, float dz) const {
@@ -81,96 +81,69 @@ __device__ __forceinline__ StepSphere<0> frame_at(float x, float y, float z) {
   return f;
 }
 
-template <int K>
-constexpr size_t am_smem_per_warp() {
-  return alm_smem_per_warp(StepSphere<K>::NCP);
-}
-template <int K>
-constexpr size_t am_table_bytes() {
-  return (size_t)StepSphere<K>::NCP * sizeof(int2);
-}
-
-// One warp per primary, one run per non-empty (primary, bin) list, as in k_alm.
-template <int K>
+// One warp per primary, one run per group of S (primary, bin) lists, as in k_alm.
+template <int K, int S>
 __global__ void __launch_bounds__(128) k_am(AlmArgs a) {
-  extern __shared__ float s_am[];
-  // [identity conversion table | per warp: flush buffers, list offsets, counts]
-  int2* s_tab = reinterpret_cast<int2*>(s_am);
-  for (int k = threadIdx.x; k < StepSphere<K>::NCP; k += blockDim.x) s_tab[k] = __ldg(a.conv + k);
-  __syncthreads();
+  extern __shared__ __align__(16) char s_am[];
+  constexpr int NCP = StepSphere<K>::NCP;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
-  char* wbase = reinterpret_cast<char*>(s_am) + am_table_bytes<K>() + (size_t)warp * am_smem_per_warp<K>();
+  // per warp: flush buffers, list offsets, counts
+  char* wbase = s_am + (size_t)warp * alm_smem_per_warp(NCP, S);
   float* sbuf = reinterpret_cast<float*>(wbase);
-  uint32_t* s_off =
-      reinterpret_cast<uint32_t*>(wbase + (size_t)(flush_buf_floats(StepSphere<K>::NCP) + StepSphere<K>::NCP) * sizeof(float));
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)(flush_buf_floats(NCP) + S * NCP) * sizeof(float));
   uint32_t* s_n = s_off + kNbinsCap;
-  const int nbins = a.nbins;
   while (true) {
     unsigned long long i = 0;
     if (lane == 0) i = atomicAdd(a.work, 1ull);
     i = __shfl_sync(0xffffffffu, i, 0);
     if (i >= (unsigned long long)a.prim_count) break;
-    const uint64_t ib = i * (uint64_t)nbins;
-    for (int b = lane; b < nbins; b += 32) {
-      const uint32_t n = __ldg(a.counts + ib + b);
-      s_n[b] = n;
-      s_off[b] = __ldg(a.offsets + ib + b);
-      if (n == 0) {
-        float4* o = reinterpret_cast<float4*>(a.M + (ib + b) * (uint64_t)a.row);
-        for (int k = 0; k < a.row / 4; ++k) o[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-    __syncwarp();
-    int b = 0;
-    while (b < nbins && s_n[b] == 0) ++b;
-    if (b < nbins) {
-      const int64_t gi = a.prim_begin + (int64_t)i;
-      const uint32_t sp = a.prim ? __ldg(a.prim + gi) : (uint32_t)gi;
-      const uint4 P = __ldg(a.pts + sp);
-      const StepSphere<0> f0 = frame_at(fmaf((float)P.x, a.sph_unit, a.sph_origin[0]),
-                                        fmaf((float)P.y, a.sph_unit, a.sph_origin[1]),
-                                        fmaf((float)P.z, a.sph_unit, a.sph_origin[2]));
-      const StepSphere<K> step{f0.ex, f0.ey, f0.nx, f0.ny, f0.nz};
-      int nb = b + 1;
-      while (nb < nbins && s_n[nb] == 0) ++nb;
-      Run cur{s_off[b], s_n[b]};
-      Run nxt = nb < nbins ? Run{s_off[nb], s_n[nb]} : Run{0, 0};
-      const uint32_t pe = s_off[nbins - 1] + s_n[nbins - 1];
-      if (lane < (int)kListPrefetchLines && cur.off + (uint32_t)lane * 32u < pe)
-        prefetch_l2(a.lists + cur.off + (uint32_t)lane * 32u);
-      Prefetch pf = prefetch_start(a.lists, a.pts, cur, nxt, P, lane);
-      while (true) {
-        run_steps(a, step, cur, nxt, P, pf, a.M + (ib + b) * (uint64_t)a.row, s_tab, sbuf, lane, pe);
-        b = nb;
-        if (b >= nbins) break;
-        cur = nxt;
-        nb = b + 1;
-        while (nb < nbins && s_n[nb] == 0) ++nb;
-        nxt = nb < nbins ? Run{s_off[nb], s_n[nb]} : Run{0, 0};
-      }
-    }
+    const uint64_t ib = i * (uint64_t)a.nbins;
+    load_lists(a, ib, s_off, s_n, true, lane);
+    const int64_t gi = a.prim_begin + (int64_t)i;
+    const uint32_t sp = a.prim ? __ldg(a.prim + gi) : (uint32_t)gi;
+    const uint4 P = __ldg(a.pts + sp);
+    const StepSphere<0> f0 = frame_at(fmaf((float)P.x, a.sph_unit, a.sph_origin[0]),
+                                      fmaf((float)P.y, a.sph_unit, a.sph_origin[1]),
+                                      fmaf((float)P.z, a.sph_unit, a.sph_origin[2]));
+    const StepSphere<K> step{f0.ex, f0.ey, f0.nx, f0.ny, f0.nz};
+    run_primary<StepSphere<K>, S>(a, step, s_off, s_n, P, a.M + ib * (uint64_t)a.row, nullptr, sbuf, lane);
     __syncwarp();
   }
 }
 
-template <int K>
+template <int K, int S>
+static constexpr size_t am_smem(int wpb) {
+  return (size_t)wpb * alm_smem_per_warp(StepSphere<K>::NCP, S);
+}
+
+template <int K, int S>
 static int am_occupancy_K(int wpb) {
-  const size_t smem = am_table_bytes<K>() + (size_t)wpb * am_smem_per_warp<K>();
-  if (cudaFuncSetAttribute(k_am<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  const size_t smem = am_smem<K, S>(wpb);
+  if (cudaFuncSetAttribute(k_am<K, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_am<K>, wpb * 32, smem) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_am<K, S>, wpb * 32, smem) != cudaSuccess) return 0;
   return nb;
 }
 
-template <int K>
-static cudaError_t launch_am_K(const AlmArgs& a, int wpb, int nblocks, cudaStream_t st) {
-  const size_t smem = am_table_bytes<K>() + (size_t)wpb * am_smem_per_warp<K>();
-  cudaError_t e = cudaFuncSetAttribute(k_am<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_am<K><<<nblocks, wpb * 32, smem, st>>>(a);
+template <int K, int S>
+static cudaError_t launch_am_KS(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
+  const int bps = am_occupancy_K<K, S>(wpb);
+  if (bps < 1) return cudaErrorInvalidConfiguration;
+  k_am<K, S><<<bps * nsm, wpb * 32, am_smem<K, S>(wpb), st>>>(a);
   ++g_launches;
   return cudaGetLastError();
+}
+
+template <int K>
+static cudaError_t launch_am_K(const AlmArgs& a, int lists, int wpb, int nsm, cudaStream_t st) {
+  switch (lists) {
+    case 2:
+      return launch_am_KS<K, 2>(a, wpb, nsm, st);
+    case 4:
+      return launch_am_KS<K, 4>(a, wpb, nsm, st);
+  }
+  return launch_am_KS<K, 1>(a, wpb, nsm, st);
 }
 
 #define CTB_SPHERE_CASES(X) \
@@ -180,7 +153,7 @@ int am_blocks_per_sm(int mmax, int wpb) {
   switch (mmax) {
 #define CASE(K) \
   case K:       \
-    return am_occupancy_K<K>(wpb);
+    return am_occupancy_K<K, 1>(wpb);
     CTB_SPHERE_CASES(CASE)
 #undef CASE
     default:
@@ -188,11 +161,11 @@ int am_blocks_per_sm(int mmax, int wpb) {
   }
 }
 
-cudaError_t launch_am(const AlmArgs& a, int mmax, int wpb, int nblocks, cudaStream_t st) {
+cudaError_t launch_am(const AlmArgs& a, int mmax, int lists, int wpb, int nsm, cudaStream_t st) {
   switch (mmax) {
 #define CASE(K) \
   case K:       \
-    return launch_am_K<K>(a, wpb, nblocks, st);
+    return launch_am_K<K>(a, lists, wpb, nsm, st);
     CTB_SPHERE_CASES(CASE)
 #undef CASE
     default:
