@@ -48,14 +48,14 @@ struct Geom {
   int lmax;            // requested ell_max
   float rlo2_u;        // r_min^2 in units^2, widened by 1e-5 (float pre-filter)
   float rhi2_u;        // r_max^2 in units^2, widened by 1e-5 (float pre-filter)
-  float rmin_u;        // r_min in units
-  float inv_dr_u;      // nbins / (r_max - r_min) in 1/units
+  float inv_dr_u;      // nbins / (r_max - r_min) in 1/units (sphere: of the angles)
+  float bin_shift;     // -r_min * inv_dr - 1/2: bin coordinate minus 1/2 = r inv_dr + bin_shift
+  float half_bin;      // 1/2 less the float error of that coordinate (padded): within it the bin is certain
   float rcell;         // r_max in cell units, padded by a small slack
   float cell_scale;    // nc / 2^shift : units -> cell units
+  int long_rows;       // 1: a primary's cell rows hold hundreds of points
   int general;         // 1: bin edges not linear in r (sphere: chords of linear angles)
   float half_unit;     // sphere: unit / 2, so that chord / 2 = r_units * half_unit
-  float tmin;          // sphere: theta_min (radians)
-  float inv_dt;        // sphere: nbins / (theta_max - theta_min)
   float shell_c[3];    // sphere: the origin of coordinates in cell units (x in x-cells)
   float shell_r2lo;    // sphere: (smallest |p|)^2 and (largest |p|)^2 of the catalogue in
   float shell_r2hi;    //   (y, z) cell units squared, padded: every point lies in that shell
@@ -311,10 +311,10 @@ struct StreamArgs {
   uint8_t* codes;                 // bin code per candidate (written: count, read: fill)
   unsigned long long code_cap;    // bytes of codes
   unsigned long long* code_total; // code bytes of this launch (count pass; the range allocator)
-  unsigned long long* code_base;  // [prim_count][row_blocks] start of each row block's codes
+  unsigned long long* code_base;  // [prim_count][row_blocks] start of each batch's codes (at most one a row block)
   Geom g;
 };
-int stream_blocks_per_sm(bool fill, int nbins, bool general);
+int stream_blocks_per_sm(const Geom& g, bool fill);
 cudaError_t launch_stream(const StreamArgs& a, bool fill, int nblocks, cudaStream_t st);
 constexpr int kStreamThreads = 256;
 

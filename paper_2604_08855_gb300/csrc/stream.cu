@@ -14,15 +14,33 @@
 // Two passes per chunk of primaries:
 //   count: pairs per (primary, bin)  -> counts (then an exclusive scan on the
 //          host stream gives each (primary, bin) list its start); the bin of
-//          every candidate is also stored as one byte (kNoBin: not a pair):
-//          each block of 32 rows takes a range of its warp's pool in the code
-//          buffer, and each cell-row segment in it starts on a 4-byte boundary
+//          every candidate is also stored as one byte (kNoBin: not a pair)
 //   fill:  walks the same candidate stream, reads the stored bin codes four
 //          per lane (no point loads, no distances) and writes each pair's
 //          neighbour index into its (primary, bin) list (match_any ranks the
 //          lanes that share a bin)
-// The kernel holds few registers, so many warps per SM hide the load latency
-// that dominates this phase.
+//
+// The candidate stream.  A row's point ranges (segments) are short where the
+// catalogue is sparse or the points lie on a surface: 0.4 points a row in a
+// 20k-point box, 15 on a half-degree sphere map.  So segments are collected
+// from the row blocks into a list in shared memory (a batch), and the batch is
+// walked as one stream, 32 candidates a step, whatever segments they come
+// from.  A lane finds its segment from the boundaries that fall into the
+// step's window: the 32 lanes hold the next 32 boundaries, one warp
+// OR-reduction makes them a bit mask, and the bits at or below the lane count
+// the segments passed.  Steps inside one segment skip the search.  Walking
+// segment by segment spent a step on every segment however short, and about
+// 25 instructions more.
+//
+// Codes.  Four steps share one 32-bit word per lane (byte k: step k of the
+// group of 128 candidates), so the count pass stores every fourth step, and a
+// step of the fill pass ranks 32 consecutive candidates.  match_any takes 8
+// cycles per distinct value (measured), which bounds the fill: 32 neighbours
+// along a row share few bins, where 32 taken four apart share twice as few.
+//
+// An idle lane of the count pass looks at the primary itself (r = 0, never a
+// pair), and the codes past the stream's end read kNoBin, so neither pass
+// tests positions.
 #include <algorithm>
 
 #include "ctb_internal.cuh"
@@ -33,9 +51,22 @@ __device__ __forceinline__ float slab_dist(int d, float fr) {
   return d > 0 ? (float)d - fr : (d < 0 ? (float)(-d - 1) + fr : 0.f);
 }
 
-__device__ __forceinline__ int pmod(int a, int n) {
-  int r = a % n;
-  return r < 0 ? r + n : r;
+// a in [-n, 2 n) wrapped into [0, n): a row window reaches at most half a
+// period to either side of its primary's cell
+__device__ __forceinline__ int wrap1(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
+
+// sqrt to 2^-22: a row's ends carry a slack of 1e-3 cells (g.rcell, and the
+// shell's padding)
+__device__ __forceinline__ float sqrt_fast(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 constexpr uint8_t kNoBin = 0xff;  // bin code of a candidate that is not a pair
@@ -48,6 +79,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // Geometry of one primary's row window, shared by both passes.
 struct RowWin {
   int W, off0, nrows;
+  uint32_t invW;  // ceil(2^32 / W): t / W = umulhi(t, invW) for t < 2^32 / W
   bool fullwin;
   float R2, fx, fry, frz;  // (r_max in cell units)^2; primary's x in x-cell units, y and z fractions
   float xs;                // x-cells per cell (ncx / nc)
@@ -55,6 +87,11 @@ struct RowWin {
   uint32_t cbase;
 };
 
+// The count and the fill pass have to see the same ranges to the bit, so every
+// product that the compiler could fuse with a sum is written out (__fmul_rn,
+// __fmaf_rn): the two instantiations fused differently, and a row's end moved
+// by an x-cell in one of them.
+//
 // The point ranges of row t of the window (up to two: periodic wrap in x,
 // or the two crossings of the sphere's shell); empty ranges have s >= e.
 // SHELL (sphere mode): every point lies in the shell of g.shell_r2lo ..
@@ -66,27 +103,28 @@ __device__ __forceinline__ void row_ranges(const StreamArgs& a, const Geom& g, c
   const uint32_t nc = g.nc;
   s0 = e0 = s1 = e1 = 0;
   if (t >= rw.nrows) return;
-  const int dy = t % rw.W + rw.off0, dz = t / rw.W + rw.off0;
+  const int tz = rw.W == 1 ? t : (int)__umulhi((uint32_t)t, rw.invW);
+  const int dy = t - tz * rw.W + rw.off0, dz = tz + rw.off0;
   float gy = slab_dist(dy, rw.fry), gz = slab_dist(dz, rw.frz);
   if (rw.fullwin) {
     gy = fminf(gy, fminf(slab_dist(dy - (int)nc, rw.fry), slab_dist(dy + (int)nc, rw.fry)));
     gz = fminf(gz, fminf(slab_dist(dz - (int)nc, rw.frz), slab_dist(dz + (int)nc, rw.frz)));
   }
-  const float rho2 = gy * gy + gz * gz;
+  const float rho2 = __fmaf_rn(gy, gy, __fmul_rn(gz, gz));
   int cy = rw.cyp + dy, cz = rw.czp + dz;
   bool ok = rho2 < rw.R2;
   if (g.periodic) {
-    cy = pmod(cy, (int)nc);
-    cz = pmod(cz, (int)nc);
+    cy = wrap1(cy, (int)nc);
+    cz = wrap1(cz, (int)nc);
   } else {
     ok = ok && cy >= 0 && cy < (int)nc && cz >= 0 && cz < (int)nc;
   }
   if (!ok) return;
   // the row's x-range in x-cells (a row is split xs times finer along x
   // than across, so its ends overshoot the ball by less)
-  const float hw = sqrtf(rw.R2 - rho2) * rw.xs;
+  const float hw = __fmul_rn(sqrt_fast(__fsub_rn(rw.R2, rho2)), rw.xs);
   const int nx = (int)g.ncx;
-  int lo = (int)floorf(rw.fx - hw), hi = (int)floorf(rw.fx + hw);
+  int lo = (int)floorf(__fsub_rn(rw.fx, hw)), hi = (int)floorf(__fadd_rn(rw.fx, hw));
   const uint32_t rb = rw.cbase + ((uint32_t)cz * nc + (uint32_t)cy) * (uint32_t)nx;
   int a0 = 1, b0 = 0, a1 = 1, b1 = 0;
   if constexpr (SHELL) {
@@ -95,15 +133,15 @@ __device__ __forceinline__ void row_ranges(const StreamArgs& a, const Geom& g, c
     const float ny = ly > 0.f ? ly : (ly + 1.f < 0.f ? -(ly + 1.f) : 0.f);
     const float nz = lz > 0.f ? lz : (lz + 1.f < 0.f ? -(lz + 1.f) : 0.f);
     const float fy = fmaxf(fabsf(ly), fabsf(ly + 1.f)), fz = fmaxf(fabsf(lz), fabsf(lz + 1.f));
-    const float d2min = ny * ny + nz * nz, d2max = fy * fy + fz * fz;
+    const float d2min = __fmaf_rn(ny, ny, __fmul_rn(nz, nz)), d2max = __fmaf_rn(fy, fy, __fmul_rn(fz, fz));
     if (d2min >= g.shell_r2hi) return;
     // x offsets (x-cells) of the shell along the row: [alo, ahi] either side of the centre
-    const float ahi = sqrtf(g.shell_r2hi - d2min) * rw.xs;
-    const float alo = g.shell_r2lo > d2max ? sqrtf(g.shell_r2lo - d2max) * rw.xs : 0.f;
-    const float xl = rw.fx - hw, xh = rw.fx + hw, cx = g.shell_c[0];
+    const float ahi = __fmul_rn(sqrt_fast(__fsub_rn(g.shell_r2hi, d2min)), rw.xs);
+    const float alo = g.shell_r2lo > d2max ? __fmul_rn(sqrt_fast(__fsub_rn(g.shell_r2lo, d2max)), rw.xs) : 0.f;
+    const float xl = __fsub_rn(rw.fx, hw), xh = __fadd_rn(rw.fx, hw), cx = g.shell_c[0];
     // the ball's x-range meets the upper crossing [cx + alo, cx + ahi] and the lower one
-    const float pl = fmaxf(xl, cx + alo), ph = fminf(xh, cx + ahi);
-    const float ml = fmaxf(xl, cx - ahi), mh = fminf(xh, cx - alo);
+    const float pl = fmaxf(xl, __fadd_rn(cx, alo)), ph = fminf(xh, __fadd_rn(cx, ahi));
+    const float ml = fmaxf(xl, __fsub_rn(cx, ahi)), mh = fminf(xh, __fsub_rn(cx, alo));
     int ma = nx, mb = -1, pa = nx, pb = -1;
     if (ml <= mh) {
       ma = max((int)floorf(ml), 0);
@@ -130,7 +168,7 @@ __device__ __forceinline__ void row_ranges(const StreamArgs& a, const Geom& g, c
       a0 = 0;
       b0 = nx - 1;
     } else {
-      const int lm = pmod(lo, nx), hm = pmod(hi, nx);
+      const int lm = wrap1(lo, nx), hm = wrap1(hi, nx);
       a0 = lm;
       if (lm <= hm) {
         b0 = hm;
@@ -154,34 +192,63 @@ __device__ __forceinline__ void row_ranges(const StreamArgs& a, const Geom& g, c
   }
 }
 
+// A batch of segments in shared memory: a row block adds at most 64, and the
+// batch is walked once it holds more than kSegCap - 64.
+constexpr int kSegCap = 96;
+
+struct WarpSegs {
+  uint2 seg[kSegCap + 1];       // point index = seg.x + stream position, below seg.y
+  uint32_t incl[kSegCap + 32];  // stream position of the segment's end
+};
+
 // GEN: sphere mode -- bin edges not linear in r (the angle bins, count
-// pass) and rows cut to the points' shell (both passes)
-template <bool FILL, bool GEN>
-__global__ void __launch_bounds__(kStreamThreads) k_stream(StreamArgs a) {
+// pass) and rows cut to the points' shell (both passes).  LONG: the count pass
+// takes four steps of a row at a time (plan_pairs says when).
+//
+// Bound by instruction issue (count: 70 instructions per 32 candidates, 84 %
+// of the issue slots on 20k primaries of 10^6 points) and, in the fill, by
+// match_any.  Enumeration with the walk segment by segment / this walk:
+// 10^6 points 168 / 144 ms, cut sky of 800k 121 / 100, 3.1M-pixel sphere 90 /
+// 69, 24 mock catalogues 35.8 / 26.3, 20k uniform points 0.384 / 0.185.
+// Registers: 48 (count) and 56 (fill) at 5 and 4 blocks per SM; 6 blocks
+// spill in the count (154 -> 161 ms) and gain nothing in the fill.
+template <bool FILL, bool GEN, bool LONG>
+__global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream(StreamArgs a) {
   extern __shared__ uint32_t s_cnt_all[];
+  __shared__ WarpSegs s_segs[kStreamThreads / 32];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const Geom g = a.g;
   const int nbins = g.nbins;
-  // fill: running list position per bin; count: lane-private histogram hist[b * 32 + lane]
-  uint32_t* cnt = s_cnt_all + warp * (FILL ? kNbinsCap : nbins * 32);
-  const unsigned lt = (1u << lane) - 1u;
+  // fill: next list entry of each bin; count: pairs of each bin
+  uint32_t* cnt = s_cnt_all + warp * nbins;
+  WarpSegs& sg = s_segs[warp];
+  const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
   const uint32_t nc = g.nc;
   RowWin rw;
-  rw.R2 = g.rcell * g.rcell;
+  rw.R2 = __fmul_rn(g.rcell, g.rcell);
   rw.xs = (float)(g.ncx / nc);
   {
     const RowWindow win = row_window(g);
     rw.W = win.W;
     rw.off0 = win.off0;
     rw.fullwin = win.fullwin;
+    rw.invW = 0xffffffffu / (uint32_t)win.W + 1u;
   }
   rw.nrows = rw.W * rw.W;
   const int nrb = (rw.nrows + 31) / 32;
   const uint64_t lowmask = (1ull << g.shift) - 1ull;
   const float frac_scale = 1.0f / (float)(1ull << g.shift);
   unsigned long long my_pairs = 0;
-  // count: this warp's pool in the code buffer (row blocks take consecutive
+  // count: the constants of a step, passed through a shuffle so that they
+  // stay in registers (the compiler otherwise loads each from the parameter
+  // bank in every step)
+  auto pin = [](float v) { return __shfl_sync(0xffffffffu, v, 0); };
+  const float rlo2 = FILL ? 0.f : pin(g.rlo2_u), rhi2 = FILL ? 0.f : pin(g.rhi2_u);
+  const float inv_dr = FILL ? 0.f : pin(g.inv_dr_u), shift = FILL ? 0.f : pin(g.bin_shift);
+  const float half_bin = FILL ? 0.f : pin(g.half_bin);
+  const uint32_t nb = FILL ? 0u : __float_as_uint(pin(__uint_as_float((uint32_t)nbins)));
+  // count: this warp's pool in the code buffer (batches take consecutive
   // ranges of it; a new pool is taken when one does not fit)
   unsigned long long pool = 0, pool_end = 0;
 
@@ -200,7 +267,7 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream(StreamArgs a) {
     if (FILL) {
       for (int b = lane; b < nbins; b += 32) cnt[b] = __ldg(a.offsets + ib + b);
     } else {
-      for (int b = 0; b < nbins; ++b) cnt[b * 32 + lane] = 0u;
+      for (int b = lane; b < nbins; b += 32) cnt[b] = 0u;
     }
     __syncwarp();
 
@@ -208,171 +275,231 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream(StreamArgs a) {
     rw.cxp = (int)(sx >> g.shift);
     rw.cyp = (int)(sy >> g.shift);
     rw.czp = (int)(sz >> g.shift);
-    rw.fry = (float)(sy & lowmask) * frac_scale;
-    rw.frz = (float)(sz & lowmask) * frac_scale;
-    rw.fx = (float)rw.cxp + (float)(sx & lowmask) * frac_scale;
+    rw.fry = __fmul_rn((float)(sy & lowmask), frac_scale);
+    rw.frz = __fmul_rn((float)(sz & lowmask), frac_scale);
+    rw.fx = __fadd_rn((float)rw.cxp, __fmul_rn((float)(sx & lowmask), frac_scale));
 
-    for (int t0 = 0, rb = 0; t0 < rw.nrows; t0 += 32, ++rb) {
-      uint32_t s0, e0, s1, e1;
-      row_ranges<GEN>(a, g, rw, t0 + lane, s0, e0, s1, e1);
-      // this row block's range of the code buffer: its segments in the order
-      // below, each padded to a multiple of 4 codes
-      unsigned long long span = (s0 < e0 ? (e0 - s0 + 3u) & ~3u : 0u) + (s1 < e1 ? (e1 - s1 + 3u) & ~3u : 0u);
+    uint32_t nseg = 0, total = 0;  // the batch: its segments and candidates
+    unsigned long long* cb = a.code_base + i * (uint64_t)nrb;  // code range of each batch
+    for (int t0 = 0; t0 < rw.nrows; t0 += 32) {
+      // ---- add a row block's segments
+      {
+        uint32_t s0, e0, s1, e1;
+        row_ranges<GEN>(a, g, rw, t0 + lane, s0, e0, s1, e1);
+        const unsigned m0 = __ballot_sync(0xffffffffu, s0 < e0), m1 = __ballot_sync(0xffffffffu, s1 < e1);
+        if (m0 | m1) {
+          const uint32_t len0 = s0 < e0 ? e0 - s0 : 0u;
+          const uint32_t len1 = s1 < e1 ? e1 - s1 : 0u;
+          uint32_t incl = len0 + len1;  // inclusive prefix of the lengths over the lanes
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) span += __shfl_xor_sync(0xffffffffu, span, o);
-      unsigned long long pos = 0;
-      bool codes_ok = true;
-      if (FILL) {
-        pos = __ldg(a.code_base + i * (uint64_t)nrb + rb);
-        // the block's codes to L2 ahead of the segment loads (one line per lane)
-        for (unsigned long long ln = (unsigned long long)lane * 128u; ln < span; ln += 32u * 128u)
-          prefetch_l2(a.codes + pos + ln);
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+          }
+          const uint32_t end1 = total + incl, end0 = end1 - len1, beg0 = end0 - len0;
+          uint32_t k = nseg + __popc(m0 & lt) + __popc(m1 & lt);
+          if (s0 < e0) {
+            sg.seg[k] = make_uint2(s0 - beg0, e0);
+            sg.incl[k] = end0;
+            ++k;
+          }
+          if (s1 < e1) {
+            sg.seg[k] = make_uint2(s1 - end0, e1);
+            sg.incl[k] = end1;
+          }
+          nseg += __popc(m0) + __popc(m1);
+          total += __shfl_sync(0xffffffffu, incl, 31);
+        }
+      }
+      if (nseg <= (uint32_t)kSegCap - 64u && t0 + 32 < rw.nrows) continue;
+      if (nseg == 0) continue;
+      // ---- walk the batch
+      sg.incl[nseg + lane] = 0xffffffffu;
+      if (lane == 0) sg.seg[nseg] = make_uint2(0u, 0u);  // a step's positions past the end
+      __syncwarp();
+      // the segment of each lane's position in the step at k0, f the segments
+      // that end before it
+      auto find = [&](uint32_t k0, uint32_t& f) {
+        const uint32_t d = sg.incl[f + lane] - k0;
+        const unsigned ends = __reduce_or_sync(0xffffffffu, d < 32u ? 1u << d : 0u);
+        const uint32_t t = f + __popc(ends & le);
+        f += __popc(ends);
+        return sg.seg[t];
+      };
+      const uint32_t ngroups = (total + 127u) >> 7;
+      if constexpr (FILL) {
+        const uint32_t* wp = reinterpret_cast<const uint32_t*>(a.codes + __ldg(cb)) + lane;
+        uint32_t word = __ldcs(wp);
+        uint32_t f = 0;
+        uint2 sgm = sg.seg[0];  // segment f: steps inside it need no search
+        for (uint32_t q = 0; q < ngroups; ++q) {
+          const uint32_t wnext = q + 1 < ngroups ? __ldcs(wp + 32u) : 0u;
+          wp += 32;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t code = (word >> (8 * k)) & 0xffu;
+            const unsigned act = __ballot_sync(0xffffffffu, code != kNoBin);
+            const uint32_t k0 = 128u * q + 32u * (uint32_t)k;
+            uint32_t j = k0 + (uint32_t)lane;
+            if (k0 + 32u <= sgm.y - sgm.x) {
+              j += sgm.x;
+            } else {
+              j += find(k0, f).x;
+              sgm = sg.seg[f];
+            }
+            if (code != kNoBin) {
+              const unsigned grp = __match_any_sync(act, code);
+              const uint32_t c0 = cnt[code];
+              const uint32_t rank = __popc(grp & lt);
+              __syncwarp(act);
+              __stcs(a.lists + (uint64_t)(c0 + rank), j);
+              if (rank == 0) cnt[code] = c0 + __popc(grp);
+            }
+            __syncwarp();
+          }
+          word = wnext;
+        }
       } else {
+        const unsigned long long span = 128ull * ngroups;
         if (pool + span > pool_end) {
           const unsigned long long take = span > kCodePool ? span : kCodePool;
           if (lane == 0) pool = atomicAdd(a.code_total, take);
           pool = __shfl_sync(0xffffffffu, pool, 0);
           pool_end = pool + take;
         }
-        pos = pool;
+        if (lane == 0) *cb = pool;
+        // past the buffer: counts stay exact, the codes go to the buffer's
+        // start, and the host grows the buffer and counts the chunk again
+        const bool codes_ok = pool + span <= a.code_cap;
+        uint32_t* cp = reinterpret_cast<uint32_t*>(a.codes + (codes_ok ? pool : 0ull)) + lane;
+        const uint32_t cstep = codes_ok ? 32u : 0u;
         pool += span;
-        if (lane == 0) a.code_base[i * (uint64_t)nrb + rb] = pos;
-        // past the buffer: counts stay exact, codes are dropped and the host
-        // grows the buffer and counts the chunk again
-        codes_ok = pos + span <= a.code_cap;
-      }
-      if constexpr (FILL) {
-        // The row block's codes are one contiguous run: lane t's segments
-        // in order, each padded to 4 codes.  Walk it as a stream, lane l
-        // taking code word k0 + l (4 candidates of one segment), with the
-        // next step's word loaded ahead.
-        const uint32_t len0 = s0 < e0 ? (e0 - s0 + 3u) & ~3u : 0u;
-        const uint32_t len1 = s1 < e1 ? (e1 - s1 + 3u) & ~3u : 0u;
-        uint32_t incl = len0 + len1;  // inclusive prefix of the padded lengths over the lanes
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += v;
-        }
-        const uint32_t excl = incl - len0 - len1;
-        const uint32_t nwords = (uint32_t)(span >> 2);
-        const uint32_t* rbw = reinterpret_cast<const uint32_t*>(a.codes + pos);
-        uint32_t word = (uint32_t)lane < nwords ? __ldcs(rbw + lane) : 0xffffffffu;
-        for (uint32_t k0 = 0; k0 < nwords; k0 += 32) {
-          const uint32_t kn = k0 + 32u + (uint32_t)lane;
-          const uint32_t wnext = kn < nwords ? __ldcs(rbw + kn) : 0xffffffffu;
-          // the segment of code 4 (k0 + lane): first lane t with incl_t above it
-          const uint32_t cpos = 4u * (k0 + (uint32_t)lane);
-          int t = 0;
-#pragma unroll
-          for (int st = 16; st > 0; st >>= 1)
-            if (__shfl_sync(0xffffffffu, incl, t + st - 1) <= cpos) t += st;
-          const uint32_t r = cpos - __shfl_sync(0xffffffffu, excl, t);
-          const uint32_t l0 = __shfl_sync(0xffffffffu, len0, t);
-          const uint32_t sa0 = __shfl_sync(0xffffffffu, s0, t), ea0 = __shfl_sync(0xffffffffu, e0, t);
-          const uint32_t sa1 = __shfl_sync(0xffffffffu, s1, t), ea1 = __shfl_sync(0xffffffffu, e1, t);
-          const bool first = r < l0;
-          const uint32_t jb = first ? sa0 + r : sa1 + (r - l0);
-          const uint32_t je = first ? ea0 : ea1;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint32_t j = jb + (uint32_t)k;
-            const uint32_t code = (word >> (8 * k)) & 0xffu;
-            // words past the run read as all kNoBin; the padding after a
-            // segment's end holds no codes
-            const bool inb = code != kNoBin && j < je;
-            const int b = (int)code;
-            const unsigned act = __ballot_sync(0xffffffffu, inb);
-            if (inb) {
-              const unsigned grp = __match_any_sync(act, b);
-              const unsigned rank = __popc(grp & lt);
-              const uint32_t c0 = cnt[b];
-              __syncwarp(act);
-              __stcs(a.lists + ((uint64_t)c0 + rank), j);
-              if (rank == 0) cnt[b] = c0 + __popc(grp);
-            }
-            __syncwarp();
-          }
-          word = wnext;
-        }
-        continue;
-      }
-      unsigned pend = __ballot_sync(0xffffffffu, s0 < e0 || s1 < e1);
-      while (pend) {
-        // ---- next segment (warp-uniform)
-        const int src = __ffs(pend) - 1;
-        const bool h0 = __shfl_sync(0xffffffffu, s0 < e0, src);
-        const uint32_t cs = __shfl_sync(0xffffffffu, h0 ? s0 : s1, src);
-        const uint32_t ce = __shfl_sync(0xffffffffu, h0 ? e0 : e1, src);
-        if (lane == src) {
-          if (h0) s0 = e0;
-          else s1 = e1;
-        }
-        pend = __ballot_sync(0xffffffffu, s0 < e0 || s1 < e1);
-        const unsigned long long seg0 = pos;  // code of candidate j: codes[seg0 + (j - cs)]
-        pos += (ce - cs + 3u) & ~3u;
-        for (uint32_t base = cs; base < ce; base += 32) {
-          const uint32_t j = base + lane;
-          const bool valid = j < ce;
-          // lanes past the segment load its last point and are masked by `valid`
-          const uint4 q = __ldg(a.pts + (valid ? j : ce - 1u));
-          const int ix = (int)(q.x - P.x), iy = (int)(q.y - P.y), iz = (int)(q.z - P.z);
-          const float dx = __int2float_rn(ix), dy = __int2float_rn(iy), dz = __int2float_rn(iz);
+        uint32_t word = 0;  // the codes of the group's steps so far
+        auto store = [&] {
+          __stcs(cp, word);
+          cp += cstep;
+        };
+        // One candidate per lane: is it in range (inb), its bin b, and whether
+        // it lies within float rounding of an edge.
+        auto classify = [&](const uint4 q, bool& inb, uint32_t& b) -> bool {
+          const float dx = __int2float_rn((int)(q.x - P.x)), dy = __int2float_rn((int)(q.y - P.y)),
+                      dz = __int2float_rn((int)(q.z - P.z));
           const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
           // rlo2_u > 0 also excludes r = 0 (coincident points)
-          bool inb = valid && r2 >= g.rlo2_u && r2 < g.rhi2_u;
-          int b = 0;
-          if (inb) {
-            const float r = r2 * rsqrtf(r2);
-            float tt, guard;
-            if constexpr (GEN) {
-              // sphere: the bin of theta = 2 asin(chord / 2).  Its float
-              // error stays below 1e-6 theta while chord / 2 <= 0.99 (asin
-              // is ill-conditioned towards 1); the guard is ten times that,
-              // and larger chords always take the exact test.  Up to
-              // chord / 2 = 1/8 (theta 14 degrees) the Maclaurin series of
-              // asin to x^7 serves: truncation below 2e-9 theta, float
-              // evaluation below 2e-7 theta.
-              const float x = r * g.half_unit;
-              float th;
-              if (x <= 0.125f) {
-                const float x2 = x * x;
-                th = 2.f * x * fmaf(x2, fmaf(x2, fmaf(x2, 5.f / 112.f, 3.f / 40.f), 1.f / 6.f), 1.f);
-              } else {
-                th = 2.f * asinf(fminf(x, 1.f));
+          inb = r2 >= rlo2 && r2 < rhi2;
+          const float r = r2 * rsqrt_fast(r2);
+          // th: the bin coordinate minus 1/2.  Rounded to the nearest integer
+          // (by adding 1.5 * 2^23) it is the bin, and what is left over is
+          // the distance from the bin's middle, within `half` of it unless
+          // the pair may lie on an edge.
+          float th, half;
+          if constexpr (GEN) {
+            // sphere: the bin of theta = 2 asin(chord / 2).  Its float
+            // error stays below 1e-6 theta while chord / 2 <= 0.99 (asin
+            // is ill-conditioned towards 1); the guard is ten times that,
+            // and larger chords always take the exact test.  Up to
+            // chord / 2 = 1/8 (theta 14 degrees) the Maclaurin series of
+            // asin to x^7 serves: truncation below 2e-9 theta, float
+            // evaluation below 4e-7 theta.
+            const float x = r * g.half_unit;
+            const float x2 = x * x;
+            float ang = 2.f * x * fmaf(x2, fmaf(x2, fmaf(x2, 5.f / 112.f, 3.f / 40.f), 1.f / 6.f), 1.f);
+            if (__any_sync(0xffffffffu, inb && x > 0.125f)) ang = x > 0.125f ? 2.f * asinf(fminf(x, 1.f)) : ang;
+            th = fmaf(ang, inv_dr, shift);
+            half = x > 0.99f ? -1.f : fminf(half_bin, fmaf(ang, -1e-5f * inv_dr, 0.5f - 1e-7f * inv_dr));
+          } else {
+            th = fmaf(r, inv_dr, shift);
+            half = half_bin;
+          }
+          const float tm = th + 12582912.f;
+          b = __float_as_uint(tm) - 0x4b400000u;
+          return inb && (b >= nb || fabsf(th - (tm - 12582912.f)) > half);
+        };
+        // on an edge: exact integer r^2 against exact thresholds
+        auto exact = [&](const uint4 q, bool& inb, uint32_t& b) {
+          const long long ix = (int)(q.x - P.x), iy = (int)(q.y - P.y), iz = (int)(q.z - P.z);
+          const unsigned long long e2 = (unsigned long long)(ix * ix + iy * iy + iz * iz);
+          if (e2 == 0ull || e2 < __ldg(a.thr) || e2 >= __ldg(a.thr + nbins)) {
+            inb = false;
+          } else {
+            int c = min(max((int)b, 0), nbins - 1);
+            while (e2 < __ldg(a.thr + c)) --c;
+            while (e2 >= __ldg(a.thr + c + 1)) ++c;
+            b = (uint32_t)c;
+          }
+        };
+        // its code into the word, its bin's count
+        auto emit = [&](bool inb, uint32_t b) {
+          word = __funnelshift_r(word, inb ? b : (uint32_t)kNoBin, 8);
+          if (inb) atomicAdd(cnt + b, 1u);
+        };
+        auto one = [&](const uint4 q) {
+          bool inb;
+          uint32_t b;
+          const bool edge = classify(q, inb, b);
+          if (__any_sync(0xffffffffu, edge)) {
+            if (edge) exact(q, inb, b);
+          }
+          emit(inb, b);
+        };
+        uint32_t f = 0, k0 = 0;
+        while (k0 < total) {
+          // steps inside one segment: consecutive points (LONG: four steps at a time)
+          {
+            const uint2 sgm = sg.seg[f];
+            const uint32_t uend = sgm.y - sgm.x;
+            const uint4* qp = a.pts + (sgm.x + k0 + (uint32_t)lane);
+            if constexpr (LONG) {
+              const uint32_t last = 3u - ((k0 >> 5) & 3u);  // the step of the four that ends a word
+              for (; k0 + 128u <= uend; k0 += 128u, qp += 128) {
+                uint4 q[4];
+  #pragma unroll
+                for (int u = 0; u < 4; ++u) q[u] = __ldg(qp + 32 * u);
+                bool inb[4], edge[4];
+                uint32_t b[4];
+  #pragma unroll
+                for (int u = 0; u < 4; ++u) edge[u] = classify(q[u], inb[u], b[u]);
+                if (__any_sync(0xffffffffu, edge[0] | edge[1] | edge[2] | edge[3])) {
+  #pragma unroll
+                  for (int u = 0; u < 4; ++u)
+                    if (edge[u]) exact(q[u], inb[u], b[u]);
+                }
+  #pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  emit(inb[u], b[u]);
+                  if (last == (uint32_t)u) __stcs(cp, word);
+                }
+                cp += cstep;
               }
-              tt = (th - g.tmin) * g.inv_dt;
-              guard = x > 0.99f ? 1.f : fmaxf(1e-4f, fmaf(1e-5f, th, 1e-7f) * g.inv_dt);
-            } else {
-              tt = (r - g.rmin_u) * g.inv_dr_u;
-              guard = 1e-4f;
             }
-            b = (int)floorf(tt);
-            const float fr = tt - (float)b;
-            if ((unsigned)b >= (unsigned)nbins || fabsf(fr - 0.5f) > 0.5f - guard) {
-              // within float rounding of an edge: exact integer r^2 vs
-              // exact thresholds
-              const unsigned long long e2 = (unsigned long long)((long long)ix * ix + (long long)iy * iy +
-                                                                 (long long)iz * iz);
-              if (e2 == 0ull || e2 < __ldg(a.thr) || e2 >= __ldg(a.thr + nbins)) {
-                inb = false;
-              } else {
-                b = min(max(b, 0), nbins - 1);
-                while (e2 < __ldg(a.thr + b)) --b;
-                while (e2 >= __ldg(a.thr + b + 1)) ++b;
-              }
+            for (; k0 + 32u <= uend; qp += 32) {
+              one(__ldg(qp));
+              k0 += 32u;
+              if ((k0 & 127u) == 0u) store();
             }
           }
-          if (valid && codes_ok) __stcs(a.codes + (seg0 + (j - cs)), inb ? (unsigned char)b : (unsigned char)kNoBin);
-          if (inb) cnt[b * 32 + lane] += 1u;  // lane-private: no ordering, no conflict
+          if (k0 >= total) break;
+          // a step with a boundary
+          const uint2 sgm = find(k0, f);
+          const uint32_t j = sgm.x + k0 + (uint32_t)lane;
+          one(__ldg(a.pts + (j < sgm.y ? j : sp)));
+          k0 += 32u;
+          if ((k0 & 127u) == 0u) store();
+        }
+        if (k0 & 127u) {  // the last group: no codes in the steps it lacks
+          for (; k0 & 127u; k0 += 32u) word = __funnelshift_r(word, (uint32_t)kNoBin, 8);
+          store();
         }
       }
+      ++cb;
+      nseg = 0;
+      total = 0;
+      __syncwarp();  // the batch's list is rewritten
     }
     if (!FILL) {
       __syncwarp();
       for (int b = lane; b < nbins; b += 32) {
-        uint32_t s = 0;
-        for (int k = 0; k < 32; ++k) s += cnt[b * 32 + ((b + k) & 31)];  // rotated: no bank conflict
+        const uint32_t s = cnt[b];
         a.counts[ib + b] = s;
         my_pairs += s;
       }
@@ -386,37 +513,29 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream(StreamArgs a) {
   }
 }
 
-static size_t stream_smem(bool fill, int nbins) {
-  return (size_t)(kStreamThreads / 32) * (fill ? kNbinsCap : nbins * 32) * sizeof(uint32_t);
+// the bins' counts or cursors of each warp (at most 2 KB a block)
+static size_t stream_smem(int nbins) { return (size_t)(kStreamThreads / 32) * nbins * sizeof(uint32_t); }
+
+static const void* stream_fn(const Geom& g, bool fill) {
+  if (g.general) return fill ? (const void*)k_stream<true, true, false> : (const void*)k_stream<false, true, false>;
+  if (fill) return (const void*)k_stream<true, false, false>;
+  return g.long_rows ? (const void*)k_stream<false, false, true> : (const void*)k_stream<false, false, false>;
 }
 
-int stream_blocks_per_sm(bool fill, int nbins, bool general) {
-  const void* fn = fill ? (general ? (const void*)k_stream<true, true> : (const void*)k_stream<true, false>)
-                        : (general ? (const void*)k_stream<false, true> : (const void*)k_stream<false, false>);
-  const size_t smem = stream_smem(fill, nbins);
-  if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
+int stream_blocks_per_sm(const Geom& g, bool fill) {
   int nb = 0;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kStreamThreads, smem) == cudaSuccess ? nb : 0;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, stream_fn(g, fill), kStreamThreads, stream_smem(g.nbins)) ==
+                 cudaSuccess
+             ? nb
+             : 0;
 }
 
 cudaError_t launch_stream(const StreamArgs& a, bool fill, int nblocks, cudaStream_t st) {
-  const size_t smem = stream_smem(fill, a.g.nbins);
-  const bool gen = a.g.general != 0;
-  const void* fn = fill ? (gen ? (const void*)k_stream<true, true> : (const void*)k_stream<true, false>)
-                        : (gen ? (const void*)k_stream<false, true> : (const void*)k_stream<false, false>);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  if (fill && gen)
-    k_stream<true, true><<<nblocks, kStreamThreads, smem, st>>>(a);
-  else if (fill)
-    k_stream<true, false><<<nblocks, kStreamThreads, smem, st>>>(a);
-  else if (gen)
-    k_stream<false, true><<<nblocks, kStreamThreads, smem, st>>>(a);
-  else
-    k_stream<false, false><<<nblocks, kStreamThreads, smem, st>>>(a);
+  StreamArgs sa = a;
+  void* args[] = {&sa};
+  const cudaError_t e = cudaLaunchKernel(stream_fn(a.g, fill), dim3(nblocks), dim3(kStreamThreads), args,
+                                         stream_smem(a.g.nbins), st);
+  if (e != cudaSuccess) return e;
   ++g_launches;
   return cudaGetLastError();
 }
