@@ -602,8 +602,10 @@ int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   // chunks follow the measured pairs per primary
   const double est = 2.0 * mean_neighbours(c) + 64.0;
   // candidates (points of the scanned cell rows) run about 1.3-1.5x the pairs
-  pl->code_cap = std::min<uint64_t>(kCodeCap, 4 * pl->list_cap);
-  pl->cand_first = 1.5 * est;
+  // (a small list capacity bounds the codes too, a primary's batch heads and one pool aside)
+  pl->code_cap = std::min<uint64_t>(kCodeCap, 4 * pl->list_cap + 1024ull * row_blocks(c->g) + kStreamCodePool);
+  // and a batch's head and segments up to 8 bytes a point or row, whichever is fewer
+  pl->cand_first = 1.5 * est + 8.0 * std::min(1.5 * est, 32.0 * row_blocks(c->g)) + 256.0;
   const double first = std::min(0.9 * (double)pl->list_cap / est, 0.9 * (double)pl->code_cap / pl->cand_first);
   pl->chunk_first = std::max<int64_t>(1, std::min<int64_t>(pl->chunk_max, (int64_t)first));
   return CTB_OK;
@@ -724,7 +726,9 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   double t_stream = 0, t_alm = 0, t_con = 0, t_pack = 0;
   uint64_t pairs = 0, chunks = 0;
   int64_t C = pl.chunk_first;
-  double cand_per = pl.cand_first;  // candidates per primary (estimate, then measured)
+  double cand_per = pl.cand_first;  // code bytes per primary (estimate, then measured)
+  // every warp of the count pass may hold a pool it does not fill
+  const double pools = 256.0 + (double)std::min<int64_t>((int64_t)pl.count_blocks * (kStreamThreads / 32), np) * kStreamCodePool;
   size_t codes_need = 0;            // bytes the last count of this chunk asked for
   int64_t c0 = 0;
   // [0] count start [1] count end [2] fill end [3] alm end [4] contraction end [5] pack end
@@ -735,7 +739,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     sa.prim_count = aa.prim_count = cnt;
     // bin codes of this chunk: the estimate, or what its last count asked for
     const size_t codes_want = std::max<size_t>(
-        codes_need, (size_t)std::min<double>((double)pl.code_cap, 1.05 * cand_per * (double)cnt + 256.0));
+        codes_need, (size_t)std::min<double>((double)pl.code_cap, 1.05 * cand_per * (double)cnt + pools));
     CK(c, ensure(c, c->codes, codes_want));
     sa.codes = P<uint8_t>(c->codes);
     sa.code_cap = c->codes.bytes;

@@ -311,12 +311,13 @@ struct StreamArgs {
   uint8_t* codes;                 // bin code per candidate (written: count, read: fill)
   unsigned long long code_cap;    // bytes of codes
   unsigned long long* code_total; // code bytes of this launch (count pass; the range allocator)
-  unsigned long long* code_base;  // [prim_count][row_blocks] start of each batch's codes (at most one a row block)
+  unsigned long long* code_base;  // [prim_count][row_blocks] start of each batch (at most one a row block; ~0 ends them)
   Geom g;
 };
 int stream_blocks_per_sm(const Geom& g, bool fill);
 cudaError_t launch_stream(const StreamArgs& a, bool fill, int nblocks, cudaStream_t st);
 constexpr int kStreamThreads = 256;
+constexpr int kStreamCodePool = 16384;  // bytes of the code buffer a warp of the count pass takes at a time
 
 // pair.cuh -- harmonic accumulation over the (primary, bin) lists
 struct AlmArgs {

@@ -15,10 +15,10 @@
 //   count: pairs per (primary, bin)  -> counts (then an exclusive scan on the
 //          host stream gives each (primary, bin) list its start); the bin of
 //          every candidate is also stored as one byte (kNoBin: not a pair)
-//   fill:  walks the same candidate stream, reads the stored bin codes four
-//          per lane (no point loads, no distances) and writes each pair's
-//          neighbour index into its (primary, bin) list (match_any ranks the
-//          lanes that share a bin)
+//   fill:  walks the same candidate stream, from the segments and bin codes
+//          that the count pass stored (no cell rows, points or distances), and
+//          writes each pair's neighbour index into its (primary, bin) list
+//          (match_any ranks the lanes that share a bin)
 //
 // The candidate stream.  A row's point ranges (segments) are short where the
 // catalogue is sparse or the points lie on a surface: 0.4 points a row in a
@@ -41,6 +41,10 @@
 // An idle lane of the count pass looks at the primary itself (r = 0, never a
 // pair), and the codes past the stream's end read kNoBin, so neither pass
 // tests positions.
+//
+// A batch in the code buffer: a 16-byte head (segments, candidates), its
+// segments (point offset, end position: 8 bytes each, padded to 16), its
+// codes.
 #include <algorithm>
 
 #include "ctb_internal.cuh"
@@ -70,7 +74,8 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 }
 
 constexpr uint8_t kNoBin = 0xff;  // bin code of a candidate that is not a pair
-constexpr unsigned long long kCodePool = 16384;  // code bytes a warp takes at a time
+constexpr unsigned long long kCodePool = (unsigned long long)kStreamCodePool;  // code bytes a warp takes at a time
+constexpr unsigned long long kNoBatch = ~0ull;  // ends a primary's batches
 
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
@@ -87,11 +92,6 @@ struct RowWin {
   uint32_t cbase;
 };
 
-// The count and the fill pass have to see the same ranges to the bit, so every
-// product that the compiler could fuse with a sum is written out (__fmul_rn,
-// __fmaf_rn): the two instantiations fused differently, and a row's end moved
-// by an x-cell in one of them.
-//
 // The point ranges of row t of the window (up to two: periodic wrap in x,
 // or the two crossings of the sphere's shell); empty ranges have s >= e.
 // SHELL (sphere mode): every point lies in the shell of g.shell_r2lo ..
@@ -201,27 +201,40 @@ struct WarpSegs {
   uint32_t incl[kSegCap + 32];  // stream position of the segment's end
 };
 
-// GEN: sphere mode -- bin edges not linear in r (the angle bins, count
-// pass) and rows cut to the points' shell (both passes).  LONG: the count pass
-// takes four steps of a row at a time (plan_pairs says when).
+__device__ __forceinline__ uint32_t batch_head(uint32_t nseg) { return (16u + 8u * nseg + 15u) & ~15u; }
+
+// Segment of this lane's position in the step at k0; f: the segments that end
+// before the step, moved past those that end in it.
+__device__ __forceinline__ uint32_t find_segment(const WarpSegs& sg, uint32_t k0, uint32_t& f, int lane, unsigned le) {
+  const uint32_t d = sg.incl[f + lane] - k0;
+  const unsigned ends = __reduce_or_sync(0xffffffffu, d < 32u ? 1u << d : 0u);
+  const uint32_t t = f + __popc(ends & le);
+  f += __popc(ends);
+  return t;
+}
+
+// Count pass.  GEN: sphere mode -- bin edges not linear in r (the angle bins)
+// and rows cut to the points' shell.  LONG: four steps of a row at a time
+// (plan_pairs says when).
 //
 // Bound by instruction issue (count: 70 instructions per 32 candidates, 84 %
 // of the issue slots on 20k primaries of 10^6 points) and, in the fill, by
-// match_any.  Enumeration with the walk segment by segment / this walk:
-// 10^6 points 168 / 144 ms, cut sky of 800k 121 / 100, 3.1M-pixel sphere 90 /
-// 69, 24 mock catalogues 35.8 / 26.3, 20k uniform points 0.384 / 0.185.
-// Registers: 48 (count) and 56 (fill) at 5 and 4 blocks per SM; 6 blocks
-// spill in the count (154 -> 161 ms) and gain nothing in the fill.
-template <bool FILL, bool GEN, bool LONG>
-__global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream(StreamArgs a) {
+// match_any.  Enumeration with the walk segment by segment / with this one:
+// 10^6 points 168 / 144 ms, cut sky of 800k 121 / 102, 3.1M-pixel sphere 90 /
+// 63, 24 mock catalogues 35.8 / 23.7, 20k uniform points 0.384 / 0.142.  The
+// last of these numbers with the fill finding the rows again, as the count
+// does: 144, 100, 69, 26.3, 0.185.  Four blocks of 8 warps per SM (64
+// registers): five spill in the count (sphere 67 ms) and cost the fill its
+// look-ahead (cut sky 106 ms).
+template <bool GEN, bool LONG>
+__global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
   extern __shared__ uint32_t s_cnt_all[];
   __shared__ WarpSegs s_segs[kStreamThreads / 32];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const Geom g = a.g;
   const int nbins = g.nbins;
-  // fill: next list entry of each bin; count: pairs of each bin
-  uint32_t* cnt = s_cnt_all + warp * nbins;
+  uint32_t* cnt = s_cnt_all + warp * nbins;  // pairs of each bin
   WarpSegs& sg = s_segs[warp];
   const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
   const uint32_t nc = g.nc;
@@ -240,15 +253,15 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
   const uint64_t lowmask = (1ull << g.shift) - 1ull;
   const float frac_scale = 1.0f / (float)(1ull << g.shift);
   unsigned long long my_pairs = 0;
-  // count: the constants of a step, passed through a shuffle so that they
+  // the constants of a step, passed through a shuffle so that they
   // stay in registers (the compiler otherwise loads each from the parameter
   // bank in every step)
   auto pin = [](float v) { return __shfl_sync(0xffffffffu, v, 0); };
-  const float rlo2 = FILL ? 0.f : pin(g.rlo2_u), rhi2 = FILL ? 0.f : pin(g.rhi2_u);
-  const float inv_dr = FILL ? 0.f : pin(g.inv_dr_u), shift = FILL ? 0.f : pin(g.bin_shift);
-  const float half_bin = FILL ? 0.f : pin(g.half_bin);
-  const uint32_t nb = FILL ? 0u : __float_as_uint(pin(__uint_as_float((uint32_t)nbins)));
-  // count: this warp's pool in the code buffer (batches take consecutive
+  const float rlo2 = pin(g.rlo2_u), rhi2 = pin(g.rhi2_u);
+  const float inv_dr = pin(g.inv_dr_u), shift = pin(g.bin_shift);
+  const float half_bin = pin(g.half_bin);
+  const uint32_t nb = __float_as_uint(pin(__uint_as_float((uint32_t)nbins)));
+  // this warp's pool in the code buffer (batches take consecutive
   // ranges of it; a new pool is taken when one does not fit)
   unsigned long long pool = 0, pool_end = 0;
 
@@ -262,13 +275,9 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
     const uint4 P = __ldg(a.pts + sp);
     // batch: the primary's catalogue owns cells [cat * ncells, (cat + 1) * ncells)
     rw.cbase = a.keys ? (__ldg(a.keys + sp) / g.ncells) * g.ncells : 0u;
-    if (!FILL && lane == 0) a.wprim[i] = a.wsub ? __ldg(a.wsub + gi) : __uint_as_float(P.w);
+    if (lane == 0) a.wprim[i] = a.wsub ? __ldg(a.wsub + gi) : __uint_as_float(P.w);
     const uint64_t ib = i * (uint64_t)nbins;
-    if (FILL) {
-      for (int b = lane; b < nbins; b += 32) cnt[b] = __ldg(a.offsets + ib + b);
-    } else {
-      for (int b = lane; b < nbins; b += 32) cnt[b] = 0u;
-    }
+    for (int b = lane; b < nbins; b += 32) cnt[b] = 0u;
     __syncwarp();
 
     const uint64_t sx = (uint64_t)P.x * g.ncx, sy = (uint64_t)P.y * nc, sz = (uint64_t)P.z * nc;
@@ -280,7 +289,7 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
     rw.fx = __fadd_rn((float)rw.cxp, __fmul_rn((float)(sx & lowmask), frac_scale));
 
     uint32_t nseg = 0, total = 0;  // the batch: its segments and candidates
-    unsigned long long* cb = a.code_base + i * (uint64_t)nrb;  // code range of each batch
+    unsigned long long* cb = a.code_base + i * (uint64_t)nrb;  // start of each batch, ended by kNoBatch
     for (int t0 = 0; t0 < rw.nrows; t0 += 32) {
       // ---- add a row block's segments
       {
@@ -317,50 +326,10 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
       sg.incl[nseg + lane] = 0xffffffffu;
       if (lane == 0) sg.seg[nseg] = make_uint2(0u, 0u);  // a step's positions past the end
       __syncwarp();
-      // the segment of each lane's position in the step at k0, f the segments
-      // that end before it
-      auto find = [&](uint32_t k0, uint32_t& f) {
-        const uint32_t d = sg.incl[f + lane] - k0;
-        const unsigned ends = __reduce_or_sync(0xffffffffu, d < 32u ? 1u << d : 0u);
-        const uint32_t t = f + __popc(ends & le);
-        f += __popc(ends);
-        return sg.seg[t];
-      };
       const uint32_t ngroups = (total + 127u) >> 7;
-      if constexpr (FILL) {
-        const uint32_t* wp = reinterpret_cast<const uint32_t*>(a.codes + __ldg(cb)) + lane;
-        uint32_t word = __ldcs(wp);
-        uint32_t f = 0;
-        uint2 sgm = sg.seg[0];  // segment f: steps inside it need no search
-        for (uint32_t q = 0; q < ngroups; ++q) {
-          const uint32_t wnext = q + 1 < ngroups ? __ldcs(wp + 32u) : 0u;
-          wp += 32;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint32_t code = (word >> (8 * k)) & 0xffu;
-            const unsigned act = __ballot_sync(0xffffffffu, code != kNoBin);
-            const uint32_t k0 = 128u * q + 32u * (uint32_t)k;
-            uint32_t j = k0 + (uint32_t)lane;
-            if (k0 + 32u <= sgm.y - sgm.x) {
-              j += sgm.x;
-            } else {
-              j += find(k0, f).x;
-              sgm = sg.seg[f];
-            }
-            if (code != kNoBin) {
-              const unsigned grp = __match_any_sync(act, code);
-              const uint32_t c0 = cnt[code];
-              const uint32_t rank = __popc(grp & lt);
-              __syncwarp(act);
-              __stcs(a.lists + (uint64_t)(c0 + rank), j);
-              if (rank == 0) cnt[code] = c0 + __popc(grp);
-            }
-            __syncwarp();
-          }
-          word = wnext;
-        }
-      } else {
-        const unsigned long long span = 128ull * ngroups;
+      {
+        const uint32_t head = batch_head(nseg);
+        const unsigned long long span = head + 128ull * ngroups;
         if (pool + span > pool_end) {
           const unsigned long long take = span > kCodePool ? span : kCodePool;
           if (lane == 0) pool = atomicAdd(a.code_total, take);
@@ -371,7 +340,12 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
         // past the buffer: counts stay exact, the codes go to the buffer's
         // start, and the host grows the buffer and counts the chunk again
         const bool codes_ok = pool + span <= a.code_cap;
-        uint32_t* cp = reinterpret_cast<uint32_t*>(a.codes + (codes_ok ? pool : 0ull)) + lane;
+        if (codes_ok) {
+          uint2* hp = reinterpret_cast<uint2*>(a.codes + pool);
+          if (lane == 0) *hp = make_uint2(nseg, total);
+          for (uint32_t k = lane; k < nseg; k += 32) hp[2 + k] = make_uint2(sg.seg[k].x, sg.incl[k]);
+        }
+        uint32_t* cp = reinterpret_cast<uint32_t*>(a.codes + (codes_ok ? pool + head : 0ull)) + lane;
         const uint32_t cstep = codes_ok ? 32u : 0u;
         pool += span;
         uint32_t word = 0;  // the codes of the group's steps so far
@@ -480,7 +454,7 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
           }
           if (k0 >= total) break;
           // a step with a boundary
-          const uint2 sgm = find(k0, f);
+          const uint2 sgm = sg.seg[find_segment(sg, k0, f, lane, le)];
           const uint32_t j = sgm.x + k0 + (uint32_t)lane;
           one(__ldg(a.pts + (j < sgm.y ? j : sp)));
           k0 += 32u;
@@ -496,20 +470,88 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
       total = 0;
       __syncwarp();  // the batch's list is rewritten
     }
-    if (!FILL) {
-      __syncwarp();
-      for (int b = lane; b < nbins; b += 32) {
-        const uint32_t s = cnt[b];
-        a.counts[ib + b] = s;
-        my_pairs += s;
-      }
+    if (lane == 0 && cb < a.code_base + (i + 1) * (uint64_t)nrb) *cb = kNoBatch;
+    __syncwarp();
+    for (int b = lane; b < nbins; b += 32) {
+      const uint32_t s = cnt[b];
+      a.counts[ib + b] = s;
+      my_pairs += s;
     }
     __syncwarp();
   }
-  if (!FILL) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) my_pairs += __shfl_xor_sync(0xffffffffu, my_pairs, o);
-    if (lane == 0 && my_pairs) atomicAdd(a.total, my_pairs);
+  for (int o = 16; o > 0; o >>= 1) my_pairs += __shfl_xor_sync(0xffffffffu, my_pairs, o);
+  if (lane == 0 && my_pairs) atomicAdd(a.total, my_pairs);
+}
+
+// Fill pass.
+__global__ void __launch_bounds__(kStreamThreads, 4) k_fill(StreamArgs a) {
+  extern __shared__ uint32_t s_cnt_all[];
+  __shared__ WarpSegs s_segs[kStreamThreads / 32];
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int nbins = a.g.nbins;
+  uint32_t* cnt = s_cnt_all + warp * nbins;  // next list entry of each bin
+  WarpSegs& sg = s_segs[warp];
+  const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
+  const int nrb = row_blocks(a.g);
+  while (true) {
+    unsigned long long i = 0;
+    if (lane == 0) i = atomicAdd(a.work, 1ull);
+    i = __shfl_sync(0xffffffffu, i, 0);
+    if (i >= (unsigned long long)a.prim_count) break;
+    for (int b = lane; b < nbins; b += 32) cnt[b] = __ldg(a.offsets + i * (uint64_t)nbins + b);
+    const unsigned long long* cb = a.code_base + i * (uint64_t)nrb;
+    unsigned long long next = __ldg(cb);
+    for (int ib = 0; ib < nrb; ++ib) {
+      const unsigned long long pos = next;
+      if (pos == kNoBatch) break;
+      if (ib + 1 < nrb) next = __ldg(cb + ib + 1);
+      const uint2* hp = reinterpret_cast<const uint2*>(a.codes + pos);
+      const uint2 hd = __ldg(hp);
+      const uint32_t nseg = hd.x, ngroups = (hd.y + 127u) >> 7;
+      const uint32_t* wp = reinterpret_cast<const uint32_t*>(a.codes + pos + batch_head(nseg)) + lane;
+      uint32_t word = __ldcs(wp);
+      for (uint32_t k = lane; k < nseg; k += 32) {
+        const uint2 v = __ldcs(hp + 2 + k);
+        sg.seg[k].x = v.x;
+        sg.incl[k] = v.y;
+      }
+      sg.incl[nseg + lane] = 0xffffffffu;
+      if (lane == 0) sg.seg[nseg].x = 0u;
+      __syncwarp();
+      uint32_t f = 0;
+      uint32_t sx = sg.seg[0].x, send = sg.incl[0];  // segment f: steps inside it need no search
+      for (uint32_t q = 0; q < ngroups; ++q) {
+        const uint32_t wnext = q + 1 < ngroups ? __ldcs(wp + 32u) : 0u;
+        wp += 32;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t code = (word >> (8 * k)) & 0xffu;
+          const unsigned act = __ballot_sync(0xffffffffu, code != kNoBin);
+          const uint32_t k0 = 128u * q + 32u * (uint32_t)k;
+          uint32_t j = k0 + (uint32_t)lane;
+          if (k0 + 32u <= send) {
+            j += sx;
+          } else {
+            j += sg.seg[find_segment(sg, k0, f, lane, le)].x;
+            sx = sg.seg[f].x;
+            send = f < nseg ? sg.incl[f] : 0u;
+          }
+          if (code != kNoBin) {
+            const unsigned grp = __match_any_sync(act, code);
+            const uint32_t c0 = cnt[code];
+            const uint32_t rank = __popc(grp & lt);
+            __syncwarp(act);
+            __stcs(a.lists + (uint64_t)(c0 + rank), j);
+            if (rank == 0) cnt[code] = c0 + __popc(grp);
+          }
+          __syncwarp();
+        }
+        word = wnext;
+      }
+    }
+    __syncwarp();  // the cursors are rewritten
   }
 }
 
@@ -517,9 +559,9 @@ __global__ void __launch_bounds__(kStreamThreads, FILL || LONG ? 4 : 5) k_stream
 static size_t stream_smem(int nbins) { return (size_t)(kStreamThreads / 32) * nbins * sizeof(uint32_t); }
 
 static const void* stream_fn(const Geom& g, bool fill) {
-  if (g.general) return fill ? (const void*)k_stream<true, true, false> : (const void*)k_stream<false, true, false>;
-  if (fill) return (const void*)k_stream<true, false, false>;
-  return g.long_rows ? (const void*)k_stream<false, false, true> : (const void*)k_stream<false, false, false>;
+  if (fill) return (const void*)k_fill;
+  if (g.general) return (const void*)k_count<true, false>;
+  return g.long_rows ? (const void*)k_count<false, true> : (const void*)k_count<false, false>;
 }
 
 int stream_blocks_per_sm(const Geom& g, bool fill) {
