@@ -19,10 +19,13 @@ namespace ctb {
 // The sum over m within a multipole is left to the end, where the slots of
 // each l are added in a fixed order.
 //
-// What bounds it: the paired FMAs (2.65 issue cycles each, measured) at 20 to
-// 64 bins, HBM for fewer.  A 10 x 10 tile does 50 of them on 20 loads; tiles
-// of 4 x 4 with 16-byte loads of transposed rows, the form before this one,
-// spent most of their time on shared-memory loads and on the transposition.
+// What bounds it: the issue of paired FMAs and their operands at three warps
+// a scheduler (FMA pipe 41 %, HBM 52 % on 200k rows of 20 bins, l_max 10:
+// 546 us).  The form before this one, 4 x 4 tiles by 16-byte loads of
+// transposed rows, spent its time on shared-memory loads and, for the
+// 121-float rows of a caller, on transposing them element by element (20k
+// such rows: 640 us; now 72).  Half tiles of 5 x 10 with twice the warps were
+// slower (667 us): more loads and address arithmetic per FMA.
 //
 // Block: CH slots x tiles x PG primary groups (group g takes the stage's
 // primaries q = g mod PG).  Rows of more than CH slots are taken in chunks of
@@ -33,15 +36,15 @@ namespace ctb {
 // deterministic.
 //
 // Copies (16 bytes each where the rows allow it): rows that fit one chunk are
-// copied as they lie, one contiguous run per stage, and read at the row's own
-// stride (kConLinear: 121-float rows then cost no more than padded ones);
+// copied as they lie, one contiguous run per stage (kConLinear; kConLinearAny
+// reads at the row's own stride where that is not CH, as for 121-float rows);
 // chunks of longer rows are copied row by row (kConRows16, kConRows4).
 constexpr int kConFlush = 1024;         // primaries of a group between two flushes
 constexpr int kConMaxQ = 64;            // primaries per stage at most
 constexpr int kConStageFloats = 11264;  // one staged buffer at most, when more than PG primaries fit it
 constexpr int kConStages = 3;
 constexpr int kConMaxTiles = 24;        // tiles per block at most (768 threads / 32)
-enum { kConRows4 = 0, kConRows16 = 1, kConLinear = 2 };
+enum { kConRows4 = 0, kConRows16 = 1, kConLinear = 2, kConLinearAny = 3 };
 constexpr size_t kConSmemCap = 220 * 1024;
 
 struct ConShape {
@@ -104,7 +107,7 @@ static ConShape con_shape(int nbins, int row) {
   // their end: slots and bins that nothing owns
   c.stage_floats = c.Q * nbins * c.stride + (nbins < c.T ? (c.T - nbins) * c.stride : 0) + c.ch;
   c.stage_floats = (c.stage_floats + 3) & ~3;
-  const int red = c.threads * c.T;  // the flush buffer aliases the stages
+  const int red = c.threads * c.T * c.T;  // the flush buffer aliases the stages (154 KB at most)
   c.stages = kConStages;
   while (c.stages > 1 && (size_t)(c.stages * (c.stage_floats + kConMaxQ)) * 4 + 4096 > kConSmemCap) --c.stages;
   const int body = c.stages * c.stage_floats > red ? c.stages * c.stage_floats : red;
@@ -121,15 +124,35 @@ __device__ __forceinline__ void con_cp16(float* dst, const float* src) {
                : "memory");
 }
 
-// one primary: S1, S2 the first bin of the tile's sides, st floats between bins
-template <int T, bool DIAG>
+__device__ __forceinline__ float con_lds(uint32_t p) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(p) : "memory");
+  return v;
+}
+
+// One primary: S1, S2 the first bin of the tile's sides, ST floats between
+// bins (0: st, at run time).  On the diagonal only pairs with a column at or
+// right of the row.
+template <int T, bool DIAG, int ST>
 __device__ __forceinline__ void con_step(float2 (&acc)[T][T / 2], const float* S1, const float* S2, int st, float w) {
   float x[T], y[T];
+  if constexpr (ST > 0) {
 #pragma unroll
-  for (int i = 0; i < T; ++i) x[i] = S1[i * st];
-  if constexpr (!DIAG) {
+    for (int i = 0; i < T; ++i) x[i] = S1[i * ST];
+    if constexpr (!DIAG) {
 #pragma unroll
-    for (int i = 0; i < T; ++i) y[i] = S2[i * st];
+      for (int i = 0; i < T; ++i) y[i] = S2[i * ST];
+    }
+  } else {
+    // the row's own stride: addresses by addition (products take the FMA pipe)
+    uint32_t p = (uint32_t)__cvta_generic_to_shared(S1);
+#pragma unroll
+    for (int i = 0; i < T; ++i, p += 4u * (uint32_t)st) x[i] = con_lds(p);
+    if constexpr (!DIAG) {
+      p = (uint32_t)__cvta_generic_to_shared(S2);
+#pragma unroll
+      for (int i = 0; i < T; ++i, p += 4u * (uint32_t)st) y[i] = con_lds(p);
+    }
   }
 #pragma unroll
   for (int i = 0; i < T; ++i) {
@@ -145,8 +168,8 @@ __device__ __forceinline__ void con_step(float2 (&acc)[T][T / 2], const float* S
 template <int T, int CH, int MODE>
 __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(ContractArgs a, ConShape sh) {
   extern __shared__ __align__(16) float s_dyn[];
-  __shared__ int s_slotl[CH];  // multipole of each slot of the chunk (-1: none)
-  __shared__ int s_ord[CH];    // the chunk's slots by multipole
+  __shared__ __align__(16) int s_slotl[CH];  // multipole of each slot of the chunk (-1: none)
+  __shared__ int s_ord[CH];                  // the chunk's slots by multipole
   __shared__ int s_l[kLmaxCap + 1], s_l0[kLmaxCap + 2], s_nl;  // its multipoles and where their slots start
   const int nb = a.nbins, L = a.lmax;
   const int nc = a.sphere ? 2 * L + 1 : (L + 1) * (L + 1);  // coefficients per (primary, bin)
@@ -179,7 +202,7 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
   const bool active = tv >= 0;
   const int B1 = active ? tv & 255 : 0, B2 = active ? tv >> 8 : 0;
   auto start = [&](int B) { return max(min(B * T, nb - T), 0); };
-  const int stride = MODE == kConLinear ? sh.stride : CH;
+  const int stride = MODE == kConLinearAny ? sh.stride : CH;
   const int off1 = start(B1) * stride + c, off2 = start(B2) * stride + c;
   const int qstride = nb * stride;
   double* out = a.partial + (size_t)(a.part0 + blockIdx.x) * (L + 1) * nb * nb;
@@ -210,36 +233,35 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
     __syncthreads();
     if (tid < CH) {
       const int l = s_slotl[tid];
-      int below = 0, distinct = 0, prev = 0;  // prev: an earlier slot has this l
-      unsigned seen = 0;                      // multipoles below l
-      for (int k = 0; k < CH; ++k) {
-        const int lk = s_slotl[k];
-        if (lk < 0) continue;
-        below += lk < l || (lk == l && k < tid);
-        prev |= lk == l && k < tid;
-        if (lk < l) seen |= 1u << lk;
+      int below = 0, n = 0;  // slots sorted before this one; all slots
+      bool first = true;     // no earlier slot has this multipole
+      unsigned seen = 0;     // multipoles of the chunk
+      const int4* sl4 = reinterpret_cast<const int4*>(s_slotl);
+#pragma unroll 4
+      for (int k = 0; k < CH; k += 4) {
+        const int4 v = sl4[k / 4];
+        const int lk[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const bool in = lk[e] >= 0, before = k + e < tid;
+          n += in;
+          below += in && (lk[e] < l || (lk[e] == l && before));
+          if (lk[e] == l && before) first = false;
+          seen |= in ? 1u << lk[e] : 0u;
+        }
       }
-      distinct = __popc(seen);
       if (l >= 0) {
         s_ord[below] = tid;
-        if (!prev) {
-          s_l[distinct] = l;
-          s_l0[distinct] = below;
+        if (first) {
+          const int rank = __popc(seen & ((1u << l) - 1u));
+          s_l[rank] = l;
+          s_l0[rank] = below;
         }
       }
-    }
-    if (tid == 0) {
-      unsigned all = 0;
-      int n = 0;
-      for (int k = 0; k < CH; ++k) {
-        const int lk = s_slotl[k];
-        if (lk >= 0) {
-          all |= 1u << lk;
-          ++n;
-        }
+      if (tid == 0) {
+        s_nl = __popc(seen);
+        s_l0[s_nl] = n;
       }
-      s_nl = __popc(all);
-      s_l0[__popc(all)] = n;
     }
     __syncthreads();
 
@@ -248,7 +270,7 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
       float* buf = s_stage + st * sh.stage_floats;
       if (tid < cnt) con_cp4(s_w + st * kConMaxQ + tid, a.wprim + pb + tid);
       const float* src = a.M + pb * nb * (int64_t)a.row;
-      if constexpr (MODE == kConLinear) {
+      if constexpr (MODE == kConLinear || MODE == kConLinearAny) {
         const int total = cnt * nb * a.row;
         int k = tid * 4;
         if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
@@ -280,36 +302,42 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
       }
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
-    // the sums over each multipole's slots, row i of every tile at a time
+    // the sums over each multipole's slots: all accumulators to shared memory
+    // ([entry of the tile][thread]), then one thread per (entry, multipole),
+    // four slots' loads in flight
     auto flush = [&] {
-      float* red = s_stage;  // [pg][tile][T][CH]
-      const int nl = s_nl, total = sh.tiles * T * nl;
+      float* red = s_stage;
+      const int nthr = blockDim.x, nl = s_nl;
+      __syncthreads();
 #pragma unroll
-      for (int i = 0; i < T; ++i) {
-        __syncthreads();
+      for (int i = 0; i < T; ++i)
 #pragma unroll
         for (int j = 0; j < T / 2; ++j) {
-          red[((pg * sh.tiles + tl) * T + 2 * j) * CH + c] = acc[i][j].x;
-          red[((pg * sh.tiles + tl) * T + 2 * j + 1) * CH + c] = acc[i][j].y;
+          red[(i * T + 2 * j) * nthr + tid] = acc[i][j].x;
+          red[(i * T + 2 * j + 1) * nthr + tid] = acc[i][j].y;
           acc[i][j] = make_float2(0.f, 0.f);
         }
-        __syncthreads();
-        for (int o = tid; o < total; o += blockDim.x) {
-          const int tj = o / nl, k = o - tj * nl;
-          const int t = tj / T, j = tj % T;
-          const int v2 = s_tile[t];
-          if (v2 < 0) continue;
-          const int C1 = v2 & 255, C2 = v2 >> 8;
-          const int b1 = start(C1) + i, b2 = start(C2) + j;
-          if (b1 >= nb || b2 >= nb || b1 > b2 || b1 < C1 * T || b2 < C2 * T) continue;
-          const int q0 = s_l0[k], q1 = s_l0[k + 1];
-          float v = 0.f;
-          for (int g = 0; g < sh.pg; ++g) {
-            const float* rg = red + ((g * sh.tiles + t) * T + j) * CH;
-            for (int q = q0; q < q1; ++q) v += rg[s_ord[q]];
+      __syncthreads();
+      const int total = sh.tiles * T * T * nl;
+      for (int o = tid; o < total; o += nthr) {
+        const int tk = o / nl, k = o - tk * nl;
+        const int t = tk / (T * T), ij = tk % (T * T);
+        const int v2 = s_tile[t];
+        if (v2 < 0) continue;
+        const int C1 = v2 & 255, C2 = v2 >> 8;
+        const int b1 = start(C1) + ij / T, b2 = start(C2) + ij % T;
+        if (b1 >= nb || b2 >= nb || b1 > b2 || b1 < C1 * T || b2 < C2 * T) continue;
+        const int q0 = s_l0[k], q1 = s_l0[k + 1];
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int g = 0; g < sh.pg; ++g) {
+          const float* rg = red + ij * nthr + (g * sh.tiles + t) * CH;
+          for (int q = q0; q < q1; q += 4) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (q + e < q1) v[e] += rg[s_ord[q + e]];
           }
-          out[((size_t)s_l[k] * nb + b1) * nb + b2] += (double)v;
         }
+        out[((size_t)s_l[k] * nb + b1) * nb + b2] += (double)((v[0] + v[1]) + (v[2] + v[3]));
       }
       __syncthreads();
     };
@@ -341,12 +369,13 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
         const float* buf = s_stage + st * sh.stage_floats + pg * qstride;
         const float* wq = s_w + st * kConMaxQ;
         if (active) {
+          constexpr int ST = MODE == kConLinearAny ? 0 : CH;
           if (B1 == B2) {
             for (int q = pg; q < cnt; q += sh.pg, buf += sh.pg * qstride)
-              con_step<T, true>(acc, buf + off1, nullptr, stride, wq[q]);
+              con_step<T, true, ST>(acc, buf + off1, nullptr, stride, wq[q]);
           } else {
             for (int q = pg; q < cnt; q += sh.pg, buf += sh.pg * qstride)
-              con_step<T, false>(acc, buf + off1, buf + off2, stride, wq[q]);
+              con_step<T, false, ST>(acc, buf + off1, buf + off2, stride, wq[q]);
           }
         }
         if (sh.stages > 1) {
@@ -362,13 +391,14 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
 
 template <int T, int CH>
 static const void* con_fn(int mode) {
-  return mode == kConLinear   ? (const void*)k_contract_fp32<T, CH, kConLinear>
-         : mode == kConRows16 ? (const void*)k_contract_fp32<T, CH, kConRows16>
+  return mode == kConLinear      ? (const void*)k_contract_fp32<T, CH, kConLinear>
+         : mode == kConLinearAny ? (const void*)k_contract_fp32<T, CH, kConLinearAny>
+         : mode == kConRows16    ? (const void*)k_contract_fp32<T, CH, kConRows16>
                               : (const void*)k_contract_fp32<T, CH, kConRows4>;
 }
 
 static const void* con_kernel(const ConShape& sh, int row, bool aligned) {
-  const int mode = sh.nchunk == 1 ? kConLinear : ((row & 3) == 0 && aligned ? kConRows16 : kConRows4);
+  const int mode = sh.nchunk == 1 ? (row == sh.ch ? kConLinear : kConLinearAny) : ((row & 3) == 0 && aligned ? kConRows16 : kConRows4);
   switch (sh.T * 1000 + sh.ch) {
     case 6032: return con_fn<6, 32>(mode);
     case 6064: return con_fn<6, 64>(mode);
