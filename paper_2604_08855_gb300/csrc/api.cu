@@ -500,7 +500,7 @@ int load_points(ctb_ctx* c, const double* xyz, const double* w, int64_t n) {
   CK(c, ensure(c, c->cell_start, ((size_t)g.ncells + 1) * 4));
   const size_t hw = sort_hist_words(n);
   CK(c, ensure(c, c->hist, hw * 4));
-  CK(c, ensure(c, c->scan_tmp, std::max(scan_tmp_words(hw), scan_tmp_words((size_t)g.ncells + 1)) * 4));
+  CK(c, ensure(c, c->scan_tmp, scan_tmp_words(hw) * 4));
 
   IngestOut io{P<uint32_t>(c->key0), P<uint32_t>(c->val0), P<uint4>(c->pts_in)};
   const double inv_unit = 1.0 / c->unit;
@@ -515,7 +515,7 @@ int load_points(ctb_ctx* c, const double* xyz, const double* w, int64_t n) {
   uint32_t* vs = in1 ? sb.v1 : sb.v0;
   CK(c, launch_gather(vs, P<uint4>(c->pts_in), n, P<uint4>(c->pts), P<uint32_t>(c->s2i), P<uint32_t>(c->i2s),
                       c->st));
-  CK(c, launch_cell_start(ks, n, g.ncells, P<uint32_t>(c->cell_start), P<uint32_t>(c->scan_tmp), c->st));
+  CK(c, launch_cell_start(ks, n, g.ncells, P<uint32_t>(c->cell_start), c->st));
   CK(c, cudaEventRecord(c->ev[2], c->st));
   uint32_t fl[4] = {0, 0, 0, 0};
   CK(c, cudaMemcpyAsync(fl, c->flags.p, sizeof(fl), cudaMemcpyDeviceToHost, c->st));
@@ -970,7 +970,7 @@ int batch_impl(ctb_ctx* c, const double* const* xyz, const double* const* w, con
   CK(c, ensure(c, c->cell_start, (size_t)(cells_all + 1) * 4));
   const size_t hw = sort_hist_words(N);
   CK(c, ensure(c, c->hist, hw * 4));
-  CK(c, ensure(c, c->scan_tmp, std::max(scan_tmp_words(hw), scan_tmp_words((size_t)cells_all + 1)) * 4));
+  CK(c, ensure(c, c->scan_tmp, scan_tmp_words(hw) * 4));
   CK(c, ensure(c, c->flags, 64));
   CK(c, cudaMemsetAsync(c->flags.p, 0, 64, c->st));
   CK(c, cudaEventRecord(c->ev[0], c->st));
@@ -1002,7 +1002,7 @@ int batch_impl(ctb_ctx* c, const double* const* xyz, const double* const* w, con
   uint32_t* ks = in1 ? sb.k1 : sb.k0;
   uint32_t* vs = in1 ? sb.v1 : sb.v0;
   CK(c, launch_gather(vs, P<uint4>(c->pts_in), N, P<uint4>(c->pts), P<uint32_t>(c->s2i), P<uint32_t>(c->i2s), c->st));
-  CK(c, launch_cell_start(ks, N, (uint32_t)cells_all, P<uint32_t>(c->cell_start), P<uint32_t>(c->scan_tmp), c->st));
+  CK(c, launch_cell_start(ks, N, (uint32_t)cells_all, P<uint32_t>(c->cell_start), c->st));
   CK(c, cudaEventRecord(c->ev[2], c->st));
   uint32_t fl = 0;
   uint32_t fl3 = 0;

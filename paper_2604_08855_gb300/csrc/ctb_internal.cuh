@@ -266,10 +266,9 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t len,
 cudaError_t launch_gather(const uint32_t* val_sorted, const uint4* pts_in, int64_t n,
                           uint4* pts_sorted, uint32_t* sorted_to_input,
                           uint32_t* input_to_sorted, cudaStream_t st);
-// cell_start[c] = first sorted position with key >= c, c in [0, ncells];
-// scan_tmp holds scan_tmp_words(ncells + 1) words
+// cell_start[c] = first sorted position with key >= c, c in [0, ncells]
 cudaError_t launch_cell_start(const uint32_t* key_sorted, int64_t n, uint32_t ncells, uint32_t* cell_start,
-                              uint32_t* scan_tmp, cudaStream_t st);
+                              cudaStream_t st);
 
 // shared.cu -- pivot groups for shared neighbour lists
 struct PivotGrid {

@@ -184,32 +184,38 @@ __global__ void k_scan_reduce(const uint32_t* __restrict__ in, size_t len, uint3
   if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// scans one tile per block; adds offs[blockIdx.x] (offs may be NULL)
-__global__ void k_scan_tile(const uint32_t* __restrict__ in, size_t len, const uint32_t* __restrict__ offs,
+// scans `tiles` consecutive tiles per block; adds offs[blockIdx.x] (offs may be NULL)
+__global__ void k_scan_tile(const uint32_t* __restrict__ in, size_t len, const uint32_t* __restrict__ offs, int tiles,
                             uint32_t* __restrict__ out) {
-  size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
-  uint32_t v[kScanItems];
-  uint32_t s = 0;
+  uint32_t carry = offs ? offs[blockIdx.x] : 0u;
+  for (int t = 0; t < tiles; ++t) {
+    size_t base = ((size_t)blockIdx.x * tiles + t) * kScanTile + (size_t)threadIdx.x * kScanItems;
+    uint32_t v[kScanItems];
+    uint32_t s = 0;
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (base + k < len) ? in[base + k] : 0;
-    s += v[k];
-  }
-  uint32_t total;
-  uint32_t ex = block_exclusive_scan(s, &total);
-  if (offs) ex += offs[blockIdx.x];
+    for (int k = 0; k < kScanItems; ++k) {
+      v[k] = (base + k < len) ? in[base + k] : 0;
+      s += v[k];
+    }
+    uint32_t total;
+    uint32_t ex = carry + block_exclusive_scan(s, &total);
+    carry += total;
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    if (base + k < len) out[base + k] = ex;
-    ex += v[k];
+    for (int k = 0; k < kScanItems; ++k) {
+      if (base + k < len) out[base + k] = ex;
+      ex += v[k];
+    }
   }
 }
+
+// One block scans up to kScanOne tiles by itself: three launches cost more.
+constexpr int kScanOne = 4;
 
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t len, uint32_t* tmp,
                                cudaStream_t st) {
   if (len == 0) return cudaSuccess;
-  if (len <= (size_t)kScanTile) {
-    k_scan_tile<<<1, kScanThreads, 0, st>>>(in, len, nullptr, out);
+  if (len <= (size_t)kScanTile * kScanOne) {
+    k_scan_tile<<<1, kScanThreads, 0, st>>>(in, len, nullptr, (int)((len + kScanTile - 1) / kScanTile), out);
     ++g_launches;
     return cudaGetLastError();
   }
@@ -222,7 +228,7 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t len, ui
   // scan the block sums in place (recursively), workspace after them
   e = exclusive_scan_u32(sums, sums, nb, tmp + nb, st);
   if (e != cudaSuccess) return e;
-  k_scan_tile<<<(unsigned)nb, kScanThreads, 0, st>>>(in, len, sums, out);
+  k_scan_tile<<<(unsigned)nb, kScanThreads, 0, st>>>(in, len, sums, 1, out);
   ++g_launches;
   return cudaGetLastError();
 }
@@ -231,21 +237,31 @@ cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t len, ui
 // LSD radix sort of (key, val) pairs, 8-bit digits, stable
 
 constexpr int kSortThreads = 256;
-constexpr int kSortRounds = 16;
-constexpr int kSortTile = kSortThreads * kSortRounds;  // keys per block
+constexpr int kSortRounds = 16;  // rounds of kSortThreads keys a block takes at most
 
-int sort_blocks(int64_t n) { return (int)((n + kSortTile - 1) / kSortTile); }
+// Rounds per block: 16, and fewer below 2.5e5 keys, so that 64 blocks share a
+// small catalogue (20,000 keys in 5 blocks of 16 rounds took 28 us a digit,
+// in 40 blocks of 2 rounds 14).
+static int sort_rounds(int64_t n) {
+  const int64_t r = (n + 64 * kSortThreads - 1) / (64 * kSortThreads);
+  return (int)(r < 1 ? 1 : (r > kSortRounds ? kSortRounds : r));
+}
+
+int sort_blocks(int64_t n) {
+  const int64_t tile = (int64_t)kSortThreads * sort_rounds(n);
+  return (int)((n + tile - 1) / tile);
+}
 size_t sort_hist_words(int64_t n) { return (size_t)256 * (size_t)(sort_blocks(n) > 0 ? sort_blocks(n) : 1); }
 
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __restrict__ key, int64_t n,
                                                              int shift, uint32_t* __restrict__ hist,
-                                                             int nblk) {
+                                                             int nblk, int rounds) {
   __shared__ uint32_t s_h[256];
   s_h[threadIdx.x] = 0;
   __syncthreads();
-  int64_t base = (int64_t)blockIdx.x * kSortTile;
+  int64_t base = (int64_t)blockIdx.x * kSortThreads * rounds;
 #pragma unroll 4
-  for (int r = 0; r < kSortRounds; ++r) {
+  for (int r = 0; r < rounds; ++r) {
     int64_t i = base + (int64_t)r * kSortThreads + threadIdx.x;
     if (i < n) atomicAdd(&s_h[(key[i] >> shift) & 255u], 1u);
   }
@@ -255,7 +271,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __r
 
 __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
-    const uint32_t* __restrict__ offs, int nblk, uint32_t* __restrict__ kout, uint32_t* __restrict__ vout) {
+    const uint32_t* __restrict__ offs, int nblk, int rounds, uint32_t* __restrict__ kout, uint32_t* __restrict__ vout) {
   __shared__ uint32_t s_wc[kSortThreads / 32][256];
   __shared__ uint32_t s_run[256];
   __shared__ uint32_t s_goff[256];
@@ -263,8 +279,8 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
   s_goff[threadIdx.x] = offs[(size_t)threadIdx.x * nblk + blockIdx.x];
   s_run[threadIdx.x] = 0;
   const unsigned lt = (1u << lane) - 1u;
-  int64_t base = (int64_t)blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortRounds; ++r) {
+  int64_t base = (int64_t)blockIdx.x * kSortThreads * rounds;
+  for (int r = 0; r < rounds; ++r) {
 #pragma unroll
     for (int w = 0; w < kSortThreads / 32; ++w) s_wc[w][threadIdx.x] = 0;
     __syncthreads();
@@ -304,16 +320,16 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
 cudaError_t radix_sort(SortBufs& b, int64_t n, int bits, bool* result_in_1, cudaStream_t st) {
   *result_in_1 = false;
   if (n <= 1 || bits <= 0) return cudaSuccess;
-  int nblk = sort_blocks(n);
+  const int nblk = sort_blocks(n), rounds = sort_rounds(n);
   uint32_t *ki = b.k0, *vi = b.v0, *ko = b.k1, *vo = b.v1;
   for (int shift = 0; shift < bits; shift += 8) {
-    k_radix_hist<<<nblk, kSortThreads, 0, st>>>(ki, n, shift, b.hist, nblk);
+    k_radix_hist<<<nblk, kSortThreads, 0, st>>>(ki, n, shift, b.hist, nblk, rounds);
     ++g_launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = exclusive_scan_u32(b.hist, b.hist, (size_t)256 * nblk, b.scan_tmp, st);
     if (e != cudaSuccess) return e;
-    k_radix_scatter<<<nblk, kSortThreads, 0, st>>>(ki, vi, n, shift, b.hist, nblk, ko, vo);
+    k_radix_scatter<<<nblk, kSortThreads, 0, st>>>(ki, vi, n, shift, b.hist, nblk, rounds, ko, vo);
     ++g_launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -348,38 +364,85 @@ cudaError_t launch_gather(const uint32_t* val_sorted, const uint4* pts_in, int64
   return cudaGetLastError();
 }
 
-// cell_start[c] = first sorted position with key >= c, for c in [0, ncells]:
-// the exclusive prefix sum of the points per cell.  The counts are added by
-// one atomic per run of equal keys within a warp (the keys are sorted), so
-// empty cells cost only the scan, however long the empty stretches.
-__global__ void k_cell_count(const uint32_t* __restrict__ key, int64_t n, uint32_t* __restrict__ cnt) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int lane = threadIdx.x & 31;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
-    const int64_t i = base + (threadIdx.x & ~31) + lane;
-    const bool ok = i < n;
-    const unsigned act = __ballot_sync(0xffffffffu, ok);
-    if (ok) {
-      const uint32_t k = key[i];
-      const unsigned grp = __match_any_sync(act, k);
-      if (lane == __ffs(grp) - 1) atomicAdd(cnt + k, (uint32_t)__popc(grp));
+// cell_start[c] = first sorted position with key >= c, for c in [0, ncells].
+// A block writes kCellTile entries: it finds the tile's first point by a
+// 32-way search of the sorted keys, counts the tile's points per cell in
+// shared memory and scans the counts.  So the table is written once and not
+// read: it is far larger than the catalogue where cells are fine (5.3 GB for
+// 3.1M points on the sphere at 8 cells per r_max), and clearing, counting,
+// reducing and scanning it took 5.2 ms and 16 MB's worth 30 us of launches
+// (now 1.1 ms and 9 us).
+constexpr int kCellThreads = 256;
+constexpr int kCellItems = 32;
+constexpr int kCellTile = kCellThreads * kCellItems;
+
+// first position whose key is at least c, by one warp
+__device__ __forceinline__ uint32_t lower_bound_warp(const uint32_t* __restrict__ key, uint32_t n, uint64_t c, int lane) {
+  uint32_t lo = 0, len = n;  // the answer lies in [lo, lo + len]
+  while (len > 0) {
+    const uint32_t step = len / 32u + 1u;
+    const uint32_t p = lo + step * (uint32_t)lane + step - 1u;  // the last of this lane's stretch
+    const bool below = p < lo + len ? key[p] < c : false;
+    const uint32_t k = (uint32_t)__popc(__ballot_sync(0xffffffffu, below));  // stretches wholly below c
+    const uint32_t nlo = min(lo + k * step, lo + len);
+    len = min(step - 1u, lo + len - nlo);
+    lo = nlo;
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(kCellThreads) k_cell_table(const uint32_t* __restrict__ key, uint32_t n,
+                                                             uint64_t entries, uint32_t* __restrict__ cell_start) {
+  // entry k of the tile at [k / kCellItems][k % kCellItems], rows padded by one: conflict-free both ways
+  __shared__ uint32_t s_cnt[kCellThreads * (kCellItems + 1)];
+  __shared__ uint32_t s_range[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint64_t c0 = (uint64_t)blockIdx.x * kCellTile;
+  if (warp < 2) {
+    const uint32_t p = lower_bound_warp(key, n, c0 + (uint64_t)warp * kCellTile, lane);
+    if (lane == 0) s_range[warp] = p;
+  }
+  for (int k = tid; k < kCellThreads * (kCellItems + 1); k += kCellThreads) s_cnt[k] = 0;
+  __syncthreads();
+  const uint32_t p0 = s_range[0], p1 = s_range[1];
+  for (uint32_t p = p0 + tid; p < p1; p += kCellThreads) {
+    const uint32_t k = (uint32_t)(key[p] - c0);
+    atomicAdd(s_cnt + k + k / kCellItems, 1u);
+  }
+  __syncthreads();
+  uint32_t v[kCellItems], s = 0;
+#pragma unroll
+  for (int k = 0; k < kCellItems; ++k) {
+    v[k] = s_cnt[tid * (kCellItems + 1) + k];
+    s += v[k];
+  }
+  uint32_t total;
+  uint32_t ex = p0 + block_exclusive_scan(s, &total);
+#pragma unroll
+  for (int k = 0; k < kCellItems; ++k) {
+    s_cnt[tid * (kCellItems + 1) + k] = ex;
+    ex += v[k];
+  }
+  __syncthreads();
+  // 16-byte stores of the tile in order (the table and the tile start on 16 bytes)
+  for (int k = 4 * tid; k < kCellTile; k += 4 * kCellThreads) {
+    const uint32_t* e = s_cnt + k + k / kCellItems;
+    const uint64_t c = c0 + k;
+    if (c + 4 <= entries) {
+      __stcs(reinterpret_cast<uint4*>(cell_start + c), make_uint4(e[0], e[1], e[2], e[3]));
+    } else {
+      for (int d = 0; d < 4 && c + d < entries; ++d) cell_start[c + d] = e[d];
     }
   }
 }
 
 cudaError_t launch_cell_start(const uint32_t* key_sorted, int64_t n, uint32_t ncells, uint32_t* cell_start,
-                              uint32_t* scan_tmp, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(cell_start, 0, ((size_t)ncells + 1) * sizeof(uint32_t), st);
-  if (e != cudaSuccess) return e;
-  if (n > 0) {
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 65535 * 4) blocks = 65535 * 4;
-    k_cell_count<<<blocks, 256, 0, st>>>(key_sorted, n, cell_start);
-    ++g_launches;
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return exclusive_scan_u32(cell_start, cell_start, (size_t)ncells + 1, scan_tmp, st);
+                              cudaStream_t st) {
+  const uint64_t entries = (uint64_t)ncells + 1;
+  k_cell_table<<<(unsigned)((entries + kCellTile - 1) / kCellTile), kCellThreads, 0, st>>>(key_sorted, (uint32_t)n,
+                                                                                          entries, cell_start);
+  ++g_launches;
+  return cudaGetLastError();
 }
 
 }  // namespace ctb
