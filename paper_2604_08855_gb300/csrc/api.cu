@@ -67,6 +67,7 @@ struct ctb_ctx {
   Buf xyz_stage, w_stage, key0, val0, key1, val1, hist, scan_tmp, pts_in, pts, s2i, i2s, cell_start;
   Buf flags, bbox_part, lists, M, wprim, partial, zeta, prim, counters, norm, slot, idx64, alm, thr;
   Buf edge_in, edge_tj;  // edge correction: staged sums, 3j table
+  bool edge_tj_ready = false;
   Buf pairsum;          // FP64 partial pair sums [catalogue][part][bin] of the last compute
   int pairsum_segs = 0;  // catalogues they cover (0: none)
   int pairsum_parts = 0;
@@ -162,6 +163,7 @@ void release_all(ctb_ctx* c) {
                 &c->gprim, &c->gw};
   for (Buf* b : all) release(c, *b);
   c->tables_ready = false;
+  c->edge_tj_ready = false;
 }
 
 int ensure_events(ctb_ctx* c) {
@@ -1534,20 +1536,49 @@ int ctb_edge_correct(ctb_ctx* c, const double* zeta_nnn, const double* zeta_rrr,
   CK(c, cudaSetDevice(c->dev));
   const int n = c->lmax + 1, nb = c->nbins;
   const size_t zsz = (size_t)n * nb * nb;
-  // the 3j table, then both inputs and the output in device memory (staged when on the host)
-  std::vector<double> tj;
-  make_threej_table(c->lmax, tj);
-  CK(c, ensure(c, c->edge_tj, tj.size() * sizeof(double)));
-  CK(c, ensure(c, c->edge_in, 3 * zsz * sizeof(double)));
-  double* dn = P<double>(c->edge_in);
-  double* dr = dn + zsz;
-  double* dout = dr + zsz;
-  CK(c, cudaMemcpyAsync(c->edge_tj.p, tj.data(), tj.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  CK(c, cudaMemcpyAsync(dn, zeta_nnn, zsz * sizeof(double), cudaMemcpyDefault, c->st));
-  CK(c, cudaMemcpyAsync(dr, zeta_rrr, zsz * sizeof(double), cudaMemcpyDefault, c->st));
-  CK(c, launch_edge_correct(dn, dr, P<double>(c->edge_tj), c->lmax, nb, dout, c->st));
-  CK(c, cudaMemcpyAsync(zeta_out, dout, zsz * sizeof(double), cudaMemcpyDefault, c->st));
-  CK(c, cudaStreamSynchronize(c->st));  // the host table and host outputs are done with
+  // the 3j table of this l_max, laid out once per context
+  if (!c->edge_tj_ready) {
+    std::vector<double> tj;
+    make_threej_table(c->lmax, tj);
+    CK(c, ensure(c, c->edge_tj, tj.size() * sizeof(double)));
+    CK(c, cudaMemcpyAsync(c->edge_tj.p, tj.data(), tj.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
+    CK(c, cudaStreamSynchronize(c->st));  // the host table goes out of scope
+    c->edge_tj_ready = true;
+  }
+  // inputs and output where they lie, if that is this device's memory; staged
+  // otherwise.  Each bin pair is read whole before it is written, so zeta_out
+  // may be an input; an output that overlaps one shifted is staged.
+  auto direct = [&](const double* p) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return (at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == c->dev)) &&
+           (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+  };
+  auto shifted = [&](const double* p) { return zeta_out != p && zeta_out < p + zsz && p < zeta_out + zsz; };
+  const bool hn = !direct(zeta_nnn), hr = !direct(zeta_rrr);
+  const bool ho = !direct(zeta_out) || shifted(zeta_nnn) || shifted(zeta_rrr);
+  const double* pn = zeta_nnn;
+  const double* pr = zeta_rrr;
+  double* po = zeta_out;
+  if (hn || hr || ho) {
+    CK(c, ensure(c, c->edge_in, 3 * zsz * sizeof(double)));
+    double* d = P<double>(c->edge_in);
+    if (hn) {
+      CK(c, cudaMemcpyAsync(d, zeta_nnn, zsz * sizeof(double), cudaMemcpyDefault, c->st));
+      pn = d;
+    }
+    if (hr) {
+      CK(c, cudaMemcpyAsync(d + zsz, zeta_rrr, zsz * sizeof(double), cudaMemcpyDefault, c->st));
+      pr = d + zsz;
+    }
+    if (ho) po = d + 2 * zsz;
+  }
+  CK(c, launch_edge_correct(pn, pr, P<double>(c->edge_tj), c->lmax, nb, po, c->st));
+  if (ho) CK(c, cudaMemcpyAsync(zeta_out, po, zsz * sizeof(double), cudaMemcpyDefault, c->st));
+  CK(c, cudaStreamSynchronize(c->st));  // zeta_out is complete
   return CTB_OK;
 }
 

@@ -8,8 +8,8 @@
 // per bin pair,
 //     n_l / r_0 = sum_l' M_ll' zeta_l',   M_ll' = (2l+1) sum_l'' (l l' l''; 0 0 0)^2 f_l'',
 // where n_l = (2l+1)/2 S_l(N), r_l = (2l+1)/2 S_l(R), f_l = r_l / r_0, all
-// sums truncated at l_max.  One thread solves one bin pair's system in FP64
-// by Gaussian elimination with partial pivoting.
+// sums truncated at l_max.  One warp solves one bin pair's system in FP64 by
+// Gaussian elimination with partial pivoting.
 #include <cmath>
 #include <vector>
 
@@ -39,68 +39,95 @@ void make_threej_table(int lmax, std::vector<double>& t) {
 }
 
 constexpr int kEdgeN = kLmaxCap + 1;
+constexpr int kEdgeStride = kEdgeN + 2;  // doubles per matrix row: the right-hand side in column n, odd
+constexpr int kEdgeWarps = 4;
 
-__global__ void k_edge_correct(const double* __restrict__ zn, const double* __restrict__ zr,
-                               const double* __restrict__ tj, int lmax, int nb, double* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nb * nb) return;
+// One warp solves one bin pair's system, the matrix in shared memory: lanes
+// take entries while it is built, rows while a pivot is chosen, and columns
+// while it is eliminated.  Bound by FP64 (two FMAs a clock and SM; about 110
+// warp FMAs a pair at l_max 10, 7 us for 36 x 36 bins) and, at 8 warps per SM,
+// by the latency of its steps.  One thread a pair kept
+// its matrix in local memory and left most of the chip idle (36 bins, l_max
+// 10: 170 us; now 52, cold caches).
+__global__ void __launch_bounds__(32 * kEdgeWarps) k_edge_correct(const double* zn, const double* zr,
+                                                                  const double* __restrict__ tj, int lmax, int nb,
+                                                                  double* out) {
+  __shared__ double s_m[kEdgeWarps][kEdgeN * kEdgeStride];
+  __shared__ double s_v[kEdgeWarps][kEdgeN + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = blockIdx.x * kEdgeWarps + warp;
+  if (t >= nb * nb) return;  // a whole warp; no block barrier below
+  double* m = s_m[warp];
+  double* v = s_v[warp];
   const int n = lmax + 1;
   const size_t plane = (size_t)nb * nb;
-  double f[kEdgeN], rhs[kEdgeN], m[kEdgeN][kEdgeN];
-  const double r0 = 0.5 * zr[t];  // (2*0+1)/2 S_0
+  const bool row = lane < n;
+  const double c = 0.5 * (2.0 * lane + 1.0);
+  const double r = row ? c * zr[lane * plane + t] : 0.0;
+  const double nn = row ? c * zn[lane * plane + t] : 0.0;
+  const double r0 = __shfl_sync(0xffffffffu, r, 0);
   bool ok = r0 != 0.0 && isfinite(r0);
-  for (int l = 0; l < n; ++l) {
-    const double c = 0.5 * (2.0 * l + 1.0);
-    f[l] = ok ? c * zr[l * plane + t] / r0 : 0.0;
-    rhs[l] = ok ? c * zn[l * plane + t] / r0 : 0.0;
+  const double f = ok ? r / r0 : 0.0;
+  // a ratio that is not finite enters every row
+  ok = ok && __all_sync(0xffffffffu, isfinite(f));
+  if (row) {
+    v[lane] = f;
+    m[lane * kEdgeStride + n] = ok ? nn / r0 : 0.0;
   }
-  for (int l = 0; l < n; ++l)
-    for (int lp = 0; lp < n; ++lp) {
-      double s = 0.0;
-      for (int lpp = 0; lpp < n; ++lpp) s += tj[((size_t)l * n + lp) * n + lpp] * f[lpp];
-      m[l][lp] = (2.0 * l + 1.0) * s;
-    }
-  // Gaussian elimination with partial pivoting
+  __syncwarp();
+  // M_ll' = (2l+1) sum_l'' (l l' l''; 000)^2 f_l'': l'' of the triangle and parity
+  for (int e = lane; e < n * n; e += 32) {
+    const int l = e / n, lp = e - l * n;
+    double s = 0.0;
+    for (int q = l > lp ? l - lp : lp - l; q <= l + lp && q < n; q += 2) s += __ldg(tj + ((size_t)l * n + lp) * n + q) * v[q];
+    m[l * kEdgeStride + lp] = (2.0 * l + 1.0) * s;
+  }
+  __syncwarp();
+  // Gaussian elimination with partial pivoting (the first of equal pivots)
   for (int k = 0; k < n && ok; ++k) {
-    int piv = k;
-    double best = fabs(m[k][k]);
-    for (int i = k + 1; i < n; ++i)
-      if (fabs(m[i][k]) > best) {
-        best = fabs(m[i][k]);
-        piv = i;
+    double best = row && lane >= k ? fabs(m[lane * kEdgeStride + k]) : -1.0;
+    const bool bad = isnan(__shfl_sync(0xffffffffu, best, k));
+    if (isnan(best)) best = -1.0;
+    int piv = lane;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double b2 = __shfl_xor_sync(0xffffffffu, best, o);
+      const int p2 = __shfl_xor_sync(0xffffffffu, piv, o);
+      if (b2 > best || (b2 == best && p2 < piv)) {
+        best = b2;
+        piv = p2;
       }
-    if (!(best > 0.0)) {
-      ok = false;
-      break;
     }
-    if (piv != k) {
-      for (int j = 0; j < n; ++j) {
-        const double tmp = m[k][j];
-        m[k][j] = m[piv][j];
-        m[piv][j] = tmp;
-      }
-      const double tmp = rhs[k];
-      rhs[k] = rhs[piv];
-      rhs[piv] = tmp;
+    ok = !bad && best > 0.0;
+    if (!ok) break;
+    // swap rows k and piv; this lane's column of the pivot row
+    const bool col = lane >= k && lane <= n;
+    const double pk = col ? m[piv * kEdgeStride + lane] : 0.0;
+    if (col && piv != k) {
+      m[piv * kEdgeStride + lane] = m[k * kEdgeStride + lane];
+      m[k * kEdgeStride + lane] = pk;
     }
-    for (int i = k + 1; i < n; ++i) {
-      const double q = m[i][k] / m[k][k];
-      for (int j = k; j < n; ++j) m[i][j] -= q * m[k][j];
-      rhs[i] -= q * rhs[k];
-    }
+    __syncwarp();
+    if (row && lane > k) v[lane] = m[lane * kEdgeStride + k] / m[k * kEdgeStride + k];
+    __syncwarp();
+    if (col)
+      for (int i = k + 1; i < n; ++i) m[i * kEdgeStride + lane] -= v[i] * pk;
+    __syncwarp();
   }
-  for (int k = n - 1; k >= 0; --k) {
-    double s = rhs[k];
-    for (int j = k + 1; j < n; ++j) s -= m[k][j] * rhs[j];
-    rhs[k] = ok ? s / m[k][k] : NAN;
+  // back substitution, a column at a time; lane l ends with zeta_l
+  double x = row ? m[lane * kEdgeStride + n] : 0.0;
+  for (int k = n - 1; k >= 0 && ok; --k) {
+    const double xk = __shfl_sync(0xffffffffu, x, k) / m[k * kEdgeStride + k];
+    if (lane == k) x = xk;
+    else if (lane < k) x -= m[lane * kEdgeStride + k] * xk;
   }
-  for (int l = 0; l < n; ++l) out[l * plane + t] = ok ? rhs[l] : NAN;
+  if (row) out[lane * plane + t] = ok ? x : NAN;
 }
 
 cudaError_t launch_edge_correct(const double* zn, const double* zr, const double* tj, int lmax, int nbins,
                                 double* out, cudaStream_t st) {
   const int total = nbins * nbins;
-  k_edge_correct<<<(total + 63) / 64, 64, 0, st>>>(zn, zr, tj, lmax, nbins, out);
+  k_edge_correct<<<(total + kEdgeWarps - 1) / kEdgeWarps, 32 * kEdgeWarps, 0, st>>>(zn, zr, tj, lmax, nbins, out);
   ++g_launches;
   return cudaGetLastError();
 }
