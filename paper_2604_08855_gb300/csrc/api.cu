@@ -3,7 +3,11 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
+#include <tuple>
+#include <utility>
 #include <vector>
 
 #include "ctb_internal.cuh"
@@ -12,7 +16,31 @@ using namespace ctb;
 
 namespace ctb {
 thread_local unsigned long long g_launches = 0;
+
+int resident_blocks(const void* fn, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int, size_t>, int> known;  // a few entries per kernel and device
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  // the limit belongs to the device's context, which a program may reset
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(dev, fn, threads, smem);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  int nb = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  known[key] = nb;
+  return nb;
 }
+}  // namespace ctb
 
 namespace {
 
@@ -63,6 +91,8 @@ struct ctb_ctx {
   int Lk = 0;
   float beta[(kLmaxCap + 1) * (kLmaxCap + 1)];
   bool tables_ready = false;
+  double thr_unit = 0;  // unit of the uploaded thresholds (0: none)
+  uint64_t* pin = nullptr;  // pinned words that counters and flags are read back into
   // device buffers
   Buf xyz_stage, w_stage, key0, val0, key1, val1, hist, scan_tmp, pts_in, pts, s2i, i2s, cell_start;
   Buf flags, bbox_part, lists, M, wprim, partial, zeta, prim, counters, norm, slot, idx64, alm, thr;
@@ -86,6 +116,7 @@ struct ctb_ctx {
   double t_ms[kStages] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   uint64_t npairs = 0;
   uint64_t nchunks = 0;  // primary chunks of the last compute
+  int chunk_open = 0;    // 1: a chunk's kernels are in flight, its times not added up yet (2: it has a pack)
   unsigned long long launches_points = 0, launches_compute = 0;
 };
 
@@ -169,6 +200,7 @@ void release_all(ctb_ctx* c) {
 int ensure_events(ctb_ctx* c) {
   if (c->ev_ready) return CTB_OK;
   for (auto& e : c->ev) CK(c, cudaEventCreate(&e));
+  if (!c->pin) CK(c, cudaMallocHost((void**)&c->pin, 64));
   c->ev_ready = true;
   return CTB_OK;
 }
@@ -317,6 +349,10 @@ namespace {
 // exact edges, the same FP64 values an FP64 evaluation of the bins uses:
 // r_min, r_min + b (r_max - r_min)/nbins, r_max
 int upload_thresholds(ctb_ctx* c) {
+  // the context's edges are fixed, so they change with the unit only (about
+  // 80 us of big-integer arithmetic for ten bins)
+  if (c->thr.p && c->thr_unit == c->unit) return CTB_OK;
+  c->thr_unit = 0;
   std::vector<unsigned long long> thr(c->nbins + 1);
   if (c->sphere) {
     // chord edges of the linear angular bins: 2 sin(theta_b / 2)
@@ -325,6 +361,7 @@ int upload_thresholds(ctb_ctx* c) {
     CK(c, ensure(c, c->thr, thr.size() * 8));
     CK(c, cudaMemcpyAsync(c->thr.p, thr.data(), thr.size() * 8, cudaMemcpyHostToDevice, c->st));
     CK(c, cudaStreamSynchronize(c->st));
+    c->thr_unit = c->unit;
     return CTB_OK;
   }
   const double dr = (c->rmax - c->rmin) / c->nbins;
@@ -337,6 +374,7 @@ int upload_thresholds(ctb_ctx* c) {
   CK(c, ensure(c, c->thr, thr.size() * 8));
   CK(c, cudaMemcpyAsync(c->thr.p, thr.data(), thr.size() * 8, cudaMemcpyHostToDevice, c->st));
   CK(c, cudaStreamSynchronize(c->st));
+  c->thr_unit = c->unit;
   return CTB_OK;
 }
 
@@ -519,8 +557,8 @@ int load_points(ctb_ctx* c, const double* xyz, const double* w, int64_t n) {
                       c->st));
   CK(c, launch_cell_start(ks, n, g.ncells, P<uint32_t>(c->cell_start), c->st));
   CK(c, cudaEventRecord(c->ev[2], c->st));
-  uint32_t fl[4] = {0, 0, 0, 0};
-  CK(c, cudaMemcpyAsync(fl, c->flags.p, sizeof(fl), cudaMemcpyDeviceToHost, c->st));
+  const uint32_t* fl = reinterpret_cast<const uint32_t*>(c->pin);
+  CK(c, cudaMemcpyAsync(c->pin, c->flags.p, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
   if (fl[0]) return fail(c, CTB_ERR_NONFINITE, "non-finite coordinate or weight");
   c->negw = fl[3] != 0;
@@ -684,6 +722,29 @@ int contract_piece(ctb_ctx* c, const PairPlan& pl, int64_t off, int64_t cnt, siz
   return CTB_OK;
 }
 
+// Wait for the chunk whose kernels were launched last and add up its stages'
+// times (events from c->ev[2]: [1] count end [2] fill end [3] accumulation end
+// [4] contraction end [5] pack end).
+cudaError_t close_chunk(ctb_ctx* c) {
+  if (!c->chunk_open) return cudaSuccess;
+  cudaEvent_t* ev = c->ev + 2;
+  const cudaError_t e = cudaEventSynchronize(ev[4]);
+  if (e != cudaSuccess) return e;
+  c->t_ms[6] += elapsed(ev[1], ev[2]);
+  c->t_ms[7] += elapsed(ev[2], ev[3]);
+  c->t_ms[2] = c->t_ms[6] + c->t_ms[7];
+  if (c->chunk_open == 2) {
+    c->t_ms[3] += elapsed(ev[3], ev[5]);
+    c->t_ms[4] += elapsed(ev[5], ev[4]);
+  } else {
+    c->t_ms[4] += elapsed(ev[3], ev[4]);
+  }
+  c->chunk_open = 0;
+  return cudaSuccess;
+}
+
+// Runs the pair pipeline.  The last chunk is left open (close_chunk): its
+// kernels may still run when this returns.
 int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, const PairPlan& pl,
               float* alm_dev_out, uint64_t* npairs_out, const std::vector<int64_t>* seg_end = nullptr) {
   const int nb = c->nbins;
@@ -692,7 +753,9 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   CK(c, ensure(c, c->scan_tmp2, scan_tmp_words((size_t)pl.chunk_max * nb) * 4));
   CK(c, ensure(c, c->M, (size_t)pl.chunk_max * nb * c->lay.row * sizeof(float)));
   CK(c, ensure(c, c->wprim, (size_t)pl.chunk_max * sizeof(float)));
-  CK(c, ensure(c, c->counters, 64));
+  // counters of a chunk: count's work, pairs, code bytes, fill's work, then one per m-pass
+  constexpr size_t kCounters = 4 + kLmaxCap + 1;
+  CK(c, ensure(c, c->counters, kCounters * 8));
   CK(c, ensure(c, c->code_base, (size_t)pl.chunk_max * row_blocks(c->g) * sizeof(unsigned long long)));
   unsigned long long* work = P<unsigned long long>(c->counters);
   unsigned long long* total = work + 1;
@@ -719,13 +782,14 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   aa.offsets = P<uint32_t>(c->offsets);
   aa.M = P<float>(c->M);
   aa.conv = P<uint8_t>(c->conv);
-  aa.work = work;
+  aa.work = work + 4;
   aa.nbins = nb;
   aa.row = c->lay.row;
   std::memcpy(aa.beta, c->beta, sizeof(aa.beta));
   for (int k = 0; k < 3; ++k) aa.sph_origin[k] = (float)c->origin[k];
   aa.sph_unit = (float)c->unit;
-  double t_stream = 0, t_alm = 0, t_con = 0, t_pack = 0;
+  for (int k : {2, 3, 4, 6, 7}) c->t_ms[k] = 0;
+  c->chunk_open = 0;
   uint64_t pairs = 0, chunks = 0;
   int64_t C = pl.chunk_first;
   double cand_per = pl.cand_first;  // code bytes per primary (estimate, then measured)
@@ -745,16 +809,17 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     CK(c, ensure(c, c->codes, codes_want));
     sa.codes = P<uint8_t>(c->codes);
     sa.code_cap = c->codes.bytes;
-    CK(c, cudaMemsetAsync(work, 0, 24, c->st));
+    CK(c, cudaMemsetAsync(work, 0, kCounters * 8, c->st));
     CK(c, cudaEventRecord(ev[0], c->st));
     sa.lists = nullptr;
+    sa.work = work;
     CK(c, launch_stream(sa, false, pl.count_blocks, c->st));
     CK(c, cudaEventRecord(ev[1], c->st));
-    unsigned long long tc[2] = {0, 0};  // pairs, candidates
-    CK(c, cudaMemcpyAsync(tc, total, sizeof(tc), cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaMemcpyAsync(c->pin, total, 16, cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
-    t_stream += elapsed(ev[0], ev[1]);
-    const unsigned long long tot = tc[0], ctot = tc[1];
+    c->t_ms[6] += elapsed(ev[0], ev[1]);
+    c->t_ms[2] = c->t_ms[6] + c->t_ms[7];
+    const unsigned long long tot = c->pin[0], ctot = c->pin[1];  // pairs, code bytes
     if (tot > pl.list_cap || ctot > pl.code_cap) {
       if (cnt > 1) {
         C = std::max<int64_t>(1, cnt / 2);
@@ -774,10 +839,9 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
                              P<uint32_t>(c->scan_tmp2), c->st));
     sa.lists = P<uint32_t>(c->lists);
     aa.lists = P<uint32_t>(c->lists);
-    CK(c, cudaMemsetAsync(work, 0, 8, c->st));
+    sa.work = work + 3;
     CK(c, launch_stream(sa, true, pl.stream_blocks, c->st));
     CK(c, cudaEventRecord(ev[2], c->st));
-    CK(c, cudaMemsetAsync(work, 0, 8, c->st));
     const int lists = lists_per_warp((double)tot / ((double)cnt * nb));
     if (c->sphere)
       CK(c, launch_am(aa, c->lmax, lists, pl.wpb, c->nsm, c->st));
@@ -809,15 +873,9 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
       CK(c, cudaGetLastError());
     }
     CK(c, cudaEventRecord(ev[4], c->st));
-    CK(c, cudaEventSynchronize(ev[4]));
-    t_stream += elapsed(ev[1], ev[2]);
-    t_alm += elapsed(ev[2], ev[3]);
-    if (contract && c->precision != CTB_PREC_FP32 && !seg_end) {
-      t_pack += elapsed(ev[3], ev[5]);
-      t_con += elapsed(ev[5], ev[4]);
-    } else {
-      t_con += elapsed(ev[3], ev[4]);
-    }
+    c->chunk_open = contract && c->precision != CTB_PREC_FP32 && !seg_end ? 2 : 1;
+    // the caller waits for the last chunk with its own results
+    if (c0 + cnt < np) CK(c, close_chunk(c));
     pairs += tot;
     ++chunks;
     c0 += cnt;
@@ -857,11 +915,6 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     }
     C = std::max<int64_t>(1, std::min<int64_t>((int64_t)nxt, pl.chunk_max));
   }
-  c->t_ms[2] = t_stream + t_alm;
-  c->t_ms[3] = t_pack;
-  c->t_ms[4] = t_con;
-  c->t_ms[6] = t_stream;
-  c->t_ms[7] = t_alm;
   c->nchunks = chunks;
   *npairs_out = pairs;
   return CTB_OK;
@@ -907,6 +960,7 @@ int compute_impl(ctb_ctx* c, const uint32_t* dprim, int64_t np, double* zeta_out
   unsigned int tc_err = 0;
   if (tc) CK(c, cudaMemcpyAsync(&tc_err, P<unsigned int>(c->flags) + 1, 4, cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
+  CK(c, close_chunk(c));
   c->npairs = pairs;
   c->t_ms[5] = elapsed(c->ev[evs], c->ev[evs + 1]);
   if (tc_err) return fail(c, CTB_ERR_TIMEOUT, "tensor-core contraction: a bounded wait timed out");
@@ -1060,6 +1114,7 @@ int batch_impl(ctb_ctx* c, const double* const* xyz, const double* const* w, con
   unsigned int tc_err = 0;
   if (tc) CK(c, cudaMemcpyAsync(&tc_err, P<unsigned int>(c->flags) + 1, 4, cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
+  CK(c, close_chunk(c));
   c->npairs = pairs;
   c->t_ms[0] = t_ingest;
   c->t_ms[1] = t_sort;
@@ -1253,6 +1308,7 @@ int autotune_grid(ctb_ctx* c, const double* xyz, const double* w, int64_t n) {
     for (int rep = 0; rep < 2; ++rep) {
       r = run_pairs(c, P<uint32_t>(c->prim), m, false, pl, nullptr, &pairs);
       if (r) return r;
+      CK(c, close_chunk(c));
     }
     const float ms = (float)(c->t_ms[6] + c->t_ms[7]);
     if (ms < best_ms) {
@@ -1336,6 +1392,7 @@ void ctb_destroy(ctb_ctx* c) {
   cudaStreamSynchronize(c->st);
   if (c->ev_ready)
     for (auto& e : c->ev) cudaEventDestroy(e);
+  if (c->pin) cudaFreeHost(c->pin);
   cudaGetLastError();
   delete c;
 }
@@ -1415,6 +1472,7 @@ int ctb_get_alm(ctb_ctx* c, const int64_t* primary_idx, int64_t m, float* alm_ou
   if (r) return r;
   if (!dev_out) CK(c, cudaMemcpyAsync(alm_out, dst, outsz * 4, cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
+  CK(c, close_chunk(c));
   c->npairs = pairs;
   return CTB_OK;
 }

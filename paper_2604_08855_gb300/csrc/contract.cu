@@ -416,15 +416,10 @@ static const void* con_kernel(const ConShape& sh, int row, bool aligned) {
 int contract_fp32_blocks_per_sm(int nbins, int row) {
   const ConShape sh = con_shape(nbins, row);
   if ((size_t)sh.smem_bytes > kConSmemCap) return 0;
-  int least = 1 << 30;
-  for (int al = 0; al < 2; ++al) {
-    const void* fn = con_kernel(sh, row, al != 0);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem_bytes) != cudaSuccess) return 0;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, sh.threads, sh.smem_bytes) != cudaSuccess) return 0;
-    if (nb < least) least = nb;
-  }
-  return least;
+  // (the copies of an aligned and of an unaligned base are two kernels)
+  const int x = resident_blocks(con_kernel(sh, row, false), sh.threads, sh.smem_bytes);
+  const int y = resident_blocks(con_kernel(sh, row, true), sh.threads, sh.smem_bytes);
+  return x < y ? x : y;
 }
 
 cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t st) {
@@ -432,12 +427,11 @@ cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t
   const ConShape sh = con_shape(a.nbins, a.row);
   if ((size_t)sh.smem_bytes > kConSmemCap) return cudaErrorInvalidValue;
   const void* fn = con_kernel(sh, a.row, (reinterpret_cast<uintptr_t>(a.M) & 15) == 0);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem_bytes);
-  if (e != cudaSuccess) return e;
+  if (resident_blocks(fn, sh.threads, sh.smem_bytes) < 1) return cudaErrorInvalidConfiguration;
   ContractArgs ca = a;
   ConShape cs = sh;
   void* args[] = {&ca, &cs};
-  e = cudaLaunchKernel(fn, dim3(nparts, (sh.ntiles + sh.tiles - 1) / sh.tiles), dim3(sh.threads), args,
+  const cudaError_t e = cudaLaunchKernel(fn, dim3(nparts, (sh.ntiles + sh.tiles - 1) / sh.tiles), dim3(sh.threads), args,
                        (size_t)sh.smem_bytes, st);
   if (e != cudaSuccess) return e;
   ++g_launches;

@@ -214,6 +214,11 @@ struct Layout {
 };
 void make_layout(int L, Layout* out);
 
+// Resident blocks per SM of a kernel at this block size and dynamic shared
+// memory (0: it cannot run), its shared-memory limit raised to that.  Both are
+// facts of the kernel and the device, asked once for each (about 3 us a call).
+int resident_blocks(const void* fn, int threads, size_t smem);
+
 // kernels launched by this host thread (every launcher adds its launches)
 extern thread_local unsigned long long g_launches;
 
@@ -329,7 +334,7 @@ struct AlmArgs {
   const uint32_t* lists;
   float* M;                       // [prim_count][nbins][row]
   const uint8_t* conv;            // flush conversion tables, pass p at conv_pass_offset(L, p)
-  unsigned long long* work;
+  unsigned long long* work;       // one zeroed work counter per m-pass
   int nbins;
   int row;
   float sph_origin[3];            // sphere mode: the points' position = origin + unit * (x, y, z)

@@ -763,16 +763,11 @@ constexpr size_t alm_smem(int wpb) {
 
 template <int L, int P, int S>
 int alm_occupancy_pass(int wpb) {
-  const size_t smem = alm_smem<L, P, S>(wpb);
-  if (cudaFuncSetAttribute(k_alm<L, P, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_alm<L, P, S>, wpb * 32, smem) != cudaSuccess) return 0;
-  return nb;
+  return resident_blocks((const void*)k_alm<L, P, S>, wpb * 32, alm_smem<L, P, S>(wpb));
 }
 
-// passes P.. of kernel L: each launch resident-sized from its own occupancy,
-// the work counter zeroed before every pass after the first
+// passes P.. of kernel L: each launch resident-sized from its own occupancy
+// and with a work counter of its own (a.work, the next pass's after it)
 template <int L, int P, int S>
 cudaError_t launch_passes(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
   if constexpr (P >= pass_count(L)) {
@@ -780,16 +775,13 @@ cudaError_t launch_passes(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
   } else {
     const int bps = alm_occupancy_pass<L, P, S>(wpb);
     if (bps < 1) return cudaErrorInvalidConfiguration;
-    cudaError_t e;
-    if (P > 0) {
-      e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), st);
-      if (e != cudaSuccess) return e;
-    }
     k_alm<L, P, S><<<bps * nsm, wpb * 32, alm_smem<L, P, S>(wpb), st>>>(a);
     ++g_launches;
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_passes<L, P + 1, S>(a, wpb, nsm, st);
+    AlmArgs next = a;
+    ++next.work;
+    return launch_passes<L, P + 1, S>(next, wpb, nsm, st);
   }
 }
 

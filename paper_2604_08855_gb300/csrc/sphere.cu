@@ -119,11 +119,7 @@ static constexpr size_t am_smem(int wpb) {
 
 template <int K, int S>
 static int am_occupancy_K(int wpb) {
-  const size_t smem = am_smem<K, S>(wpb);
-  if (cudaFuncSetAttribute(k_am<K, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_am<K, S>, wpb * 32, smem) != cudaSuccess) return 0;
-  return nb;
+  return resident_blocks((const void*)k_am<K, S>, wpb * 32, am_smem<K, S>(wpb));
 }
 
 template <int K, int S>

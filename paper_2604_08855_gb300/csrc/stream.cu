@@ -565,11 +565,7 @@ static const void* stream_fn(const Geom& g, bool fill) {
 }
 
 int stream_blocks_per_sm(const Geom& g, bool fill) {
-  int nb = 0;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, stream_fn(g, fill), kStreamThreads, stream_smem(g.nbins)) ==
-                 cudaSuccess
-             ? nb
-             : 0;
+  return resident_blocks(stream_fn(g, fill), kStreamThreads, stream_smem(g.nbins));
 }
 
 cudaError_t launch_stream(const StreamArgs& a, bool fill, int nblocks, cudaStream_t st) {
