@@ -89,7 +89,6 @@ struct ctb_ctx {
   double bbox_volume = 0;
   Layout lay{};
   int Lk = 0;
-  float beta[(kLmaxCap + 1) * (kLmaxCap + 1)];
   bool tables_ready = false;
   double thr_unit = 0;  // unit of the uploaded thresholds (0: none)
   uint64_t* pin = nullptr;  // pinned words that counters and flags are read back into
@@ -238,7 +237,6 @@ int ensure_tables(ctb_ctx* c) {
   if (c->sphere) return ensure_tables_sphere(c);
   c->Lk = lmax_kernel(c->lmax);
   make_layout(c->Lk, &c->lay);
-  fill_beta(c->beta);
   std::vector<float> norm(c->lay.row, 0.f);
   for (int l = 0; l <= c->Lk; ++l)
     for (int m = -l; m <= l; ++m) norm[c->lay.slot[l * l + l + m]] = (float)norm_lm(l, m);
@@ -785,7 +783,6 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   aa.work = work + 4;
   aa.nbins = nb;
   aa.row = c->lay.row;
-  std::memcpy(aa.beta, c->beta, sizeof(aa.beta));
   for (int k = 0; k < 3; ++k) aa.sph_origin[k] = (float)c->origin[k];
   aa.sph_unit = (float)c->unit;
   for (int k : {2, 3, 4, 6, 7}) c->t_ms[k] = 0;

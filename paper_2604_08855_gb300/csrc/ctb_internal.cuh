@@ -89,11 +89,11 @@ __host__ __device__ inline int row_blocks(const Geom& g) {
 //
 // The pair kernel accumulates the (l, m) coefficients in passes over m ranges
 // [m0, m1] (one pass when ell_max <= 10).  Each pass accumulates moments of
-// its columns in one polynomial basis q_k(z), k = 0..L - m0: the Chebyshev
-// T_k for the pass that starts at m = 0, and the monic recurrence
-// polynomials of its first column, p^{m0}_{m0+k}, for the others.  Moment k
-// of column m, sum_j w_j (x+iy)^m q_k(z_j), sits in the slot of (m + k, +-m);
-// the flush turns moments into normalised a_lm by a fixed linear map.
+// its columns in one polynomial basis q_k(z) = U_k(z / s), k = 0..L - m0, the
+// Chebyshev polynomials of the second kind scaled to the range of z that
+// (1 - z^2)^{m0/2} leaves.  Moment k of column m, sum_j w_j (x+iy)^m q_k(z_j),
+// sits in the slot of (m + k, +-m); the flush turns moments into normalised
+// a_lm by a fixed linear map.
 //
 // Slots of a pass: first the (+m, -m) pairs, for l = max(m0,1)..L and
 // m = max(m0,1)..min(l, m1), each pair on an even slot (+m) and the odd slot
@@ -108,11 +108,17 @@ __host__ __device__ constexpr int coef_count(int L, int m0, int m1) {
   return s;
 }
 
-// Largest l_max whose whole coefficient set is one pass (Chebyshev basis).
+// Largest l_max whose whole coefficient set is one pass.
 constexpr int kSinglePassLmax = 10;
-// Columns of the first pass when l_max > kSinglePassLmax: the Chebyshev
-// moments lose float32 accuracy as m grows, so this pass stops at m = 2.
+// Columns of the first pass when l_max > kSinglePassLmax: its basis (s = 1)
+// suits small m, and with three columns it runs 12 warps per SM.
 constexpr int kFirstPassM1 = 2;
+
+// 2 / s of the basis of the pass that starts at column m0.  s = 1 - 0.041 m0
+// lies within 0.03 of the value that amplifies rounding least for the passes
+// [3, 7] and [8, 20] of l_max 20 (0.88 and 0.67), and amplifies at most 10.5
+// times in every pass of l_max 11 to 20.
+__host__ __device__ constexpr float basis_scale(int m0) { return (float)(2.0 / (1.0 - 0.041 * m0)); }
 
 // end column of the pass starting at m0 when every further pass holds at
 // most `cap` coefficients
@@ -227,8 +233,7 @@ extern thread_local unsigned long long g_launches;
 // beyond `edge` exactly when T >= threshold.
 unsigned long long sq_threshold(double edge, double unit);
 
-// recurrence constants (pair_dispatch.cu)
-void fill_beta(float* beta);   // beta_lm at [l*(kLmaxCap+1)+m]
+// normalisation (pair_dispatch.cu)
 double norm_lm(int l, int m);  // C_lm of the real orthonormal Y_l,m
 // flush conversion tables of kernel L, pass after pass: accumulator totals ->
 // normalised a_lm (entries padded per pass to conv_entries(L, m0_p), entry-
@@ -339,7 +344,6 @@ struct AlmArgs {
   int row;
   float sph_origin[3];            // sphere mode: the points' position = origin + unit * (x, y, z)
   float sph_unit;
-  float beta[(kLmaxCap + 1) * (kLmaxCap + 1)];  // recurrence beta_lm at [l*(kLmaxCap+1)+m]
 };
 int alm_blocks_per_sm(int lmax_kernel, int warps_per_block);
 // sphere.cu: projected multipoles m = 0..mmax (mmax <= CTB_MMAX_CAP)

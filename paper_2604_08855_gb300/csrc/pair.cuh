@@ -8,32 +8,36 @@
 // histograms, with a per-multipole recurrence cost.
 //
 // GB300 design.  The neighbour lists of a primary are grouped by bin
-// (stream.cu).  One warp owns one primary: for each of its (primary, bin)
-// lists each lane takes one neighbour per step, evaluates polynomial moments
-// of the direction by recurrences in float32 registers and accumulates them
-// (one paired FMA per (+m, -m) pair of moments).  Up to l_max 10 one kernel
-// holds all coefficients; above, the m columns are split into passes of at
-// most kPassCap accumulators, each its own kernel and launch (see k_alm).  At
-// the end of the list the 32 lanes' accumulators are summed through a
-// shared-memory transpose, mapped to normalised a_lm and stored as the
-// (primary, bin) row of M.
-// Each list is one run, so the cross-lane reduction happens once per
-// (primary, bin), and the first loads of the next list are issued while the
-// current one is still being accumulated.
+// (stream.cu).  One warp owns one primary and takes its (primary, bin) lists
+// one at a time (long lists) or two or four side by side, 32, 16 or 8 lanes a
+// list (short ones): each lane takes one neighbour per step, evaluates
+// polynomial moments of the direction by recurrences in float32 registers and
+// accumulates them (one paired FMA per (+m, -m) pair of moments).  Up to
+// l_max 10 one kernel holds all coefficients; above, the m columns are split
+// into passes of at most kPassCap accumulators, each its own kernel and
+// launch (see k_alm).  At the end of the list its lanes' accumulators are
+// summed through a shared-memory transpose, mapped to normalised a_lm and
+// stored as the (primary, bin) row of M.  The cross-lane reduction happens
+// once per list, and the first loads of the next lists are issued while the
+// current ones are still being accumulated.
 //
 // Moments (real Y_lm up to a fixed linear map per (l, m), applied at the flush):
 //   (c_m + i s_m) = w (x + i y)^m        one paired FMUL + FFMA per m
-//   q_k(z)        = the pass's basis: Chebyshev T_k (T_0 = 1, T_1 = z,
-//                   T_k = 2z T_{k-1} - T_{k-2}: one FMA per degree) for the
-//                   pass that starts at m = 0, else the monic recurrence
-//                   polynomials of the pass's first column m0 (q_0 = 1,
-//                   q_1 = z, q_k = z q_{k-1} - beta q_{k-2}: two per degree)
+//   q_k(z)        = the pass's basis, U_k(z / s): Chebyshev polynomials of the
+//                   second kind, scaled (q_0 = 1, q_1 = t, q_k = t q_{k-1} -
+//                   q_{k-2}, t = 2 z / s: one FMA per degree)
 //   S_{m,k}      += q_k (c_m, s_m)       one paired FFMA per (k, +-m)
 // The (1 - z^2)^{m/2} factor of the associated Legendre function is absorbed
-// in (x + i y)^m.  Blackwell's paired FP32 instructions (FFMA2 / FMUL2 /
-// FADD2) update the (+m, -m) accumulator pair in one issue slot; in a stream
-// of independent accumulations they reach about 1.5x the FMA throughput of
-// scalar FFMA on this part.
+// in (x + i y)^m, and it keeps |z| small where m is large: so the pass that
+// starts at column m0 takes s < 1 (basis_scale), which makes its polynomials
+// nearly orthogonal under that factor.  The flush's map then amplifies
+// rounding by at most 10 (rms over z; l_max 10: 9, l_max 20: 6, 11 and 7 in
+// the three passes).  T_k(z) for the first pass and the monic recurrence of
+// column m0 for the others, the bases before these, amplified by up to 39 at
+// l_max 10 and 64 at l_max 20 and took two instructions a degree above m = 2.
+// Blackwell's paired FP32 instructions (FFMA2 / FMUL2 / FADD2) update the
+// (+m, -m) accumulator pair in one issue slot; a stream of them takes 2.65
+// cycles each against 1.65 for a scalar FFMA, 1.25 times the FMA rate.
 #pragma once
 
 #include <type_traits>
@@ -94,21 +98,12 @@ __device__ __forceinline__ void columns(float2* acc, const float* Q, float2 xy, 
   }
 }
 
-// T_k(z), k = K..KMAX, by T_k = 2z T_{k-1} - T_{k-2}: one FMA per degree.
+// q_k, k = K..KMAX: q_k = t q_{k-1} - q_{k-2}.
 template <int K, int KMAX>
-__device__ __forceinline__ void cheb_seq(float* T, float z2) {
+__device__ __forceinline__ void basis_seq(float* Q, float t) {
   if constexpr (K <= KMAX) {
-    T[K] = fmaf(z2, T[K - 1], -T[K - 2]);
-    cheb_seq<K + 1, KMAX>(T, z2);
-  }
-}
-
-// q_k = p^{M0}_{M0+k}(z), k = K..KMAX: q_k = z q_{k-1} - beta_{M0+k, M0} q_{k-2}.
-template <int M0, int K, int KMAX>
-__device__ __forceinline__ void basis_seq(const AlmArgs& a, float* Q, float z) {
-  if constexpr (K <= KMAX) {
-    Q[K] = fmaf(z, Q[K - 1], -(a.beta[(M0 + K) * (kLmaxCap + 1) + M0] * Q[K - 2]));
-    basis_seq<M0, K + 1, KMAX>(a, Q, z);
+    Q[K] = fmaf(t, Q[K - 1], -Q[K - 2]);
+    basis_seq<K + 1, KMAX>(Q, t);
   }
 }
 
@@ -138,14 +133,12 @@ __device__ __forceinline__ void cpow(float x, float y, float& r, float& i) {
 // time (against all L - m0 + 1 in column-major order), which keeps the wide
 // passes of l_max 20 within their register budget.
 template <int L, int M0, int M1, int K, int KMAX, int MS, int ME>
-__device__ __forceinline__ void degrees(const AlmArgs& a, float2* acc, const float2* cs, float w, float z, float z2,
-                                        float q2, float q1) {
+__device__ __forceinline__ void degrees(float2* acc, const float2* cs, float w, float t, float q2, float q1) {
   if constexpr (K <= KMAX) {
     float q;
     if constexpr (K == 0) q = 1.f;
-    else if constexpr (K == 1) q = z;
-    else if constexpr (M0 == 0) q = fmaf(z2, q1, -q2);
-    else q = fmaf(z, q1, -(a.beta[(M0 + K) * (kLmaxCap + 1) + M0] * q2));
+    else if constexpr (K == 1) q = t;
+    else q = fmaf(t, q1, -q2);
     if constexpr (M0 == 0) {
       float& c0 = slot_ref<local_slot(L, K, 0, M0, M1)>(acc);
       c0 = K == 0 ? c0 + w : fmaf(w, q, c0);
@@ -158,7 +151,7 @@ __device__ __forceinline__ void degrees(const AlmArgs& a, float2* acc, const flo
         else acc[i] = __ffma2_rn(make_float2(q, q), cs[m - MS], acc[i]);
       }
     }
-    degrees<L, M0, M1, K + 1, KMAX, MS, ME>(a, acc, cs, w, z, z2, q1, q);
+    degrees<L, M0, M1, K + 1, KMAX, MS, ME>(acc, cs, w, t, q1, q);
   }
 }
 
@@ -169,9 +162,10 @@ __host__ __device__ constexpr bool degree_major(int L, int m0, int m1) {
 
 // Add one neighbour (weight w, unit direction x, y, z) to the pass's
 // accumulators: the pass's basis sequence, the complex powers, and one
-// paired FMA per (k, +-m) moment (one FMA per moment of column 0).
+// paired FMA per (k, +-m) moment (one FMA per moment of column 0).  The
+// caller passes t = basis_scale(M0) z, the only form z appears in.
 template <int L, int M0, int M1>
-__device__ __forceinline__ void accum_pass(const AlmArgs& a, float2* acc, float w, float x, float y, float z) {
+__device__ __forceinline__ void accum_pass(float2* acc, float w, float x, float y, float t) {
   constexpr int KMAX = L - M0;  // highest basis degree this pass needs
   constexpr int MS = M0 < 1 ? 1 : M0;
   constexpr int ME = M1 < L ? M1 : L;
@@ -187,13 +181,12 @@ __device__ __forceinline__ void accum_pass(const AlmArgs& a, float2* acc, float 
       for (int c = 1; c < NC; ++c)
         cs[c] = __ffma2_rn(make_float2(cs[c - 1].x, cs[c - 1].x), xy, __fmul2_rn(make_float2(cs[c - 1].y, cs[c - 1].y), myx));
     }
-    degrees<L, M0, M1, 0, KMAX, MS, ME>(a, acc, cs, w, z, z + z, 0.f, 0.f);
+    degrees<L, M0, M1, 0, KMAX, MS, ME>(acc, cs, w, t, 0.f, 0.f);
   } else {
     float Q[KMAX + 1 > 2 ? KMAX + 1 : 2];
     Q[0] = 1.f;
-    Q[1] = z;
-    if constexpr (M0 == 0) cheb_seq<2, KMAX>(Q, z + z);
-    else basis_seq<M0, 2, KMAX>(a, Q, z);
+    Q[1] = t;
+    basis_seq<2, KMAX>(Q, t);
     if constexpr (M0 == 0) column_zero<L, M0, M1, 0>(acc, Q, w);
     if constexpr (MS <= ME) {
       float pr, pi;
@@ -333,6 +326,18 @@ __device__ __forceinline__ uint32_t rec_at(const uint32_t* __restrict__ lists, R
   return k < nxt.n ? __ldcs(lists + nxt.off + k) : kNone;
 }
 
+// The points' base, as a register pair in k_alm.  Its arguments stay in
+// constant memory (__grid_constant__), which suits every pointer but this
+// one, used once a step to address the gather: against arguments that the
+// compiler may copy, at l_max 10 with one list a warp (3.36e10 pairs) 219.5
+// ms with this base in registers, 222.2 without, 225.6 with all of them
+// copied; two lists a warp (1.51e10 pairs) 108.5, 111.9 and 108.3.
+template <class Step>
+__device__ __forceinline__ const uint4* points_base(const uint4* p) {
+  if constexpr (Step::kPtsInRegs) asm volatile("" : "+l"(p));
+  return p;
+}
+
 __device__ __forceinline__ uint4 gather(const uint4* __restrict__ pts, uint32_t j, uint4 P) {
   return j != kNone ? __ldg(pts + j) : P;
 }
@@ -358,16 +363,15 @@ struct Step3D {
   // Each launch runs one m-pass, so the full-lane copy of the step and the
   // general one are the only code in the instruction cache.
   static constexpr bool kFullLaneLoop = true;
+  static constexpr bool kPtsInRegs = true;
   // flush conversion entries per unit: moment degrees of the same parity, and
   // how many the units of one round of 32 need (they are sorted by degree)
   static constexpr int kConvE = conv_entries(L, M0);
   static constexpr int conv_round(int r) { return conv_round_entries(L, M0, M1, r); }
-  const AlmArgs& a;
   __device__ __forceinline__ void operator()(float2* acc, float w, float dx, float dy, float dz) const {
-    const float ir = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-    accum_pass<L, M0, M1>(a, acc, w, dx * ir, dy * ir, dz * ir);
+    accum(acc, unit(w, dx, dy, dz));
   }
-  // The unit direction and weight of a neighbour, ahead of its
+  // The unit direction (x, y, basis_scale z) and weight of a neighbour, ahead of its
   // accumulation.  The full-lane loop of a single-pass kernel (l_max <= 10)
   // prepares each step's direction one iteration ahead (5 % faster at
   // l_max 10); in the 255-register passes of l_max 20 the extra live state
@@ -380,9 +384,9 @@ struct Step3D {
   }
   __device__ __forceinline__ float4 unit(float w, float dx, float dy, float dz) const {
     const float ir = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-    return make_float4(dx * ir, dy * ir, dz * ir, w);
+    return make_float4(dx * ir, dy * ir, dz * (ir * basis_scale(M0)), w);
   }
-  __device__ __forceinline__ void accum(float2* acc, float4 s) const { accum_pass<L, M0, M1>(a, acc, s.w, s.x, s.y, s.z); }
+  __device__ __forceinline__ void accum(float2* acc, float4 s) const { accum_pass<L, M0, M1>(acc, s.w, s.x, s.y, s.z); }
   static constexpr bool kPrep = L <= kSinglePassLmax;
 };
 
@@ -421,7 +425,7 @@ __device__ __forceinline__ void run_steps(const AlmArgs& a, const Step& step, Ru
                                           int lane, uint32_t pe) {
   constexpr int NCP = Step::NCP;
   const uint32_t* __restrict__ lists = a.lists;
-  const uint4* __restrict__ pts = a.pts;
+  const uint4* pts = points_base<Step>(a.pts);
   float2 acc[NCP / 2];
 #pragma unroll
   for (int i = 0; i < NCP / 2; ++i) acc[i] = make_float2(0.f, 0.f);
@@ -559,6 +563,7 @@ __device__ __forceinline__ void run_groups(const AlmArgs& a, const Step& step, c
                                            const uint32_t* s_n, const uint4 P, float* __restrict__ rows,
                                            const float2* ctab, float* sbuf, int lane) {
   constexpr uint32_t G = 32 / S;
+  const uint4* pts = points_base<Step>(a.pts);
   constexpr int NCP = Step::NCP;
   const int nbins = a.nbins;
   const int ls = lane / (int)G;
@@ -604,7 +609,7 @@ __device__ __forceinline__ void run_groups(const AlmArgs& a, const Step& step, c
     return j;
   };
   uint32_t j0 = word(), j1 = word(), j2 = word();
-  uint4 q0 = gather(a.pts, j0, P), q1 = gather(a.pts, j1, P);
+  uint4 q0 = gather(pts, j0, P), q1 = gather(pts, j1, P);
   auto sep = [&](uint4 q, bool valid, float& w, float& dx, float& dy, float& dz) {
     dx = valid ? __int2float_rn((int)(q.x - P.x)) : 1.f;  // an idle lane holds q = P
     dy = __int2float_rn((int)(q.y - P.y));
@@ -627,7 +632,7 @@ __device__ __forceinline__ void run_groups(const AlmArgs& a, const Step& step, c
       if constexpr (use_prep<Step>()) {
         sep(q1, j1 != kNone, w, dx, dy, dz);
         const float4 Dn = step.unit(w, dx, dy, dz);
-        q1 = gather(a.pts, j2, P);
+        q1 = gather(pts, j2, P);
         j1 = j2;
         j2 = word();
         step.accum(acc, D);
@@ -636,7 +641,7 @@ __device__ __forceinline__ void run_groups(const AlmArgs& a, const Step& step, c
         sep(q0, j0 != kNone, w, dx, dy, dz);
         q0 = q1;
         j0 = j1;
-        q1 = gather(a.pts, j2, P);
+        q1 = gather(pts, j2, P);
         j1 = j2;
         j2 = word();
         step(acc, w, dx, dy, dz);
@@ -725,7 +730,7 @@ __device__ __forceinline__ void load_lists(const AlmArgs& a, uint64_t ib, uint32
 // register budget (a pass with fewer accumulators runs more warps per SM).
 // The lists are re-read once per pass; the points stay in L2.
 template <int L, int P, int S>
-__global__ void __launch_bounds__(128, alm_min_blocks(pass_ncp(L, P))) k_alm(AlmArgs a) {
+__global__ void __launch_bounds__(128, alm_min_blocks(pass_ncp(L, P))) k_alm(const __grid_constant__ AlmArgs a) {
   constexpr int M0 = pass_m0(L, P), M1 = pass_m1(L, P), NCP = pass_ncp(L, P), BASE = pass_base(L, P);
   constexpr int TB = (int)conv_bytes(L, P);
   extern __shared__ __align__(16) char s_alm[];
@@ -750,7 +755,7 @@ __global__ void __launch_bounds__(128, alm_min_blocks(pass_ncp(L, P))) k_alm(Alm
     const int64_t gi = a.prim_begin + (int64_t)i;
     const uint32_t sp = a.prim ? __ldg(a.prim + gi) : (uint32_t)gi;
     const uint4 Pt = __ldg(a.pts + sp);
-    run_primary<Step3D<L, M0, M1>, S>(a, Step3D<L, M0, M1>{a}, s_off, s_n, Pt, a.M + ib * (uint64_t)a.row + BASE, ctab,
+    run_primary<Step3D<L, M0, M1>, S>(a, Step3D<L, M0, M1>{}, s_off, s_n, Pt, a.M + ib * (uint64_t)a.row + BASE, ctab,
                                       sbuf, lane);
     __syncwarp();  // s_n / s_off are rewritten for the next primary
   }

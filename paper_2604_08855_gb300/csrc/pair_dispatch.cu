@@ -50,13 +50,6 @@ static double rec_b(int l, int m) {
   return std::sqrt((((double)(l - 1) * (l - 1)) - (double)m * m) / (4.0 * (l - 1) * (l - 1) - 1.0));
 }
 
-// Monic form p_l = z p_{l-1} - beta p_{l-2}:  beta_lm = b_lm / a_{l-1,m}.
-void fill_beta(float* beta) {
-  for (int i = 0; i < (kLmaxCap + 1) * (kLmaxCap + 1); ++i) beta[i] = 0.f;
-  for (int m = 0; m <= kLmaxCap; ++m)
-    for (int l = m + 2; l <= kLmaxCap; ++l) beta[l * (kLmaxCap + 1) + m] = (float)(rec_b(l, m) / rec_a(l - 1, m));
-}
-
 // Normalisation C_lm turning the monic p_l^m times Re/Im (x+iy)^m into the
 // real orthonormal Y_l,+-m (Condon-Shortley phase and sqrt 2 for m != 0):
 //   C_mm = (-1)^m / sqrt(4 pi) prod_{k=1..m} sqrt((2k+1)/(2k)),
@@ -98,15 +91,35 @@ static std::vector<double> monic_in_T(int l, int m) {
   return std::vector<double>(p1.begin(), p1.begin() + n + 1);
 }
 
-// Coefficients D of p^m_l in the basis q_k = p^{m0}_{m0+k} (k <= l - m):
-// p^m_l = sum_k D_k q_k, by back substitution on the T-basis coefficients
-// (q_k has degree k with a nonzero T_k coefficient).
+// T-basis coefficients of the basis of the pass that starts at column m0:
+// q_0 = 1, q_1 = c z, q_k = c z q_{k-1} - q_{k-2} with c the device's float
+// constant.
+static std::vector<std::vector<double>> pass_basis(int n, int m0) {
+  const double c = (double)basis_scale(m0);
+  std::vector<std::vector<double>> q(n + 1, std::vector<double>(n + 1, 0.0));
+  q[0][0] = 1.0;
+  for (int k = 1; k <= n; ++k) {
+    for (int j = 0; j < k; ++j) {
+      if (j == 0) {
+        q[k][1] += c * q[k - 1][0];
+      } else {
+        q[k][j + 1] += 0.5 * c * q[k - 1][j];
+        q[k][j - 1] += 0.5 * c * q[k - 1][j];
+      }
+    }
+    if (k >= 2)
+      for (int j = 0; j <= k - 2; ++j) q[k][j] -= q[k - 2][j];
+  }
+  return q;
+}
+
+// Coefficients D of p^m_l in that basis: p^m_l = sum_k D_k q_k, by back
+// substitution on the T-basis coefficients (q_k has degree k with a nonzero
+// T_k coefficient).
 static std::vector<double> monic_in_basis(int l, int m, int m0) {
   const int n = l - m;
-  const std::vector<double> target = monic_in_T(l, m);
-  std::vector<std::vector<double>> q(n + 1);
-  for (int k = 0; k <= n; ++k) q[k] = monic_in_T(m0 + k, m0);
-  std::vector<double> r(target), d(n + 1, 0.0);
+  const std::vector<std::vector<double>> q = pass_basis(n, m0);
+  std::vector<double> r = monic_in_T(l, m), d(n + 1, 0.0);
   for (int k = n; k >= 0; --k) {
     d[k] = r[k] / q[k][k];
     for (int j = 0; j <= k; ++j) r[j] -= d[k] * q[k][j];
@@ -115,8 +128,7 @@ static std::vector<double> monic_in_basis(int l, int m, int m0) {
 }
 
 // Each pass accumulates moments S_{m,k} = sum w c_m q_k(z) of its columns in
-// slot (m + k, +-m), q_k its basis: the Chebyshev T_k for the pass that
-// starts at m = 0, else p^{m0}_{m0+k}.  Normalised a_lm = C_lm sum_k D_k S_{m,k},
+// slot (m + k, +-m), q_k its basis.  Normalised a_lm = C_lm sum_k D_k S_{m,k},
 // D the coefficients of p^m_l in that basis.
 bool make_conversion(const Layout& lay, std::vector<uint8_t>& tab) {
   const int L = lay.L;
@@ -129,7 +141,7 @@ bool make_conversion(const Layout& lay, std::vector<uint8_t>& tab) {
     const int m0 = lay.m0[p];
     for (int am = m0; am <= lay.m1[p] && am <= L; ++am) {
       for (int l = am; l <= L; ++l) {
-        const std::vector<double> d = m0 == 0 ? monic_in_T(l, am) : monic_in_basis(l, am, m0);
+        const std::vector<double> d = monic_in_basis(l, am, m0);
         const int s = lay.slot[l * l + l + am];
         std::vector<Ent>& v = ent[s / 2];
         // degrees of the polynomial's parity, from the highest (the others

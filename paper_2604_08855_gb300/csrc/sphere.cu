@@ -26,6 +26,7 @@ template <int K>
 struct StepSphere {
   static constexpr int NCP = round32(2 * K + 1);
   static constexpr bool kFullLaneLoop = true;
+  static constexpr bool kPtsInRegs = false;
   static constexpr int kConvE = 0;  // the row holds a_m itself: no conversion
   float ex, ey;      // east unit vector (its z component is zero)
   float nx, ny, nz;  // north unit vector
