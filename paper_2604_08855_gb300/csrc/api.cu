@@ -384,18 +384,21 @@ void finish_geom(ctb_ctx* c, Geom& g, uint32_t nc) {
   g.ncx = nc * xs;
   g.ncells = nc * nc * g.ncx;
   const double rmin_u = c->rmin / c->unit, rmax_u = c->rmax / c->unit;
-  // the float pre-filter; never 0, so that it also rejects r = 0
-  g.rlo2_u = std::max((float)(rmin_u * rmin_u * (1.0 - 1e-5)), 0.25f);
-  g.rhi2_u = (float)(rmax_u * rmax_u * (1.0 + 1e-5));
+  // the float pre-filter, 1e-6 wide of the edges (the float r^2 is good to
+  // 3e-7); never 0, so that it also rejects r = 0
+  g.rlo2_u = std::max((float)(rmin_u * rmin_u * (1.0 - 1e-6)), 0.25f);
+  g.rhi2_u = (float)(rmax_u * rmax_u * (1.0 + 1e-6));
   // Bin coordinate minus 1/2: r inv_dr + bin_shift.  Its float error (r to 5
   // ulp from conversions, r^2, rsqrt and product; scale and shift to one ulp
-  // each) stays below 8e-7 of r_max in bins, and 1e-4 of a bin covers r_max up
-  // to 125 bins wide.  On the sphere the coordinate is the angle's, with its
-  // own guard beside this one.
+  // each) stays below 8e-7 of r_max in bins; a pair that the pre-filter lets
+  // through lies at most 7e-7 of r_max past the first or last edge, so with
+  // 1.5e-6 of r_max as the margin it is within it, never a bin too far.  1e-4
+  // of a bin covers r_max up to 66 bins wide.  On the sphere the coordinate is
+  // the angle's, with its own guard (1e-5 of the angle) beside this one.
   const double inv_dr = c->sphere ? c->nbins / (c->tmax - c->tmin) : c->nbins / (rmax_u - rmin_u);
   g.inv_dr_u = (float)inv_dr;
   g.bin_shift = (float)(-(c->sphere ? c->tmin : rmin_u) * inv_dr - 0.5);
-  g.half_bin = (float)(0.5 - (c->sphere ? std::max(1e-4, 4e-7 * c->tmax * inv_dr) : std::max(1e-4, 8e-7 * rmax_u * inv_dr)));
+  g.half_bin = (float)(0.5 - (c->sphere ? std::max(1e-4, 4e-7 * c->tmax * inv_dr) : std::max(1e-4, 1.5e-6 * rmax_u * inv_dr)));
   g.cell_scale = (float)(nc / std::ldexp(1.0, g.shift));
   g.rcell = (float)(rmax_u * nc / std::ldexp(1.0, g.shift) * (1.0 + 1e-5) + 1e-3);
   g.general = c->sphere;
@@ -610,10 +613,10 @@ double mean_row(const ctb_ctx* c) {
 
 int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   // The count pass takes four steps of a row at a time (four loads in flight,
-  // one vote and one store) where rows are long; it holds 60 registers so,
-  // 12 fewer warps' worth, and short rows lose by that.  Enumeration with one
-  // / four steps: 296 points a row (10^6 points) 151.4 / 143.8 ms, 231 (cut
-  // sky) 98.3 / 101.7, 30 (mock catalogues) 26.3 / 28.5.
+  // one vote, one store, paired FP32 instructions) where rows are long; its
+  // state fills 64 registers so, and short rows lose by that.  Enumeration
+  // with one / four steps: 296 points a row (10^6 points) 150.7 / 132.8 ms,
+  // 231 (cut sky) 98.8 / 98.6, 30 (mock catalogues) 23.0 / 25.5.
   c->g.long_rows = mean_row(c) >= 256.0;
   int wpb = c->wpb > 0 ? c->wpb : 4;
   int bps = c->sphere ? am_blocks_per_sm(c->lmax, wpb) : alm_blocks_per_sm(c->Lk, wpb);

@@ -46,8 +46,8 @@ struct Geom {
   uint32_t ncells;     // nc * nc * ncx
   int nbins;
   int lmax;            // requested ell_max
-  float rlo2_u;        // r_min^2 in units^2, widened by 1e-5 (float pre-filter)
-  float rhi2_u;        // r_max^2 in units^2, widened by 1e-5 (float pre-filter)
+  float rlo2_u;        // r_min^2 in units^2, widened by 1e-6 (float pre-filter)
+  float rhi2_u;        // r_max^2 in units^2, widened by 1e-6 (float pre-filter)
   float inv_dr_u;      // nbins / (r_max - r_min) in 1/units (sphere: of the angles)
   float bin_shift;     // -r_min * inv_dr - 1/2: bin coordinate minus 1/2 = r inv_dr + bin_shift
   float half_bin;      // 1/2 less the float error of that coordinate (padded): within it the bin is certain

@@ -217,15 +217,14 @@ __device__ __forceinline__ uint32_t find_segment(const WarpSegs& sg, uint32_t k0
 // and rows cut to the points' shell.  LONG: four steps of a row at a time
 // (plan_pairs says when).
 //
-// Bound by instruction issue (count: 70 instructions per 32 candidates, 84 %
-// of the issue slots on 20k primaries of 10^6 points) and, in the fill, by
-// match_any.  Enumeration with the walk segment by segment / with this one:
-// 10^6 points 168 / 144 ms, cut sky of 800k 121 / 102, 3.1M-pixel sphere 90 /
-// 63, 24 mock catalogues 35.8 / 23.7, 20k uniform points 0.384 / 0.142.  The
-// last of these numbers with the fill finding the rows again, as the count
-// does: 144, 100, 69, 26.3, 0.185.  Four blocks of 8 warps per SM (64
-// registers): five spill in the count (sphere 67 ms) and cost the fill its
-// look-ahead (cut sky 106 ms).
+// Bound by instruction issue (about 60 instructions per 32 candidates; 71 %
+// of the issue slots) and, in the fill, by match_any.  Enumeration with the
+// walk segment by segment / with this one: 10^6 points 168 / 133 ms, cut sky
+// of 800k 121 / 98.7, 3.1M-pixel sphere 90 / 60.5, 24 mock catalogues 35.8 /
+// 22.9, 20k uniform points 0.384 / 0.139.  With the fill finding the rows
+// again, as the count does, the second numbers rose by 0, -2, 6.4, 2.6 and
+// 0.043.  Four blocks of 8 warps per SM (64 registers): five spill in the
+// count (sphere 67 ms) and cost the fill its look-ahead (cut sky 106 ms).
 template <bool GEN, bool LONG>
 __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
   extern __shared__ uint32_t s_cnt_all[];
@@ -260,7 +259,6 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
   const float rlo2 = pin(g.rlo2_u), rhi2 = pin(g.rhi2_u);
   const float inv_dr = pin(g.inv_dr_u), shift = pin(g.bin_shift);
   const float half_bin = pin(g.half_bin);
-  const uint32_t nb = __float_as_uint(pin(__uint_as_float((uint32_t)nbins)));
   // this warp's pool in the code buffer (batches take consecutive
   // ranges of it; a new pool is taken when one does not fit)
   unsigned long long pool = 0, pool_end = 0;
@@ -365,7 +363,9 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
           // th: the bin coordinate minus 1/2.  Rounded to the nearest integer
           // (by adding 1.5 * 2^23) it is the bin, and what is left over is
           // the distance from the bin's middle, within `half` of it unless
-          // the pair may lie on an edge.
+          // the pair may lie on an edge.  rlo2 and rhi2 are so close to the
+          // first and last edge that a pair past them is within that margin
+          // too: b needs no range test (10^6 points: 144 ms with one).
           float th, half;
           if constexpr (GEN) {
             // sphere: the bin of theta = 2 asin(chord / 2).  Its float
@@ -387,7 +387,28 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
           }
           const float tm = th + 12582912.f;
           b = __float_as_uint(tm) - 0x4b400000u;
-          return inb && (b >= nb || fabsf(th - (tm - 12582912.f)) > half);
+          return inb & (fabsf(th - (tm - 12582912.f)) > half);
+        };
+        // Two candidates of a lane in paired FP32 instructions, the same
+        // operations as above in half the issue slots: count and fill of 10^6
+        // points in 132.8 ms against 134.9.
+        auto classify2 = [&](const uint4 qa, const uint4 qb, bool* in, uint32_t* bin, bool* edge) {
+          auto sep = [](uint32_t p, uint32_t u, uint32_t v) {
+            return make_float2(__int2float_rn((int)(u - p)), __int2float_rn((int)(v - p)));
+          };
+          auto both = [](float v) { return make_float2(v, v); };
+          const float2 dx = sep(P.x, qa.x, qb.x), dy = sep(P.y, qa.y, qb.y), dz = sep(P.z, qa.z, qb.z);
+          const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+          const float2 r = __fmul2_rn(r2, make_float2(rsqrt_fast(r2.x), rsqrt_fast(r2.y)));
+          const float2 th = __ffma2_rn(r, both(inv_dr), both(shift));
+          const float2 tm = __fadd2_rn(th, both(12582912.f));
+          const float2 d = __ffma2_rn(__fadd2_rn(tm, both(-12582912.f)), both(-1.f), th);
+          in[0] = r2.x >= rlo2 && r2.x < rhi2;
+          in[1] = r2.y >= rlo2 && r2.y < rhi2;
+          bin[0] = __float_as_uint(tm.x) - 0x4b400000u;
+          bin[1] = __float_as_uint(tm.y) - 0x4b400000u;
+          edge[0] = in[0] & (fabsf(d.x) > half_bin);
+          edge[1] = in[1] & (fabsf(d.y) > half_bin);
         };
         // on an edge: exact integer r^2 against exact thresholds
         auto exact = [&](const uint4 q, bool& inb, uint32_t& b) {
@@ -427,18 +448,18 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
               const uint32_t last = 3u - ((k0 >> 5) & 3u);  // the step of the four that ends a word
               for (; k0 + 128u <= uend; k0 += 128u, qp += 128) {
                 uint4 q[4];
-  #pragma unroll
+#pragma unroll
                 for (int u = 0; u < 4; ++u) q[u] = __ldg(qp + 32 * u);
                 bool inb[4], edge[4];
                 uint32_t b[4];
-  #pragma unroll
-                for (int u = 0; u < 4; ++u) edge[u] = classify(q[u], inb[u], b[u]);
+#pragma unroll
+                for (int u = 0; u < 4; u += 2) classify2(q[u], q[u + 1], inb + u, b + u, edge + u);
                 if (__any_sync(0xffffffffu, edge[0] | edge[1] | edge[2] | edge[3])) {
-  #pragma unroll
+#pragma unroll
                   for (int u = 0; u < 4; ++u)
                     if (edge[u]) exact(q[u], inb[u], b[u]);
                 }
-  #pragma unroll
+#pragma unroll
                 for (int u = 0; u < 4; ++u) {
                   emit(inb[u], b[u]);
                   if (last == (uint32_t)u) __stcs(cp, word);
