@@ -56,7 +56,7 @@ INST_PER_UPDATE = 2.6
 # the captured launches, summed over the m-pass launches of one chunk: one at
 # l_max 10, three at l_max 20).  Keyed by l_max; a missing entry reports null
 # traffic.
-K_ALM_DRAM_BYTES_PER_PAIR = {10: 4.383, 20: 21.17}
+K_ALM_DRAM_BYTES_PER_PAIR = {10: 4.382, 20: 24.39}
 FP32_LANES_PER_SM = 128
 
 
@@ -107,7 +107,7 @@ def workload(name: str):
 
 PASS_CAP = 184          # accumulators per pass of the accumulation kernel
 SINGLE_PASS_LMAX = 10   # up to here one pass holds every coefficient
-FIRST_PASS_M1 = 2       # above it the first (Chebyshev) pass ends at m = 2
+FIRST_PASS_M1 = 2       # above it the first pass ends at m = 2
 
 
 def _coefs(L: int, m0: int, m1: int) -> int:
@@ -167,17 +167,16 @@ def _cpow_flops(e: int) -> int:
 def flops_per_pair(lmax: int) -> int:
     """Algorithmic FP32 FLOPs per pair of the accumulation kernel (FMA = 2),
     counted from its formulation: per m-range pass the separation norm and
-    direction (8), the pass's basis sequence (Chebyshev: one FMA per degree;
-    the first column's monic recurrence: MUL + FMA per degree), the pass's
-    first power w (x+iy)^m0 by squaring, one complex multiplication (6) per
+    direction (8), the pass's basis sequence (the scaled z, then one FMA per
+    degree), the pass's first power w (x+iy)^m0 by squaring, one complex multiplication (6) per
     further column, and one FMA per moment (an ADD for degree 0)."""
     L = lmax
     f = 0
     for m0, m1 in pass_split(L):
         f += 8
         K = L - m0
-        if K >= 2:
-            f += (K - 1) * (2 if m0 == 0 else 3)
+        if K >= 1:
+            f += 1 + 2 * (K - 1)
         ms = max(m0, 1)
         if m0 == 0:
             f += 1 + 2 * L                                # column 0

@@ -31,7 +31,7 @@
 // in (x + i y)^m, and it keeps |z| small where m is large: so the pass that
 // starts at column m0 takes s < 1 (basis_scale), which makes its polynomials
 // nearly orthogonal under that factor.  The flush's map then amplifies
-// rounding by at most 10 (rms over z; l_max 10: 9, l_max 20: 6, 11 and 7 in
+// rounding by at most 11 (rms over z; l_max 10: 9, l_max 20: 6, 11 and 7 in
 // the three passes).  T_k(z) for the first pass and the monic recurrence of
 // column m0 for the others, the bases before these, amplified by up to 39 at
 // l_max 10 and 64 at l_max 20 and took two instructions a degree above m = 2.

@@ -36,7 +36,7 @@
 // group of 128 candidates), so the count pass stores every fourth step, and a
 // step of the fill pass ranks 32 consecutive candidates.  match_any takes 8
 // cycles per distinct value (measured), which bounds the fill: 32 neighbours
-// along a row share few bins, where 32 taken four apart share twice as few.
+// along a row lie in few bins, 32 taken four apart in twice as many.
 //
 // An idle lane of the count pass looks at the primary itself (r = 0, never a
 // pair), and the codes past the stream's end read kNoBin, so neither pass
