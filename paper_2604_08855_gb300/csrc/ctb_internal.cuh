@@ -220,6 +220,18 @@ struct Layout {
 };
 void make_layout(int L, Layout* out);
 
+// The 128-byte lines of the list words [off, end) that this lane of a warp
+// prefetches, f(word) for the first word of each.  `end` is taken modulo 2^32:
+// a chunk may hold 2^32 entries, so its last list may end at 0.  The loop runs
+// on the distance from `off` (a primary's lists hold fewer than 2^31 words),
+// which cannot wrap; on the word itself it never ended where `end` lies within
+// 1024 of 2^32.
+template <class F>
+__host__ __device__ __forceinline__ void each_list_line(uint32_t off, uint32_t end, uint32_t lane, F f) {
+  const uint32_t n = end - off;
+  for (uint32_t k = lane * 32u; k < n; k += 1024u) f(off + k);
+}
+
 // Resident blocks per SM of a kernel at this block size and dynamic shared
 // memory (0: it cannot run), its shared-memory limit raised to that.  Both are
 // facts of the kernel and the device, asked once for each (about 3 us a call).

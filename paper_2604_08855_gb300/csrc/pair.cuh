@@ -583,8 +583,8 @@ __device__ __forceinline__ void run_groups(const AlmArgs& a, const Step& step, c
   // a group's list words to L2, while the group before it is read
   auto fetch = [&](int b) {
     if (b >= nbins) return;
-    const uint32_t e = s_off[b + S - 1] + s_n[b + S - 1];
-    for (uint32_t w = s_off[b] + (uint32_t)lane * 32u; w < e; w += 1024u) prefetch_l2(a.lists + w);
+    each_list_line(s_off[b], s_off[b + S - 1] + s_n[b + S - 1], (uint32_t)lane,
+                   [&](uint32_t w) { prefetch_l2(a.lists + w); });
   };
   uint32_t T;
   int b = skip(0, T);
