@@ -717,6 +717,7 @@ int contract_piece(ctb_ctx* c, const PairPlan& pl, int64_t off, int64_t cnt, siz
     ca.slot = P<int>(c->slot);
     ca.partial = P<double>(c->partial) + seg * pl.ncon * zsz;
     ca.part0 = 0;
+    ca.runs = 2;
     ca.sphere = c->sphere;
     CK(c, launch_contract_fp32(ca, pl.ncon, c->st));
   }

@@ -29,11 +29,28 @@ namespace ctb {
 //
 // Block: CH slots x tiles x PG primary groups (group g takes the stage's
 // primaries q = g mod PG).  Rows of more than CH slots are taken in chunks of
-// CH, the block walking its slice once per chunk: each element is still read
-// from HBM once.  Where the tiles do not fit a block they are split over
-// blockIdx.y.  FP32 over at most kConFlush primaries of a group, then one
-// FP64 add per (l, b1 <= b2) entry by one owner thread: the partial sums are
-// deterministic.
+// CH, the block walking its slice once per chunk, and where the tiles do not
+// fit a block they are split over blockIdx.y: a block reads each element of
+// its slice once, so the rows come from HBM once up to 40 bins, twice from 41
+// and three times from 61 (less what L2 still holds).
+//
+// Rounding.  A thread adds a run of primaries in FP32; at its end (flush) the
+// slots of a multipole and the groups are added with their rounding errors
+// carried along, and one owner thread adds each (l, b1 <= b2) entry to the
+// block's FP64 partial row.  So an entry's error is that of the runs alone.
+// l = 0 has one slot, nothing averages over it, and its run is the longest
+// for its size: a block with one group takes its slice in two runs (the
+// length that two blocks per SM would give it), and no run is longer than
+// kConFlush.  Rows of eight chunks or more (32 bins from l_max 15) stay at
+// one run: they flush once a chunk already, and a second of each took 72 us
+// of 5.2 ms at 200k rows, l_max 20.  Float64 output at l = 0 against 64 bits,
+// one run / two, relative rms: 20k rows of 20 bins at l_max 10 1.43e-8 /
+// 7.0e-9, 100k rows 3.1e-8 / 1.5e-8, 20k of 16 bins 1.36e-8 / 7.0e-9; with
+// several groups, plain sums / errors carried: 2000 rows of 10 bins 3.9e-9 /
+// 2.2e-9.  The second flush costs 2 us of 71 at 20k rows of 20 bins.  (With
+// one thread per entry and multipole, whose loads collide in the shared
+// memory's banks and whose partial row is read, added to and written in turn,
+// a flush took 8 us.)
 //
 // Copies (16 bytes each where the rows allow it): rows that fit one chunk are
 // copied as they lie, one contiguous run per stage (kConLinear; kConLinearAny
@@ -107,7 +124,7 @@ static ConShape con_shape(int nbins, int row) {
   // their end: slots and bins that nothing owns
   c.stage_floats = c.Q * nbins * c.stride + (nbins < c.T ? (c.T - nbins) * c.stride : 0) + c.ch;
   c.stage_floats = (c.stage_floats + 3) & ~3;
-  const int red = c.threads * c.T * c.T;  // the flush buffer aliases the stages (154 KB at most)
+  const int red = (c.threads + 1) * c.T * c.T;  // the flush buffer aliases the stages (154 KB at most)
   c.stages = kConStages;
   while (c.stages > 1 && (size_t)(c.stages * (c.stage_floats + kConMaxQ)) * 4 + 4096 > kConSmemCap) --c.stages;
   const int body = c.stages * c.stage_floats > red ? c.stages * c.stage_floats : red;
@@ -179,10 +196,21 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
   const int tid = threadIdx.x;
   const int c = tid % CH;
   const int tl = (tid / CH) % sh.tiles, pg = tid / (CH * sh.tiles);
-  const int64_t slice = ((a.np + gridDim.x - 1) / gridDim.x + 3) & ~(int64_t)3;
+  // Slices and runs of whole multiples of `gran` primaries, so that they start
+  // on 16 bytes when the base does; long ones on whole 128-byte lines where
+  // four primaries or fewer make one (100k rows of 16 bins x 121: 229 us
+  // against 241 where every other run started in the middle of a line).
+  const int64_t even = (a.np + gridDim.x - 1) / gridDim.x;
+  int gran = 1;
+  while (gran < 4 && (gran * nb * a.row) % (even >= 64 ? 32 : 4) != 0) gran *= 2;
+  auto whole = [&](int64_t n) { return (n + gran - 1) / gran * gran; };
+  const int64_t slice = whole(even);
   const int64_t p0 = (int64_t)blockIdx.x * slice;
   const int64_t p1 = min(a.np, p0 + slice);
   if (p0 >= p1) return;  // uniform for the block
+  // primaries between two flushes
+  const int runs = sh.pg > 1 || sh.nchunk >= 8 ? 1 : a.runs;
+  const int64_t run = min(whole((slice + runs - 1) / runs), (int64_t)kConFlush * sh.pg);
   // tile -> (B1 <= B2); the last tile of a side is moved back so that it ends
   // at the last bin (its bins before B T are computed twice, written once)
   for (int t = tid; t < sh.tiles; t += blockDim.x) {
@@ -303,47 +331,52 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
     // the sums over each multipole's slots: all accumulators to shared memory
-    // ([entry of the tile][thread]), then one thread per (entry, multipole),
-    // four slots' loads in flight
+    // ([entry of the tile][thread], rows padded by one), then a warp takes 32
+    // entries of one multipole, every lane the same slots of its entry
     auto flush = [&] {
       float* red = s_stage;
-      const int nthr = blockDim.x, nl = s_nl;
+      const int nthr = blockDim.x, ld = nthr + 1, nl = s_nl;
       __syncthreads();
 #pragma unroll
       for (int i = 0; i < T; ++i)
 #pragma unroll
         for (int j = 0; j < T / 2; ++j) {
-          red[(i * T + 2 * j) * nthr + tid] = acc[i][j].x;
-          red[(i * T + 2 * j + 1) * nthr + tid] = acc[i][j].y;
+          red[(i * T + 2 * j) * ld + tid] = acc[i][j].x;
+          red[(i * T + 2 * j + 1) * ld + tid] = acc[i][j].y;
           acc[i][j] = make_float2(0.f, 0.f);
         }
       __syncthreads();
-      const int total = sh.tiles * T * T * nl;
-      for (int o = tid; o < total; o += nthr) {
-        const int tk = o / nl, k = o - tk * nl;
-        const int t = tk / (T * T), ij = tk % (T * T);
+      const int entries = sh.tiles * T * T;
+      const int items = (entries + 31) / 32 * nl;
+      for (int o = tid >> 5; o < items; o += nthr >> 5) {
+        const int gr = o / nl;
+        const int k = (o - gr * nl + gr) % nl;  // rotated, so that every warp gets long and short ones
+        const int en = gr * 32 + (tid & 31);
+        const int t = en < entries ? en / (T * T) : 0, ij = en < entries ? en - t * T * T : 0;
         const int v2 = s_tile[t];
-        if (v2 < 0) continue;
         const int C1 = v2 & 255, C2 = v2 >> 8;
         const int b1 = start(C1) + ij / T, b2 = start(C2) + ij % T;
-        if (b1 >= nb || b2 >= nb || b1 > b2 || b1 < C1 * T || b2 < C2 * T) continue;
+        const bool own = en < entries && v2 >= 0 && b1 < nb && b2 < nb && b1 <= b2 && b1 >= C1 * T && b2 >= C2 * T;
         const int q0 = s_l0[k], q1 = s_l0[k + 1];
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        float v = 0.f, c = 0.f;  // the sum and the errors of its additions
         for (int g = 0; g < sh.pg; ++g) {
-          const float* rg = red + ij * nthr + (g * sh.tiles + t) * CH;
-          for (int q = q0; q < q1; q += 4) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              if (q + e < q1) v[e] += rg[s_ord[q + e]];
+          const float* rg = red + ij * ld + (g * sh.tiles + t) * CH;
+#pragma unroll 4
+          for (int q = q0; q < q1; ++q) {
+            const float x = rg[s_ord[q]], s = v + x, b = s - v;
+            c += (v - (s - b)) + (x - b);
+            v = s;
           }
         }
-        out[((size_t)s_l[k] * nb + b1) * nb + b2] += (double)((v[0] + v[1]) + (v[2] + v[3]));
+        // one thread an entry, one flush after another: the order of the adds is fixed
+        if (own)
+          atomicAdd(out + ((size_t)s_l[k] * nb + b1) * nb + b2, (double)v + (isfinite(c) ? (double)c : 0.0));  // v may be infinite
       }
       __syncthreads();
     };
 
-    for (int64_t f0 = p0; f0 < p1; f0 += (int64_t)kConFlush * sh.pg) {
-      const int64_t f1 = min(p1, f0 + (int64_t)kConFlush * sh.pg);
+    for (int64_t f0 = p0; f0 < p1; f0 += run) {
+      const int64_t f1 = min(p1, f0 + run);
       const int nst = (int)((f1 - f0 + sh.Q - 1) / sh.Q);
       auto count = [&](int k) { return (int)min((int64_t)sh.Q, f1 - f0 - (int64_t)k * sh.Q); };
       for (int k = 0; k < sh.stages - 1; ++k) {

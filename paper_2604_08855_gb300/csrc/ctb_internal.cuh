@@ -378,6 +378,7 @@ struct ContractArgs {
   const int* slot;         // device copy of Layout::slot
   double* partial;         // [nparts][(lmax+1)][nbins][nbins] (upper triangle used)
   int part0;               // first partial row this launch writes
+  int runs;                // FP32 runs a block takes its slice in, at least (more than one group: one will do)
   int sphere;              // 0: group l = components l^2 .. l^2+2l; 1: group m = {0} or {2m-1, 2m}
 };
 cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t st);
