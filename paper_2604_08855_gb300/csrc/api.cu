@@ -17,14 +17,24 @@ using namespace ctb;
 namespace ctb {
 thread_local unsigned long long g_launches = 0;
 
+cudaError_t allow_smem(const void* fn, size_t smem) {
+  static std::mutex mu;
+  if (smem <= 48 * 1024) return cudaSuccess;
+  // the limit is one per kernel and device context, and the context may have
+  // been reset: it is read each time, and never lowered under another thread
+  std::lock_guard<std::mutex> lock(mu);
+  cudaFuncAttributes at{};
+  const cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  if (e != cudaSuccess || (size_t)at.maxDynamicSharedSizeBytes >= smem) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 int resident_blocks(const void* fn, int threads, size_t smem) {
   static std::mutex mu;
   static std::map<std::tuple<int, const void*, int, size_t>, int> known;  // a few entries per kernel and device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  // the limit belongs to the device's context, which a program may reset
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (allow_smem(fn, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }

@@ -699,12 +699,12 @@ cudaError_t launch_pack(bool tf32, const float* M, const float* wprim, int64_t n
   const size_t smem = ((size_t)2 * kPackPrims * row + kPackPrims + (size_t)(lmax + 1) * (lmax + 1)) * 4;
   cudaError_t e;
   if (tf32) {
-    e = cudaFuncSetAttribute(k_pack<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem((const void*)k_pack<true>, smem);
     if (e != cudaSuccess) return e;
     k_pack<true><<<(unsigned)blocks, kPackThreads, smem, st>>>(M, wprim, np, nbins, row, lmax, slot, lbase, kp, outS,
                                                                outH, outL, err, kTcTimeoutCycles);
   } else {
-    e = cudaFuncSetAttribute(k_pack<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem((const void*)k_pack<false>, smem);
     if (e != cudaSuccess) return e;
     k_pack<false><<<(unsigned)blocks, kPackThreads, smem, st>>>(M, wprim, np, nbins, row, lmax, slot, lbase, kp, outS,
                                                                 outH, outL, err, kTcTimeoutCycles);
@@ -775,7 +775,7 @@ cudaError_t launch_contract_tc(bool tf32, int64_t np, int nbins, int lmax, const
   const int grid = std::max(1, std::min(kTcCtasPerSm * nsm, nsplit));
   void (*fn)(const TcArgsMaps) = tf32 ? (a.nchain == 2 ? k_contract_tc<true, 2> : k_contract_tc<true, 1>)
                                      : (a.nchain == 2 ? k_contract_tc<false, 2> : k_contract_tc<false, 1>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<grid, kTcThreads, smem, st>>>(am);
   ++g_launches;

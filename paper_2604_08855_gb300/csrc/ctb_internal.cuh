@@ -232,9 +232,14 @@ __host__ __device__ __forceinline__ void each_list_line(uint32_t off, uint32_t e
   for (uint32_t k = lane * 32u; k < n; k += 1024u) f(off + k);
 }
 
+// Raises a kernel's limit of dynamic shared memory to `smem` if it is lower.
+// Host threads launch one kernel with several sizes: a limit set to each
+// launch's own size could be lowered between another thread's call and its launch.
+cudaError_t allow_smem(const void* fn, size_t smem);
+
 // Resident blocks per SM of a kernel at this block size and dynamic shared
-// memory (0: it cannot run), its shared-memory limit raised to that.  Both are
-// facts of the kernel and the device, asked once for each (about 3 us a call).
+// memory (0: it cannot run), its shared-memory limit raised to that.  The
+// number is a fact of the kernel and the device, asked once for each (about 3 us a call).
 int resident_blocks(const void* fn, int threads, size_t smem);
 
 // kernels launched by this host thread (every launcher adds its launches)
