@@ -365,16 +365,23 @@ cudaError_t launch_gather(const uint32_t* val_sorted, const uint4* pts_in, int64
 }
 
 // cell_start[c] = first sorted position with key >= c, for c in [0, ncells].
-// A block writes kCellTile entries: it finds the tile's first point by a
-// 32-way search of the sorted keys, counts the tile's points per cell in
-// shared memory and scans the counts.  So the table is written once and not
-// read: it is far larger than the catalogue where cells are fine (5.3 GB for
-// 3.1M points on the sphere at 8 cells per r_max), and clearing, counting,
-// reducing and scanning it took 5.2 ms and 16 MB's worth 30 us of launches
-// (now 1.1 ms and 9 us).
+// A block writes a tile of kCellThreads * ITEMS entries: it finds the tile's
+// first point by a 32-way search of the sorted keys, counts the tile's points
+// per cell in shared memory and scans the counts.  So the table is written
+// once and not read: it is far larger than the catalogue where cells are fine
+// (5.3 GB for 3.1M points on the sphere at 8 cells per r_max), and clearing,
+// counting, reducing and scanning it took 5.2 ms and 16 MB's worth 30 us of
+// launches (now 1.1 ms and 9 us).
+//
+// A tile's count takes as long as it has points.  Where they are many times
+// its cells (kCellHeavy: a coarse grid, a clump in a fine one), every entry is
+// searched for instead, log2(points) loads each; and tables of few tiles are
+// cut into smaller ones (ITEMS 2), so that the chip is filled.  Sort and grid
+// of 4M points, counting alone in tiles of 8192 / now: 1728 cells 0.881 /
+// 0.228 ms, 64,000 cells 0.328 / 0.253, nearly all points in a clump among 35M cells
+// 0.871 / 0.316.
 constexpr int kCellThreads = 256;
-constexpr int kCellItems = 32;
-constexpr int kCellTile = kCellThreads * kCellItems;
+constexpr uint32_t kCellHeavy = 16;  // points per cell of a tile: a count of P / 256 steps against ITEMS log2(P) of search
 
 // first position whose key is at least c, by one warp
 __device__ __forceinline__ uint32_t lower_bound_warp(const uint32_t* __restrict__ key, uint32_t n, uint64_t c, int lane) {
@@ -391,58 +398,96 @@ __device__ __forceinline__ uint32_t lower_bound_warp(const uint32_t* __restrict_
   return lo;
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kCellThreads) k_cell_table(const uint32_t* __restrict__ key, uint32_t n,
                                                              uint64_t entries, uint32_t* __restrict__ cell_start) {
-  // entry k of the tile at [k / kCellItems][k % kCellItems], rows padded by one: conflict-free both ways
-  __shared__ uint32_t s_cnt[kCellThreads * (kCellItems + 1)];
+  constexpr int TILE = kCellThreads * ITEMS;
+  // entry k of the tile at [k / ITEMS][k % ITEMS], rows padded by one: conflict-free both ways
+  __shared__ uint32_t s_cnt[kCellThreads * (ITEMS + 1)];
   __shared__ uint32_t s_range[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t c0 = (uint64_t)blockIdx.x * kCellTile;
+  const uint64_t c0 = (uint64_t)blockIdx.x * TILE;
   if (warp < 2) {
-    const uint32_t p = lower_bound_warp(key, n, c0 + (uint64_t)warp * kCellTile, lane);
+    const uint32_t p = lower_bound_warp(key, n, c0 + (uint64_t)warp * TILE, lane);
     if (lane == 0) s_range[warp] = p;
   }
-  for (int k = tid; k < kCellThreads * (kCellItems + 1); k += kCellThreads) s_cnt[k] = 0;
+  for (int k = tid; k < kCellThreads * (ITEMS + 1); k += kCellThreads) s_cnt[k] = 0;
   __syncthreads();
   const uint32_t p0 = s_range[0], p1 = s_range[1];
+  if (p1 - p0 > kCellHeavy * TILE) {  // uniform for the block
+    constexpr int G = ITEMS < 4 ? ITEMS : 4;  // searches side by side
+    for (int e = tid; e < TILE; e += G * kCellThreads) {
+      uint32_t lo[G];
+#pragma unroll
+      for (int u = 0; u < G; ++u) lo[u] = p0;
+      uint32_t len = p1 - p0;  // entry's answer in [lo, lo + len]
+      while (len > 0) {
+        const uint32_t half = (len + 1) / 2;
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+          if (key[lo[u] + half - 1] < c0 + e + u * kCellThreads) lo[u] += half;
+        len -= half;
+      }
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        const uint64_t c = c0 + e + u * kCellThreads;
+        if (c < entries) cell_start[c] = lo[u];
+      }
+    }
+    return;
+  }
+#pragma unroll 4
   for (uint32_t p = p0 + tid; p < p1; p += kCellThreads) {
     const uint32_t k = (uint32_t)(key[p] - c0);
-    atomicAdd(s_cnt + k + k / kCellItems, 1u);
+    atomicAdd(s_cnt + k + k / ITEMS, 1u);
   }
   __syncthreads();
-  uint32_t v[kCellItems], s = 0;
+  uint32_t v[ITEMS], s = 0;
 #pragma unroll
-  for (int k = 0; k < kCellItems; ++k) {
-    v[k] = s_cnt[tid * (kCellItems + 1) + k];
+  for (int k = 0; k < ITEMS; ++k) {
+    v[k] = s_cnt[tid * (ITEMS + 1) + k];
     s += v[k];
   }
   uint32_t total;
   uint32_t ex = p0 + block_exclusive_scan(s, &total);
 #pragma unroll
-  for (int k = 0; k < kCellItems; ++k) {
-    s_cnt[tid * (kCellItems + 1) + k] = ex;
+  for (int k = 0; k < ITEMS; ++k) {
+    s_cnt[tid * (ITEMS + 1) + k] = ex;
     ex += v[k];
   }
   __syncthreads();
-  // 16-byte stores of the tile in order (the table and the tile start on 16 bytes)
-  for (int k = 4 * tid; k < kCellTile; k += 4 * kCellThreads) {
-    const uint32_t* e = s_cnt + k + k / kCellItems;
-    const uint64_t c = c0 + k;
-    if (c + 4 <= entries) {
-      __stcs(reinterpret_cast<uint4*>(cell_start + c), make_uint4(e[0], e[1], e[2], e[3]));
-    } else {
-      for (int d = 0; d < 4 && c + d < entries; ++d) cell_start[c + d] = e[d];
+  if constexpr (ITEMS % 4 == 0) {
+    // 16-byte stores of the tile in order (the table and the tile start on 16 bytes)
+    for (int k = 4 * tid; k < TILE; k += 4 * kCellThreads) {
+      const uint32_t* e = s_cnt + k + k / ITEMS;
+      const uint64_t c = c0 + k;
+      if (c + 4 <= entries) {
+        __stcs(reinterpret_cast<uint4*>(cell_start + c), make_uint4(e[0], e[1], e[2], e[3]));
+      } else {
+        for (int d = 0; d < 4 && c + d < entries; ++d) cell_start[c + d] = e[d];
+      }
     }
+  } else {
+    for (int k = tid; k < TILE; k += kCellThreads)
+      if (c0 + k < entries) cell_start[c0 + k] = s_cnt[k + k / ITEMS];
   }
+}
+
+template <int ITEMS>
+static cudaError_t cell_table(const uint32_t* key, int64_t n, uint64_t entries, uint32_t* cell_start, cudaStream_t st) {
+  constexpr int TILE = kCellThreads * ITEMS;
+  k_cell_table<ITEMS><<<(unsigned)((entries + TILE - 1) / TILE), kCellThreads, 0, st>>>(key, (uint32_t)n, entries,
+                                                                                       cell_start);
+  ++g_launches;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_cell_start(const uint32_t* key_sorted, int64_t n, uint32_t ncells, uint32_t* cell_start,
                               cudaStream_t st) {
   const uint64_t entries = (uint64_t)ncells + 1;
-  k_cell_table<<<(unsigned)((entries + kCellTile - 1) / kCellTile), kCellThreads, 0, st>>>(key_sorted, (uint32_t)n,
-                                                                                          entries, cell_start);
-  ++g_launches;
-  return cudaGetLastError();
+  // below two tiles of 8192 for each of the 152 SMs: tiles of 512
+  return entries < 304ull * kCellThreads * 32 ? cell_table<2>(key_sorted, n, entries, cell_start, st)
+                                              : cell_table<32>(key_sorted, n, entries, cell_start, st);
 }
 
 }  // namespace ctb
