@@ -214,6 +214,9 @@ int ctb_get_pivot_groups(ctb_ctx* ctx, double* pivot_cell, int64_t* groups);
  *                coefficient (l, m) of the real basis at index l*l + l + m,
  *                Y_l,+m ~ cos(m phi), Y_l,-m ~ sin(m phi), Condon-Shortley
  *                phase included.
+ * A primary's rows depend on the catalogue, its grid and the configuration,
+ * not on the other primaries of the call: they are the same bits alone, in
+ * any list and in any chunk.
  */
 int ctb_get_alm(ctb_ctx* ctx, const int64_t* primary_idx, int64_t m, float* alm_out);
 

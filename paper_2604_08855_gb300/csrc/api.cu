@@ -765,8 +765,8 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   CK(c, ensure(c, c->scan_tmp2, scan_tmp_words((size_t)pl.chunk_max * nb) * 4));
   CK(c, ensure(c, c->M, (size_t)pl.chunk_max * nb * c->lay.row * sizeof(float)));
   CK(c, ensure(c, c->wprim, (size_t)pl.chunk_max * sizeof(float)));
-  // counters of a chunk: count's work, pairs, code bytes, fill's work, then one per m-pass
-  constexpr size_t kCounters = 4 + kLmaxCap + 1;
+  // counters of a chunk: count's work, pairs, code bytes, list classes, fill's work, then one per m-pass
+  constexpr size_t kCounters = 5 + kLmaxCap + 1;
   CK(c, ensure(c, c->counters, kCounters * 8));
   CK(c, ensure(c, c->code_base, (size_t)pl.chunk_max * row_blocks(c->g) * sizeof(unsigned long long)));
   unsigned long long* work = P<unsigned long long>(c->counters);
@@ -783,6 +783,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   sa.wsub = c->wsub;
   sa.work = work;
   sa.total = total;
+  sa.classes = work + 3;
   sa.keys = c->batch_keys;
   sa.code_total = code_total;
   sa.code_base = P<unsigned long long>(c->code_base);
@@ -794,7 +795,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   aa.offsets = P<uint32_t>(c->offsets);
   aa.M = P<float>(c->M);
   aa.conv = P<uint8_t>(c->conv);
-  aa.work = work + 4;
+  aa.work = work + 5;
   aa.nbins = nb;
   aa.row = c->lay.row;
   for (int k = 0; k < 3; ++k) aa.sph_origin[k] = (float)c->origin[k];
@@ -826,7 +827,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     sa.work = work;
     CK(c, launch_stream(sa, false, pl.count_blocks, c->st));
     CK(c, cudaEventRecord(ev[1], c->st));
-    CK(c, cudaMemcpyAsync(c->pin, total, 16, cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaMemcpyAsync(c->pin, total, 24, cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
     c->t_ms[6] += elapsed(ev[0], ev[1]);
     c->t_ms[2] = c->t_ms[6] + c->t_ms[7];
@@ -850,10 +851,11 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
                              P<uint32_t>(c->scan_tmp2), c->st));
     sa.lists = P<uint32_t>(c->lists);
     aa.lists = P<uint32_t>(c->lists);
-    sa.work = work + 3;
+    sa.work = work + 4;
     CK(c, launch_stream(sa, true, pl.stream_blocks, c->st));
     CK(c, cudaEventRecord(ev[2], c->st));
-    const int lists = lists_per_warp((double)tot / ((double)cnt * nb));
+    // one form for every primary of the chunk where they agree on it
+    const int lists = c->pin[2] == 1 ? 1 : (c->pin[2] == 4 ? 4 : 0);
     if (c->sphere)
       CK(c, launch_am(aa, c->lmax, lists, pl.wpb, c->nsm, c->st));
     else

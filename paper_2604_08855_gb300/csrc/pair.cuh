@@ -656,8 +656,21 @@ template <class Step, int S>
 __device__ __forceinline__ void run_primary(const AlmArgs& a, const Step& step, const uint32_t* s_off,
                                             const uint32_t* s_n, const uint4 P, float* __restrict__ rows,
                                             const float2* ctab, float* sbuf, int lane) {
-  if constexpr (S == 1) run_primary1(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
-  else run_groups<Step, S>(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+  if constexpr (S == 0) {
+    const uint32_t total = s_off[a.nbins - 1] + s_n[a.nbins - 1] - s_off[0];
+    switch (lists_per_warp(total, a.nbins)) {
+      case 1:
+        return run_primary1(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+      case 2:
+        return run_groups<Step, 2>(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+      default:
+        return run_groups<Step, 4>(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+    }
+  } else if constexpr (S == 1) {
+    run_primary1(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+  } else {
+    run_groups<Step, S>(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
+  }
 }
 
 // number of m-passes of kernel L, and the columns and row offset of pass P
@@ -694,10 +707,11 @@ __host__ __device__ constexpr size_t conv_pass_offset(int L, int P) {
 // warps per scheduler allow 255 registers a thread, 3 allow 168, 4 allow 128)
 __host__ __device__ constexpr int alm_min_blocks(int ncp) { return ncp <= 32 ? 5 : (ncp <= 64 ? 4 : (ncp <= 136 ? 3 : 2)); }
 
-// per warp: the flush's transpose buffer, the slot totals of S lists, then
-// the primary's list offsets and counts
+// per warp: the flush's transpose buffer and the slot totals of S lists (four
+// for S = 0), then the primary's list offsets and counts
+__host__ __device__ constexpr int alm_flush_floats(int ncp, int S) { return flush_buf_floats(ncp) + (S ? S : 4) * ncp; }
 __host__ __device__ constexpr size_t alm_smem_per_warp(int ncp, int S) {
-  return (size_t)(flush_buf_floats(ncp) + S * ncp) * sizeof(float) + 2 * kNbinsCap * sizeof(uint32_t);
+  return (size_t)alm_flush_floats(ncp, S) * sizeof(float) + 2 * kNbinsCap * sizeof(uint32_t);
 }
 
 // Counts and offsets of primary i into shared memory (empty lists at the end
@@ -721,7 +735,12 @@ __device__ __forceinline__ void load_lists(const AlmArgs& a, uint64_t ib, uint32
 // One warp per primary: its (primary, bin) lists are consecutive runs of the
 // lists buffer; S of them at a time are accumulated in registers for m-pass P
 // of kernel L and flushed once, with the next lists' first loads already in
-// flight.  S: see alm_lists_per_warp.
+// flight.  S: lists_per_warp of every primary (1 or 4), or 0 where they
+// differ: the three forms in one kernel, each primary with its own.  Its code
+// is scheduled less well in the longest loops (chosen primaries of 10^6 points
+// at l_max 10, all with S = 1: 3.55 ms against 3.50; 3.1M pixels on the
+// sphere, all 4: 94.7 against 94.1), and gains where S = 2 is the most
+// frequent (250k primaries of 4M, l_max 20: 157.2 against 158.8).
 //
 // The passes of a kernel with several (l_max > 10) are separate kernels,
 // launched one after another.  With all passes in one launch, warps in
@@ -743,7 +762,7 @@ __global__ void __launch_bounds__(128, alm_min_blocks(pass_ncp(L, P))) k_alm(con
   const int warp = threadIdx.x >> 5;
   char* wbase = s_alm + TB + (size_t)warp * alm_smem_per_warp(NCP, S);
   float* sbuf = reinterpret_cast<float*>(wbase);
-  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)(flush_buf_floats(NCP) + S * NCP) * sizeof(float));
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)alm_flush_floats(NCP, S) * sizeof(float));
   uint32_t* s_n = s_off + kNbinsCap;
   while (true) {
     unsigned long long i = 0;
@@ -793,12 +812,12 @@ cudaError_t launch_passes(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
 template <int L>
 cudaError_t launch_alm_L(const AlmArgs& a, int lists, int wpb, int nsm, cudaStream_t st) {
   switch (lists) {
-    case 2:
-      return launch_passes<L, 0, 2>(a, wpb, nsm, st);
+    case 1:
+      return launch_passes<L, 0, 1>(a, wpb, nsm, st);
     case 4:
       return launch_passes<L, 0, 4>(a, wpb, nsm, st);
   }
-  return launch_passes<L, 0, 1>(a, wpb, nsm, st);
+  return launch_passes<L, 0, 0>(a, wpb, nsm, st);
 }
 
 // the smallest occupancy over the passes (0: some pass cannot be resident)

@@ -196,20 +196,6 @@ int alm_blocks_per_sm(int L, int wpb) {
   }
 }
 
-// Four lists side by side below a mean of 160 neighbours, two below 800, one
-// above.  A flush costs the same for S lists as for one, but a group of S runs
-// as long as its longest list and its steps carry the validity of each lane
-// (about 5 % more).  Accumulation with 1 / 2 / 4 lists (8: slower than 4
-// except at 8 neighbours a list, where they tie):
-//   mean list 8 (20k uniform points, l_max 10)      0.226 / 0.144 / 0.116 ms
-//   28 (200k points, l_max 20)                      24.0 / 16.7 / 14.7 ms
-//   80 (24 mock catalogues, l_max 10)               52.3 / 39.4 / 39.4 ms
-//   132 (3.1M-pixel sphere, m_max 8)                38.0 / 29.6 / 28.4 ms
-//   522 (cut sky of 800k points, l_max 10)          118.1 / 111.1 / 113.2 ms
-//   525 (250k primaries of 4M, l_max 20)            134.1 / 132.3 / 145.7 ms
-//   1680 (10^6 points, l_max 10)                    221.5 / 243.1 / 274.0 ms
-int lists_per_warp(double mean_list) { return mean_list < 160.0 ? 4 : (mean_list < 800.0 ? 2 : 1); }
-
 cudaError_t launch_alm(const AlmArgs& a, int L, int lists, int wpb, int nsm, cudaStream_t st) {
   switch (L) {
 #define CASE(X) \

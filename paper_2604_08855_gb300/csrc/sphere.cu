@@ -82,7 +82,7 @@ __device__ __forceinline__ StepSphere<0> frame_at(float x, float y, float z) {
   return f;
 }
 
-// One warp per primary, one run per group of S (primary, bin) lists, as in k_alm.
+// One warp per primary, one run per group of S (primary, bin) lists (S = 0: the primary's own), as in k_alm.
 template <int K, int S>
 __global__ void __launch_bounds__(128) k_am(AlmArgs a) {
   extern __shared__ __align__(16) char s_am[];
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(128) k_am(AlmArgs a) {
   // per warp: flush buffers, list offsets, counts
   char* wbase = s_am + (size_t)warp * alm_smem_per_warp(NCP, S);
   float* sbuf = reinterpret_cast<float*>(wbase);
-  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)(flush_buf_floats(NCP) + S * NCP) * sizeof(float));
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(wbase + (size_t)alm_flush_floats(NCP, S) * sizeof(float));
   uint32_t* s_n = s_off + kNbinsCap;
   while (true) {
     unsigned long long i = 0;
@@ -135,12 +135,12 @@ static cudaError_t launch_am_KS(const AlmArgs& a, int wpb, int nsm, cudaStream_t
 template <int K>
 static cudaError_t launch_am_K(const AlmArgs& a, int lists, int wpb, int nsm, cudaStream_t st) {
   switch (lists) {
-    case 2:
-      return launch_am_KS<K, 2>(a, wpb, nsm, st);
+    case 1:
+      return launch_am_KS<K, 1>(a, wpb, nsm, st);
     case 4:
       return launch_am_KS<K, 4>(a, wpb, nsm, st);
   }
-  return launch_am_KS<K, 1>(a, wpb, nsm, st);
+  return launch_am_KS<K, 0>(a, wpb, nsm, st);
 }
 
 #define CTB_SPHERE_CASES(X) \

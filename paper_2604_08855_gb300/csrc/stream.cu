@@ -228,7 +228,10 @@ __device__ __forceinline__ uint32_t find_segment(const WarpSegs& sg, uint32_t k0
 template <bool GEN, bool LONG>
 __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
   extern __shared__ uint32_t s_cnt_all[];
+  __shared__ uint32_t s_classes;  // lists_per_warp of this block's primaries, OR-ed
   __shared__ WarpSegs s_segs[kStreamThreads / 32];
+  if (threadIdx.x == 0) s_classes = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const Geom g = a.g;
@@ -493,16 +496,22 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
     }
     if (lane == 0 && cb < a.code_base + (i + 1) * (uint64_t)nrb) *cb = kNoBatch;
     __syncwarp();
+    uint32_t mine = 0;
     for (int b = lane; b < nbins; b += 32) {
       const uint32_t s = cnt[b];
       a.counts[ib + b] = s;
-      my_pairs += s;
+      mine += s;
     }
+    my_pairs += mine;
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0 && mine) atomicOr(&s_classes, (uint32_t)lists_per_warp(mine, nbins));
     __syncwarp();
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) my_pairs += __shfl_xor_sync(0xffffffffu, my_pairs, o);
   if (lane == 0 && my_pairs) atomicAdd(a.total, my_pairs);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_classes) atomicOr(a.classes, (unsigned long long)s_classes);
 }
 
 // Fill pass.
