@@ -355,8 +355,9 @@ int ctb_get_grid(ctb_ctx* ctx, int* cells_per_rmax, int* cells_per_axis);
  * blocks); otherwise CTB_ERR_ARG.  A failed CUDA call gives CTB_ERR_CUDA.
  * ctb_last_error() does not describe failures of this call.
  * The first call on a device looks up the array's device address and the SM
- * count with that device current (no device work); make that first call
- * before any stream capture.  The partials use one wave of the contraction's
+ * count with that device current and loads the kernels of every shape (no
+ * device work); make that first call before any stream capture and before the
+ * device is reserved: the kernels' code takes some megabytes of it.  The partials use one wave of the contraction's
  * resident blocks, as far as the array holds them.  All calls share the
  * array: calls whose work overlaps on the GPU race and must be serialised by
  * the caller (e.g. one stream).  Each call first clears the partial blocks it

@@ -506,6 +506,18 @@ __global__ void __launch_bounds__(32 * kFinGroups) k_finalize(const double* __re
   }
 }
 
+// Loads every kernel of launch_contract_fp32 and launch_finalize.
+cudaError_t load_contract_fp32() {
+  cudaFuncAttributes at{};
+  cudaError_t e = cudaFuncGetAttributes(&at, k_finalize);
+  for (int mode = kConRows4; mode <= kConLinearAny; ++mode)
+    for (const void* fn : {con_fn<6, 32>(mode), con_fn<6, 64>(mode), con_fn<6, 128>(mode), con_fn<8, 32>(mode),
+                           con_fn<8, 64>(mode), con_fn<8, 128>(mode), con_fn<10, 32>(mode), con_fn<10, 64>(mode),
+                           con_fn<10, 128>(mode)})
+      if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+  return e;
+}
+
 cudaError_t launch_finalize(const double* partial, int nparts, int lmax, int nbins, double* zeta, bool sphere,
                             int ncat, cudaStream_t st) {
   const int total = (lmax + 1) * nbins * nbins;

@@ -408,6 +408,7 @@ struct ContractArgs {
 };
 cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t st);
 int contract_fp32_blocks_per_sm(int nbins, int row);
+cudaError_t load_contract_fp32();
 
 // edge.cu
 void make_threej_table(int lmax, std::vector<double>& t);  // (a b c; 0 0 0)^2, [a][b][c], a,b,c <= lmax

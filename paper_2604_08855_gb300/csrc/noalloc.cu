@@ -13,7 +13,8 @@
 // holds it until the process exits, and every call shares it (calls that
 // overlap on the GPU race on it).  Host code must not use the array's name as
 // a device address: the device address is taken with cudaGetSymbolAddress,
-// once per device, with that device current, on the first call.
+// once per device, with that device current, on the first call, which also
+// loads the kernels of every shape.
 #include <algorithm>
 #include <mutex>
 
@@ -74,7 +75,7 @@ extern "C" int ctb_contract_noalloc(const float* alm, const float* w, int64_t np
     DevScratch& d = g_noalloc_dev[dev];
     if (!d.ready) {
       // set-up, once per device, with this device current: the device
-      // addresses of the file-scope arrays and the SM count (no device work)
+      // addresses of the file-scope arrays, the SM count and the kernels (no device work)
       void* p = nullptr;
       e = cudaGetSymbolAddress(&p, g_noalloc_partial);
       if (e != cudaSuccess) return CTB_ERR_CUDA;
@@ -84,6 +85,9 @@ extern "C" int ctb_contract_noalloc(const float* alm, const float* w, int64_t np
       d.slot = static_cast<int*>(p);
       e = cudaDeviceGetAttribute(&d.nsm, cudaDevAttrMultiProcessorCount, dev);
       if (e != cudaSuccess || d.nsm < 1) return CTB_ERR_CUDA;
+      // a kernel is loaded, into device memory, when it is first used: all of
+      // them now, so that no later call with another shape has to
+      if (load_contract_fp32() != cudaSuccess) return CTB_ERR_CUDA;
       d.ready = true;
     }
     sc = d;
