@@ -598,6 +598,7 @@ struct PairPlan {
   double cand_first;     // candidates per primary assumed for the first chunk
   int nparts;            // pair-sum partial rows (blocks of k_pair_sums)
   int ncon;              // contraction partial rows (blocks of the contraction kernel in use)
+  ListLimits limits;     // lists a warp accumulates side by side
 };
 
 // Bin-code buffer bound: one byte per candidate of a chunk, at most four per
@@ -641,6 +642,17 @@ int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   pl->chunk_max = std::max<int64_t>(1, std::min<int64_t>(chunk, std::max<int64_t>(np, 1)));
   pl->list_cap = c->list_cap;
   pl->nparts = 2 * c->nsm;
+  {
+    // the bins' shares of the neighbours at the mean density: shells, or rings on the sphere
+    double share[kNbinsCap];
+    auto upto = [&](int b) {
+      if (c->sphere) return -std::cos(c->tmin + b * (c->tmax - c->tmin) / c->nbins);
+      const double r = c->rmin + b * (c->rmax - c->rmin) / c->nbins;
+      return r * r * r;
+    };
+    for (int b = 0; b < c->nbins; ++b) share[b] = upto(b + 1) - upto(b);
+    pl->limits = list_limits(share, c->nbins);
+  }
   if (c->precision == CTB_PREC_FP32) {
     // one wave of the FP32 contraction's resident blocks
     const int cb = contract_fp32_blocks_per_sm(c->nbins, c->lay.row);
@@ -784,6 +796,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   sa.work = work;
   sa.total = total;
   sa.classes = work + 3;
+  sa.limits = pl.limits;
   sa.keys = c->batch_keys;
   sa.code_total = code_total;
   sa.code_base = P<unsigned long long>(c->code_base);
@@ -796,6 +809,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
   aa.M = P<float>(c->M);
   aa.conv = P<uint8_t>(c->conv);
   aa.work = work + 5;
+  aa.limits = pl.limits;
   aa.nbins = nb;
   aa.row = c->lay.row;
   for (int k = 0; k < 3; ++k) aa.sph_origin[k] = (float)c->origin[k];
@@ -854,7 +868,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     sa.work = work + 4;
     CK(c, launch_stream(sa, true, pl.stream_blocks, c->st));
     CK(c, cudaEventRecord(ev[2], c->st));
-    // one form for every primary of the chunk where they agree on it
+    // one form for all primaries of the chunk where they agree on it
     const int lists = c->pin[2] == 1 ? 1 : (c->pin[2] == 4 ? 4 : 0);
     if (c->sphere)
       CK(c, launch_am(aa, c->lmax, lists, pl.wpb, c->nsm, c->st));

@@ -319,24 +319,17 @@ cudaError_t launch_group_reduce(const uint32_t* val_sorted, const uint32_t* head
                                 cudaStream_t st);
 
 // Lists that a warp accumulates side by side for a primary with `total`
-// neighbours in `nbins` lists.  It is the primary's own choice, so its rows do
-// not depend on the primaries that it shares a launch with.
-//
-// Four lists side by side below a mean of 160 neighbours, two below 800, one
-// above.  A flush costs the same for S lists as for one, but a group of S runs
-// as long as its longest list and its steps carry the validity of each lane
-// (about 5 % more).  Accumulation with 1 / 2 / 4 lists (8: slower than 4
-// except at 8 neighbours a list, where they tie):
-//   mean list 8 (20k uniform points, l_max 10)      0.226 / 0.144 / 0.116 ms
-//   28 (200k points, l_max 20)                      24.0 / 16.7 / 14.7 ms
-//   80 (24 mock catalogues, l_max 10)               52.3 / 39.4 / 39.4 ms
-//   132 (3.1M-pixel sphere, m_max 8)                38.0 / 29.6 / 28.4 ms
-//   522 (cut sky of 800k points, l_max 10)          118.1 / 111.1 / 113.2 ms
-//   525 (250k primaries of 4M, l_max 20)            134.1 / 132.3 / 145.7 ms
-//   1680 (10^6 points, l_max 10)                    221.5 / 243.1 / 274.0 ms
-__host__ __device__ constexpr int lists_per_warp(uint32_t total, int nbins) {
-  return total < 160u * (uint32_t)nbins ? 4 : (total < 800u * (uint32_t)nbins ? 2 : 1);
+// neighbours: four below ListLimits::four, two below ListLimits::two, else one.
+// It is the primary's own choice, so its rows do not depend on the primaries
+// that share its launch.
+struct ListLimits {
+  uint32_t four, two;
+};
+__host__ __device__ constexpr int lists_per_warp(uint32_t total, ListLimits m) {
+  return total < m.four ? 4 : (total < m.two ? 2 : 1);
 }
+// The limits for lists that grow from bin to bin as `share` (pair_dispatch.cu).
+ListLimits list_limits(const double* share, int nbins);
 
 // stream.cu -- neighbour enumeration (count pass, then fill pass)
 struct StreamArgs {
@@ -354,6 +347,7 @@ struct StreamArgs {
   unsigned long long* work;       // work counter (zeroed before launch)
   unsigned long long* total;      // binned pairs of this launch (count pass, accumulated)
   unsigned long long* classes;    // OR of lists_per_warp over the primaries with neighbours (count pass)
+  ListLimits limits;
   const uint32_t* keys;           // sorted cell keys of a batch (catalogue = key / ncells), or NULL
   uint8_t* codes;                 // bin code per candidate (written: count, read: fill)
   unsigned long long code_cap;    // bytes of codes
@@ -378,6 +372,7 @@ struct AlmArgs {
   float* M;                       // [prim_count][nbins][row]
   const uint8_t* conv;            // flush conversion tables, pass p at conv_pass_offset(L, p)
   unsigned long long* work;       // one zeroed work counter per m-pass
+  ListLimits limits;              // lists a warp takes side by side
   int nbins;
   int row;
   float sph_origin[3];            // sphere mode: the points' position = origin + unit * (x, y, z)

@@ -658,7 +658,7 @@ __device__ __forceinline__ void run_primary(const AlmArgs& a, const Step& step, 
                                             const float2* ctab, float* sbuf, int lane) {
   if constexpr (S == 0) {
     const uint32_t total = s_off[a.nbins - 1] + s_n[a.nbins - 1] - s_off[0];
-    switch (lists_per_warp(total, a.nbins)) {
+    switch (lists_per_warp(total, a.limits)) {
       case 1:
         return run_primary1(a, step, s_off, s_n, P, rows, ctab, sbuf, lane);
       case 2:

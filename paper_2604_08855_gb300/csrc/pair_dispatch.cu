@@ -1,5 +1,6 @@
 // pair_dispatch.cu -- coefficient layout, recurrence constants, and the
 // ell_max dispatch of the pair-multipole kernel.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <utility>
@@ -194,6 +195,56 @@ int alm_blocks_per_sm(int L, int wpb) {
     default:
       return 0;
   }
+}
+
+// A flush costs little more for S lists than for one, but a group of S runs as
+// long as its longest list, on 32 / S lanes a list, and the last group does so
+// with fewer lists.  Cost of a primary with T neighbours, in hundredths of a
+// step of one list (fitted at l_max 10; l_max 4 and 20 lie within 30 %):
+//   S 1   100 (T / 32 + nbins / 2)            + 500 nbins
+//   S 2   104 (T w2 / 16 + nbins / 2 / 2)     + 460 nbins / 2
+//   S 4   104 (T w4 / 8 + nbins / 4 / 2)      + 490 nbins / 4
+// w2, w4: the longest lists of the groups as a share of all; numbers of groups
+// rounded up.  With many bins that puts the limits near means of 160 and 800
+// neighbours a list, where they are held at most; with few they are lower.
+// Accumulation with 1 / 2 / 4 lists (8: slower than 4 except at 8 neighbours a
+// list, where they tie):
+//   mean list 8 (20k uniform points, l_max 10)      0.226 / 0.144 / 0.116 ms
+//   28 (200k points, l_max 20)                      24.0 / 16.7 / 14.7
+//   80 (24 mock catalogues, l_max 10)               52.3 / 39.4 / 39.4
+//   132 (3.1M-pixel sphere, m_max 8)                38.0 / 29.6 / 28.4
+//   522 (cut sky of 800k points, l_max 10)          118.1 / 111.1 / 113.2
+//   525 (250k primaries of 4M, l_max 20)            134.1 / 132.3 / 145.7
+//   1680 (10^6 points, l_max 10)                    221.5 / 243.1 / 274.0
+//   100k points from r_min 0, l_max 10: 1 bin of 130  0.247 / 0.299 / 0.448
+//     5 bins of 60   0.738 / 0.616 / 0.784;  of 400   1.720 / 2.345 / 4.002
+//     10 bins of 16  1.081 / 0.688 / 0.586;  of 130   1.793 / 1.374 / 1.797
+// (160 and 800 for any number of bins took up to 1.9 times the best there.)
+// A choice by each primary's list lengths, the same costs on its own counts,
+// was slower: neighbours in space then differ in S, and three forms running
+// at once overflow the instruction cache (7 bins of 60: 0.95 ms).
+ListLimits list_limits(const double* share, int nbins) {
+  if (nbins < 2) return ListLimits{0, 0};
+  double sum = 0, m2 = 0, m4 = 0;
+  for (int b = 0; b < nbins; ++b) {
+    sum += share[b];
+    if (b % 2 == 0) m2 += std::max(share[b], b + 1 < nbins ? share[b + 1] : 0.0);
+    if (b % 4 == 0) m4 += *std::max_element(share + b, share + std::min(b + 4, nbins));
+  }
+  if (!(sum > 0)) sum = m2 = m4 = 1;
+  const int g2 = (nbins + 1) / 2, g4 = (nbins + 3) / 4;
+  const double a[3] = {100.0 / 32, 104 * m2 / sum / 16, 104 * m4 / sum / 8};  // per neighbour: S 1, 2, 4
+  const double f[3] = {550.0 * nbins, 512.0 * g2, 542.0 * g4};                 // per primary
+  // neighbours below which form i is cheaper than form j of fewer lists
+  auto below = [&](int i, int j) {
+    if (f[i] >= f[j]) return 0.0;
+    return a[i] > a[j] ? (f[j] - f[i]) / (a[i] - a[j]) : 1e300;
+  };
+  const double two = std::max(below(1, 0), below(2, 0)), four = std::min(below(2, 1), below(2, 0));
+  ListLimits m;
+  m.four = (uint32_t)std::min(four, 160.0 * nbins);
+  m.two = std::max(m.four, (uint32_t)std::min(two, 800.0 * nbins));
+  return m;
 }
 
 cudaError_t launch_alm(const AlmArgs& a, int L, int lists, int wpb, int nsm, cudaStream_t st) {

@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
     }
     my_pairs += mine;
     mine = __reduce_add_sync(0xffffffffu, mine);
-    if (lane == 0 && mine) atomicOr(&s_classes, (uint32_t)lists_per_warp(mine, nbins));
+    if (lane == 0 && mine) atomicOr(&s_classes, (uint32_t)lists_per_warp(mine, a.limits));
     __syncwarp();
   }
 #pragma unroll
