@@ -185,8 +185,8 @@ __device__ __forceinline__ void con_step(float2 (&acc)[T][T / 2], const float* S
 template <int T, int CH, int MODE>
 __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(ContractArgs a, ConShape sh) {
   extern __shared__ __align__(16) float s_dyn[];
-  __shared__ __align__(16) int s_slotl[CH];  // multipole of each slot of the chunk (-1: none)
-  __shared__ int s_ord[CH];                  // the chunk's slots by multipole
+  __shared__ int s_coef[(kLmaxCap + 1) * (kLmaxCap + 1)];  // slot of each coefficient | its multipole << 16
+  __shared__ int s_ord[CH];                                // the chunk's slots by multipole
   __shared__ int s_l[kLmaxCap + 1], s_l0[kLmaxCap + 2], s_nl;  // its multipoles and where their slots start
   const int nb = a.nbins, L = a.lmax;
   const int nc = a.sphere ? 2 * L + 1 : (L + 1) * (L + 1);  // coefficients per (primary, bin)
@@ -225,6 +225,14 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
     }
     s_tile[t] = v;
   }
+  for (int k = tid; k < nc; k += blockDim.x) {
+    int l = a.sphere ? (k + 1) / 2 : (int)sqrtf((float)k);
+    if (!a.sphere) {
+      while ((l + 1) * (l + 1) <= k) ++l;
+      while (l * l > k) --l;
+    }
+    s_coef[k] = __ldg(a.slot + k) | l << 16;
+  }
   __syncthreads();
   const int tv = s_tile[tl];
   const bool active = tv >= 0;
@@ -240,59 +248,39 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
 #pragma unroll
     for (int j = 0; j < T / 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
+  // the slots of the chunk at c0 by multipole (the coefficients are in that
+  // order), and the multipoles that have any: by one warp, while the chunk's
+  // first copies are in flight
+  auto order_slots = [&](int c0) {
+    const int lane = tid & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    int n = 0, nl = 0, last = -1;  // slots and multipoles so far, and the last of these
+    for (int k = lane; k - lane < nc; k += 32) {
+      const int v = k < nc ? s_coef[k] : -1;
+      const int s = (v & 0xffff) - c0, l = v >> 16;
+      const bool in = v >= 0 && s >= 0 && s < CH;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      const int before = __shfl_sync(0xffffffffu, l, 31 - __clz((m & lt) | 1u));
+      const bool first = in && l != (m & lt ? before : last);
+      const unsigned mf = __ballot_sync(0xffffffffu, first);
+      const int at = n + __popc(m & lt);
+      if (in) s_ord[at] = s;
+      if (first) {
+        s_l[nl + __popc(mf & lt)] = l;
+        s_l0[nl + __popc(mf & lt)] = at;
+      }
+      n += __popc(m);
+      nl += __popc(mf);
+      const int end = __shfl_sync(0xffffffffu, l, 31 - __clz(m | 1u));
+      if (m) last = end;
+    }
+    if (lane == 0) {
+      s_nl = nl;
+      s_l0[nl] = n;
+    }
+  };
   for (int ck = 0; ck < sh.nchunk; ++ck) {
     const int c0 = ck * CH;
-    // the multipole of each slot of the chunk, its slots sorted by multipole,
-    // and the multipoles that have any
-    __syncthreads();
-    if (tid < CH) s_slotl[tid] = -1;
-    __syncthreads();
-    for (int k = tid; k < nc; k += blockDim.x) {
-      const int s = __ldg(a.slot + k) - c0;
-      if (s >= 0 && s < CH) {
-        int l = a.sphere ? (k + 1) / 2 : (int)sqrtf((float)k);
-        if (!a.sphere) {
-          while ((l + 1) * (l + 1) <= k) ++l;
-          while (l * l > k) --l;
-        }
-        s_slotl[s] = l;
-      }
-    }
-    __syncthreads();
-    if (tid < CH) {
-      const int l = s_slotl[tid];
-      int below = 0, n = 0;  // slots sorted before this one; all slots
-      bool first = true;     // no earlier slot has this multipole
-      unsigned seen = 0;     // multipoles of the chunk
-      const int4* sl4 = reinterpret_cast<const int4*>(s_slotl);
-#pragma unroll 4
-      for (int k = 0; k < CH; k += 4) {
-        const int4 v = sl4[k / 4];
-        const int lk[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const bool in = lk[e] >= 0, before = k + e < tid;
-          n += in;
-          below += in && (lk[e] < l || (lk[e] == l && before));
-          if (lk[e] == l && before) first = false;
-          seen |= in ? 1u << lk[e] : 0u;
-        }
-      }
-      if (l >= 0) {
-        s_ord[below] = tid;
-        if (first) {
-          const int rank = __popc(seen & ((1u << l) - 1u));
-          s_l[rank] = l;
-          s_l0[rank] = below;
-        }
-      }
-      if (tid == 0) {
-        s_nl = __popc(seen);
-        s_l0[s_nl] = n;
-      }
-    }
-    __syncthreads();
-
     // copy of the stage of primaries [pb, pb + cnt)
     auto issue = [&](int64_t pb, int cnt, int st) {
       float* buf = s_stage + st * sh.stage_floats;
@@ -335,8 +323,9 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
     // entries of one multipole, every lane the same slots of its entry
     auto flush = [&] {
       float* red = s_stage;
-      const int nthr = blockDim.x, ld = nthr + 1, nl = s_nl;
+      const int nthr = blockDim.x, ld = nthr + 1;
       __syncthreads();
+      const int nl = s_nl;
 #pragma unroll
       for (int i = 0; i < T; ++i)
 #pragma unroll
@@ -383,6 +372,7 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
         if (k < nst) issue(f0 + (int64_t)k * sh.Q, count(k), k);
         commit();
       }
+      if (f0 == p0 && tid < 32) order_slots(c0);
       int st = 0, nx = sh.stages - 1;
       for (int k = 0; k < nst; ++k) {
         if (sh.stages == 1) {  // one buffer: copy, wait, use
