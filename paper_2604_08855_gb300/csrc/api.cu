@@ -34,16 +34,13 @@ int resident_blocks(const void* fn, int threads, size_t smem) {
   static std::map<std::tuple<int, const void*, int, size_t>, int> known;  // a few entries per kernel and device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (allow_smem(fn, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
   std::lock_guard<std::mutex> lock(mu);
   const auto key = std::make_tuple(dev, fn, threads, smem);
   const auto it = known.find(key);
   if (it != known.end()) return it->second;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) {
+  if (allow_smem(fn, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }

@@ -450,7 +450,7 @@ cudaError_t launch_contract_fp32(const ContractArgs& a, int nparts, cudaStream_t
   const ConShape sh = con_shape(a.nbins, a.row);
   if ((size_t)sh.smem_bytes > kConSmemCap) return cudaErrorInvalidValue;
   const void* fn = con_kernel(sh, a.row, (reinterpret_cast<uintptr_t>(a.M) & 15) == 0);
-  if (resident_blocks(fn, sh.threads, sh.smem_bytes) < 1) return cudaErrorInvalidConfiguration;
+  if (allow_smem(fn, sh.smem_bytes) != cudaSuccess) return cudaErrorInvalidConfiguration;
   ContractArgs ca = a;
   ConShape cs = sh;
   void* args[] = {&ca, &cs};

@@ -238,8 +238,8 @@ __host__ __device__ __forceinline__ void each_list_line(uint32_t off, uint32_t e
 cudaError_t allow_smem(const void* fn, size_t smem);
 
 // Resident blocks per SM of a kernel at this block size and dynamic shared
-// memory (0: it cannot run), its shared-memory limit raised to that.  The
-// number is a fact of the kernel and the device, asked once for each (about 3 us a call).
+// memory (0: it cannot run): a fact of the kernel and the device, asked once
+// for each (about 3 us a call).
 int resident_blocks(const void* fn, int threads, size_t smem);
 
 // kernels launched by this host thread (every launcher adds its launches)

@@ -799,9 +799,11 @@ cudaError_t launch_passes(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
   } else {
     const int bps = alm_occupancy_pass<L, P, S>(wpb);
     if (bps < 1) return cudaErrorInvalidConfiguration;
+    cudaError_t e = allow_smem((const void*)k_alm<L, P, S>, alm_smem<L, P, S>(wpb));
+    if (e != cudaSuccess) return e;
     k_alm<L, P, S><<<bps * nsm, wpb * 32, alm_smem<L, P, S>(wpb), st>>>(a);
     ++g_launches;
-    const cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     AlmArgs next = a;
     ++next.work;

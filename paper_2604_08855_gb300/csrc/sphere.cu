@@ -127,6 +127,8 @@ template <int K, int S>
 static cudaError_t launch_am_KS(const AlmArgs& a, int wpb, int nsm, cudaStream_t st) {
   const int bps = am_occupancy_K<K, S>(wpb);
   if (bps < 1) return cudaErrorInvalidConfiguration;
+  const cudaError_t e = allow_smem((const void*)k_am<K, S>, am_smem<K, S>(wpb));
+  if (e != cudaSuccess) return e;
   k_am<K, S><<<bps * nsm, wpb * 32, am_smem<K, S>(wpb), st>>>(a);
   ++g_launches;
   return cudaGetLastError();
