@@ -5,6 +5,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <tuple>
 #include <utility>
@@ -44,7 +45,10 @@ int resident_blocks(const void* fn, int threads, size_t smem) {
     cudaGetLastError();
     return 0;
   }
-  known[key] = nb;
+  try {
+    known[key] = nb;
+  } catch (const std::bad_alloc&) {  // not noted: asked again next time
+  }
   return nb;
 }
 }  // namespace ctb
