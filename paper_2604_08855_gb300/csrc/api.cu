@@ -666,7 +666,7 @@ int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   // chunks follow the measured pairs per primary
   const double est = 2.0 * mean_neighbours(c) + 64.0;
   // candidates (points of the scanned cell rows) run about 1.3-1.5x the pairs
-  // (a small list capacity bounds the codes too, a primary's batch heads and one pool aside)
+  // (a small list capacity bounds the codes too, a primary's batch heads and segments and one pool aside)
   pl->code_cap = std::min<uint64_t>(kCodeCap, 4 * pl->list_cap + 1024ull * row_blocks(c->g) + kStreamCodePool);
   // and a batch's head and segments up to 8 bytes a point or row, whichever is fewer
   pl->cand_first = 1.5 * est + 8.0 * std::min(1.5 * est, 32.0 * row_blocks(c->g)) + 256.0;
@@ -839,6 +839,9 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     CK(c, cudaMemsetAsync(work, 0, kCounters * 8, c->st));
     CK(c, cudaEventRecord(ev[0], c->st));
     sa.lists = nullptr;
+    // a primary alone takes what it needs, so that the capacity holds its
+    // candidates' codes and not the unused ends of pools
+    sa.code_pool = cnt > 1 ? kStreamCodePool : 0;
     sa.work = work;
     CK(c, launch_stream(sa, false, pl.count_blocks, c->st));
     CK(c, cudaEventRecord(ev[1], c->st));

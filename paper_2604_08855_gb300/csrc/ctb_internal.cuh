@@ -351,6 +351,7 @@ struct StreamArgs {
   const uint32_t* keys;           // sorted cell keys of a batch (catalogue = key / ncells), or NULL
   uint8_t* codes;                 // bin code per candidate (written: count, read: fill)
   unsigned long long code_cap;    // bytes of codes
+  unsigned long long code_pool;   // code bytes a warp takes at a time (a longer batch takes its own length)
   unsigned long long* code_total; // code bytes of this launch (count pass; the range allocator)
   unsigned long long* code_base;  // [prim_count][row_blocks] start of each batch (at most one a row block; ~0 ends them)
   Geom g;
@@ -358,7 +359,7 @@ struct StreamArgs {
 int stream_blocks_per_sm(const Geom& g, bool fill);
 cudaError_t launch_stream(const StreamArgs& a, bool fill, int nblocks, cudaStream_t st);
 constexpr int kStreamThreads = 256;
-constexpr int kStreamCodePool = 16384;  // bytes of the code buffer a warp of the count pass takes at a time
+constexpr int kStreamCodePool = 16384;  // StreamArgs::code_pool, except for a chunk of one primary
 
 // pair.cuh -- harmonic accumulation over the (primary, bin) lists
 struct AlmArgs {

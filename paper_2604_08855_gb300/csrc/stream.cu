@@ -74,7 +74,6 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 }
 
 constexpr uint8_t kNoBin = 0xff;  // bin code of a candidate that is not a pair
-constexpr unsigned long long kCodePool = (unsigned long long)kStreamCodePool;  // code bytes a warp takes at a time
 constexpr unsigned long long kNoBatch = ~0ull;  // ends a primary's batches
 
 __device__ __forceinline__ void prefetch_l2(const void* p) {
@@ -332,7 +331,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4) k_count(StreamArgs a) {
         const uint32_t head = batch_head(nseg);
         const unsigned long long span = head + 128ull * ngroups;
         if (pool + span > pool_end) {
-          const unsigned long long take = span > kCodePool ? span : kCodePool;
+          const unsigned long long take = span > a.code_pool ? span : a.code_pool;
           if (lane == 0) pool = atomicAdd(a.code_total, take);
           pool = __shfl_sync(0xffffffffu, pool, 0);
           pool_end = pool + take;
