@@ -105,7 +105,7 @@ struct ctb_ctx {
   uint64_t* pin = nullptr;  // pinned words that counters and flags are read back into
   // device buffers
   Buf xyz_stage, w_stage, key0, val0, key1, val1, hist, scan_tmp, pts_in, pts, s2i, i2s, cell_start;
-  Buf flags, bbox_part, lists, M, wprim, partial, zeta, prim, counters, norm, slot, idx64, alm, thr;
+  Buf flags, bbox_part, lists, M, wprim, partial, zeta, prim, counters, slot, idx64, alm, thr;
   Buf edge_in, edge_tj;  // edge correction: staged sums, 3j table
   bool edge_tj_ready = false;
   Buf pairsum;          // FP64 partial pair sums [catalogue][part][bin] of the last compute
@@ -198,7 +198,7 @@ void release_all(ctb_ctx* c) {
   Buf* all[] = {&c->xyz_stage, &c->w_stage, &c->key0, &c->val0, &c->key1, &c->val1, &c->hist,
                 &c->scan_tmp, &c->pts_in, &c->pts, &c->s2i, &c->i2s, &c->cell_start, &c->flags,
                 &c->bbox_part, &c->lists, &c->M, &c->wprim, &c->partial, &c->zeta, &c->prim,
-                &c->counters, &c->norm, &c->slot, &c->idx64, &c->alm, &c->thr, &c->codes, &c->code_base, &c->pairsum, &c->edge_in, &c->edge_tj, &c->counts,
+                &c->counters, &c->slot, &c->idx64, &c->alm, &c->thr, &c->codes, &c->code_base, &c->pairsum, &c->edge_in, &c->edge_tj, &c->counts,
                 &c->offsets, &c->scan_tmp2, &c->ops[0], &c->ops[1], &c->ops[2], &c->ops[3],
                 &c->slot_lm, &c->lbase_d, &c->kp_d, &c->partial_tc, &c->conv, &c->gk0, &c->gv0, &c->gk1, &c->gv1, &c->glo, &c->ghi, &c->ghead, &c->gid, &c->gscan,
                 &c->gprim, &c->gw};
@@ -224,7 +224,7 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
   return ms;
 }
 
-// normalisation per slot and the slot table of the context's layout
+// slot and conversion tables of the context's layout
 int ensure_tables_sphere(ctb_ctx* c) {
   // row = [Re a_1, Im a_1, ..., Re a_K, Im a_K, a_0], padded to 32; every
   // slot its own coefficient.  Coefficient index i (0: a_0, 2m-1: Re a_m,
@@ -248,12 +248,7 @@ int ensure_tables(ctb_ctx* c) {
   if (c->sphere) return ensure_tables_sphere(c);
   c->Lk = lmax_kernel(c->lmax);
   make_layout(c->Lk, &c->lay);
-  std::vector<float> norm(c->lay.row, 0.f);
-  for (int l = 0; l <= c->Lk; ++l)
-    for (int m = -l; m <= l; ++m) norm[c->lay.slot[l * l + l + m]] = (float)norm_lm(l, m);
-  CK(c, ensure(c, c->norm, norm.size() * sizeof(float)));
   CK(c, ensure(c, c->slot, sizeof(c->lay.slot)));
-  CK(c, cudaMemcpyAsync(c->norm.p, norm.data(), norm.size() * sizeof(float), cudaMemcpyHostToDevice, c->st));
   CK(c, cudaMemcpyAsync(c->slot.p, c->lay.slot, sizeof(c->lay.slot), cudaMemcpyHostToDevice, c->st));
   // slot -> (l, m + l) for the tensor-core pack: l * 64 + (m + l), -1 for padding and l > ell_max
   std::vector<int> slot_lm(c->lay.row, -1);

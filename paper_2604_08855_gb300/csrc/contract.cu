@@ -59,7 +59,7 @@ namespace ctb {
 constexpr int kConFlush = 1024;         // primaries of a group between two flushes
 constexpr int kConMaxQ = 64;            // primaries per stage at most
 constexpr int kConStageFloats = 11264;  // one staged buffer at most, when more than PG primaries fit it
-constexpr int kConStages = 3;
+constexpr int kConStages = 3;           // staged buffers: one in use, one in, one on its way
 constexpr int kConMaxTiles = 24;        // tiles per block at most (768 threads / 32)
 enum { kConRows4 = 0, kConRows16 = 1, kConLinear = 2, kConLinearAny = 3 };
 constexpr size_t kConSmemCap = 220 * 1024;
@@ -75,7 +75,6 @@ struct ConShape {
   int threads;
   int stride;   // staged floats between bins: the row, or CH when the row is chunked
   int Q;        // primaries per stage
-  int stages;
   int stage_floats;  // one staged buffer
   int smem_bytes;
 };
@@ -125,10 +124,8 @@ static ConShape con_shape(int nbins, int row) {
   c.stage_floats = c.Q * nbins * c.stride + (nbins < c.T ? (c.T - nbins) * c.stride : 0) + c.ch;
   c.stage_floats = (c.stage_floats + 3) & ~3;
   const int red = (c.threads + 1) * c.T * c.T;  // the flush buffer aliases the stages (154 KB at most)
-  c.stages = kConStages;
-  while (c.stages > 1 && (size_t)(c.stages * (c.stage_floats + kConMaxQ)) * 4 + 4096 > kConSmemCap) --c.stages;
-  const int body = c.stages * c.stage_floats > red ? c.stages * c.stage_floats : red;
-  c.smem_bytes = (body + c.stages * kConMaxQ + kConMaxTiles) * 4;
+  const int body = kConStages * c.stage_floats > red ? kConStages * c.stage_floats : red;
+  c.smem_bytes = (body + kConStages * kConMaxQ + kConMaxTiles) * 4;  // 187 KB at most
   return c;
 }
 
@@ -192,7 +189,7 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
   const int nc = a.sphere ? 2 * L + 1 : (L + 1) * (L + 1);  // coefficients per (primary, bin)
   int* s_tile = reinterpret_cast<int*>(s_dyn);              // [kConMaxTiles] B1 | B2 << 8 (-1: none)
   float* s_w = s_dyn + kConMaxTiles;                        // [stages][kConMaxQ]
-  float* s_stage = s_w + sh.stages * kConMaxQ;              // [stages][Q][nb][stride]
+  float* s_stage = s_w + kConStages * kConMaxQ;             // [stages][Q][nb][stride]
   const int tid = threadIdx.x;
   const int c = tid % CH;
   const int tl = (tid / CH) % sh.tiles, pg = tid / (CH * sh.tiles);
@@ -368,26 +365,18 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
       const int64_t f1 = min(p1, f0 + run);
       const int nst = (int)((f1 - f0 + sh.Q - 1) / sh.Q);
       auto count = [&](int k) { return (int)min((int64_t)sh.Q, f1 - f0 - (int64_t)k * sh.Q); };
-      for (int k = 0; k < sh.stages - 1; ++k) {
+      for (int k = 0; k < kConStages - 1; ++k) {
         if (k < nst) issue(f0 + (int64_t)k * sh.Q, count(k), k);
         commit();
       }
       if (f0 == p0 && tid < 32) order_slots(c0);
-      int st = 0, nx = sh.stages - 1;
+      int st = 0, nx = kConStages - 1;
       for (int k = 0; k < nst; ++k) {
-        if (sh.stages == 1) {  // one buffer: copy, wait, use
-          __syncthreads();
-          issue(f0 + (int64_t)k * sh.Q, count(k), 0);
-          commit();
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-          __syncthreads();
-        } else {
-          if (sh.stages == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
-          else asm volatile("cp.async.wait_group 1;" ::: "memory");
-          __syncthreads();  // stage k is in, and every thread is done with stage k - 1
-          if (k + sh.stages - 1 < nst) issue(f0 + (int64_t)(k + sh.stages - 1) * sh.Q, count(k + sh.stages - 1), nx);
-          commit();
-        }
+        asm volatile("cp.async.wait_group %0;" ::"n"(kConStages - 2) : "memory");
+        __syncthreads();  // stage k is in, and every thread is done with stage k - 1
+        const int kn = k + kConStages - 1;
+        if (kn < nst) issue(f0 + (int64_t)kn * sh.Q, count(kn), nx);
+        commit();
         const int cnt = count(k);
         const float* buf = s_stage + st * sh.stage_floats + pg * qstride;
         const float* wq = s_w + st * kConMaxQ;
@@ -401,10 +390,8 @@ __global__ void __launch_bounds__(con_max_threads(T), 1) k_contract_fp32(Contrac
               con_step<T, false, ST>(acc, buf + off1, buf + off2, stride, wq[q]);
           }
         }
-        if (sh.stages > 1) {
-          st = st + 1 == sh.stages ? 0 : st + 1;
-          nx = nx + 1 == sh.stages ? 0 : nx + 1;
-        }
+        st = st + 1 == kConStages ? 0 : st + 1;
+        nx = nx + 1 == kConStages ? 0 : nx + 1;
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       flush();

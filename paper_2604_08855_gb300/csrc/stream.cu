@@ -76,11 +76,7 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 constexpr uint8_t kNoBin = 0xff;  // bin code of a candidate that is not a pair
 constexpr unsigned long long kNoBatch = ~0ull;  // ends a primary's batches
 
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-// Geometry of one primary's row window, shared by both passes.
+// Geometry of one primary's row window (count pass).
 struct RowWin {
   int W, off0, nrows;
   uint32_t invW;  // ceil(2^32 / W): t / W = umulhi(t, invW) for t < 2^32 / W
