@@ -868,7 +868,7 @@ int run_pairs(ctb_ctx* c, const uint32_t* dprim, int64_t np, bool contract, cons
     CK(c, launch_stream(sa, true, pl.stream_blocks, c->st));
     CK(c, cudaEventRecord(ev[2], c->st));
     // one form for all primaries of the chunk where they agree on it
-    const int lists = c->pin[2] == 1 ? 1 : (c->pin[2] == 4 ? 4 : 0);
+    const int lists = c->pin[2] == 1 || c->pin[2] == 2 || c->pin[2] == 4 ? (int)c->pin[2] : 0;
     if (c->sphere)
       CK(c, launch_am(aa, c->lmax, lists, pl.wpb, c->nsm, c->st));
     else

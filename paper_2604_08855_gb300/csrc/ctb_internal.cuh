@@ -385,7 +385,7 @@ int am_blocks_per_sm(int mmax, int warps_per_block);
 cudaError_t launch_am(const AlmArgs& a, int mmax, int lists, int warps_per_block, int nsm, cudaStream_t st);
 // one launch per m-pass, each sized from its own occupancy on nsm SMs; lists:
 // (primary, bin) lists a warp accumulates side by side, for every primary of
-// the launch (1 or 4), or 0: by each primary's own lists (the same sums)
+// the launch (1, 2 or 4), or 0: by each primary's own lists (the same sums)
 cudaError_t launch_alm(const AlmArgs& a, int lmax_kernel, int lists, int warps_per_block, int nsm, cudaStream_t st);
 
 // contract.cu

@@ -735,8 +735,8 @@ __device__ __forceinline__ void load_lists(const AlmArgs& a, uint64_t ib, uint32
 // One warp per primary: its (primary, bin) lists are consecutive runs of the
 // lists buffer; S of them at a time are accumulated in registers for m-pass P
 // of kernel L and flushed once, with the next lists' first loads already in
-// flight.  S: lists_per_warp of every primary (1 or 4), or 0 where they
-// differ: the three forms in one kernel, each primary with its own.  Its code
+// flight.  S: lists_per_warp of every primary (1 or 4), or 0 for 2 and where
+// they differ: the three forms in one kernel, each primary with its own.  Its code
 // is scheduled less well in the longest loops (chosen primaries of 10^6 points
 // at l_max 10, all with S = 1: 3.55 ms against 3.50; 3.1M pixels on the
 // sphere, all 4: 94.7 against 94.1), and gains where S = 2 is the most
