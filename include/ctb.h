@@ -245,7 +245,8 @@ int ctb_compute_batch(ctb_ctx* ctx, const double* const* xyz, const double* cons
  * out of range, CTB_ERR_UNSUPPORTED for a precision the library cannot run.
  * CTB_OPT_LIST_CAPACITY bounds the neighbour lists of one chunk of primaries
  * (4 bytes per entry) and the candidates' bin codes of that chunk (1 byte per
- * candidate, at most 4 per list entry of the capacity); chunks are sized to
+ * candidate and 8 per cell row that holds any, at most 4 per list entry of the
+ * capacity, aside from one primary's rows and 16 KB); chunks are sized to
  * fit, and a compute in which one primary alone has more pairs (or candidates)
  * than that fails with CTB_ERR_OOM.
  * CTB_OPT_AUTOTUNE = 1 (with CTB_OPT_CELLS_PER_RMAX left at 0) makes the next
@@ -319,10 +320,12 @@ int ctb_get_2pcf(ctb_ctx* ctx, double* out, int cap);
  * sum_l zeta_l P_l(mu) solve  n_l / r_0 = sum_l' M_ll' zeta_l'  with
  *   n_l = (2l+1)/2 zeta_nnn_l,  r_l = (2l+1)/2 zeta_rrr_l,  f_l = r_l / r_0,
  *   M_ll' = (2l+1) sum_l'' (l l' l''; 0 0 0)^2 f_l''   (all l <= ell_max),
- * in FP64 on the device (one thread per bin pair, partial pivoting).
+ * in FP64 on the device (one warp per bin pair, partial pivoting).
  * zeta_out receives zeta_l [(ell_max+1)][nbins][nbins]; bin pairs without
  * random triplets or with a singular system are NaN.  Pointers may be host
- * or device memory; the caller keeps them.  Returns CTB_OK, CTB_ERR_ARG,
+ * or device memory; the caller keeps them.  Arrays in this device's memory are
+ * read and written where they lie; zeta_out may be one of the inputs, or
+ * overlap one shifted (it is then written through a buffer).  Returns CTB_OK, CTB_ERR_ARG,
  * CTB_ERR_OOM or CTB_ERR_CUDA.
  */
 int ctb_edge_correct(ctb_ctx* ctx, const double* zeta_nnn, const double* zeta_rrr, double* zeta_out);

@@ -621,7 +621,7 @@ double mean_row(const ctb_ctx* c) {
 int plan_pairs(ctb_ctx* c, int64_t np, PairPlan* pl) {
   // The count pass takes four steps of a row at a time (four loads in flight,
   // one vote, one store, paired FP32 instructions) where rows are long; its
-  // state fills 64 registers so, and short rows lose by that.  Enumeration
+  // state takes 60 of the 64 registers, and short rows lose by that.  Enumeration
   // with one / four steps: 296 points a row (10^6 points) 150.7 / 132.8 ms,
   // 231 (cut sky) 98.8 / 98.6, 30 (mock catalogues) 23.0 / 25.5.
   c->g.long_rows = mean_row(c) >= 256.0;

@@ -20,12 +20,13 @@ namespace ctb {
 // each l are added in a fixed order.
 //
 // What bounds it: the issue of paired FMAs and their operands at three warps
-// a scheduler (FMA pipe 41 %, HBM 52 % on 200k rows of 20 bins, l_max 10:
-// 546 us).  The form before this one, 4 x 4 tiles by 16-byte loads of
-// transposed rows, spent its time on shared-memory loads and, for the
+// a scheduler (20k rows of 20 bins x 128, l_max 10: 62 us, FMA pipe 42 %, issue
+// 54 %, 0.49 of HBM).  The form before this one, 4 x 4 tiles by 16-byte loads
+// of transposed rows, spent its time on shared-memory loads and, for the
 // 121-float rows of a caller, on transposing them element by element (20k
-// such rows: 640 us; now 72).  Half tiles of 5 x 10 with twice the warps were
-// slower (667 us): more loads and address arithmetic per FMA.
+// such rows, the whole call: 734 us; now 86).  Half tiles of 5 x 10 with twice
+// the warps were slower (200k rows: 667 us against 546): more loads and
+// address arithmetic per FMA.
 //
 // Block: CH slots x tiles x PG primary groups (group g takes the stage's
 // primaries q = g mod PG).  Rows of more than CH slots are taken in chunks of
@@ -47,7 +48,7 @@ namespace ctb {
 // one run / two, relative rms: 20k rows of 20 bins at l_max 10 1.43e-8 /
 // 7.0e-9, 100k rows 3.1e-8 / 1.5e-8, 20k of 16 bins 1.36e-8 / 7.0e-9; with
 // several groups, plain sums / errors carried: 2000 rows of 10 bins 3.9e-9 /
-// 2.2e-9.  The second flush costs 2 us of 71 at 20k rows of 20 bins.  (With
+// 2.2e-9.  The second flush costs 2 us at 20k rows of 20 bins.  (With
 // one thread per entry and multipole, whose loads collide in the shared
 // memory's banks and whose partial row is read, added to and written in turn,
 // a flush took 8 us.)

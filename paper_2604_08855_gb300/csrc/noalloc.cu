@@ -115,7 +115,8 @@ extern "C" int ctb_contract_noalloc(const float* alm, const float* w, int64_t np
     ca.partial = sc.partial;
     ca.part0 = 0;
     // two runs a slice where every SM has a block; one where the array holds
-    // fewer rows than that (500 rows of 32 bins at l_max 15: 120 us with two, 79 with one)
+    // fewer rows than that (500 rows of 32 bins at l_max 15: 120 us with two, 79
+    // with one)
     ca.runs = nparts < bps * sc.nsm ? 1 : 2;
     e = launch_contract_fp32(ca, nparts, st);
     if (e != cudaSuccess) return CTB_ERR_CUDA;
